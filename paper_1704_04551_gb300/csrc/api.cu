@@ -1029,6 +1029,9 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.work_floats = (int)membrane_work_floats(D.nv, D.nt, D.ne);
     D.A0 = (float)hm.A0;
     D.V0 = (float)hm.V0;
+    // the rest area and volume are about 2^20 units of the coarse half of the sums
+    D.fix_a = std::ldexp(1.0f, 20 - std::ilogb(hm.A0));
+    D.fix_v = std::ldexp(1.0f, 20 - std::ilogb(hm.V0));
     int most = 1;  // contributions a vertex receives: its edge roles and triangles
     for (int v = 0; v < D.nv; ++v)
       most = std::max(most, hm.v_edge_start[v + 1] - hm.v_edge_start[v] + hm.v_tri_start[v + 1] - hm.v_tri_start[v]);

@@ -150,6 +150,7 @@ struct MeshDev {
   int off_edges, off_edge_tris, off_edge_rest, off_tris, off_area0, off_ve_start, off_ve, off_vt_start, off_vt;
   int work_floats;   // per-body shared work area: 9 nv + 4 nt words
   float A0, V0;
+  float fix_a, fix_v;  // powers of two: fixed-point scales of the area and volume sums
   float qcap;        // fixed-point force scatter: largest |contribution| in units, such
                      // that a vertex's sum of all its contributions fits in int32
 };
@@ -168,11 +169,41 @@ struct MarkersDev {
   float* frac;        // [3][M]
 };
 
+// X = c + f with c = floor(X) and f = X - c rounded once to FP32, for
+// |X| < 2^30. Integer arithmetic on the bits of X: an SM does 2 FP64 lanes a
+// cycle here, and floor, conversion, subtraction and conversion in FP64 cost
+// four of them per coordinate (of the fused kernel's 49 us per body about 2).
+// The result is the same, bit for bit.
+__device__ __forceinline__ void split_coord(double X, int& c, float& f) {
+  const unsigned hw = (unsigned)__double2hiint(X);
+  const int e = (int)((hw >> 20) & 0x7ffu) - 1023;
+  if (e < -8 || e > 30) {  // tiny (or out of range): the plain way
+    const double fl = floor(X);
+    c = (int)fl;
+    f = (float)(X - fl);
+    return;
+  }
+  const unsigned long long mant =
+      ((unsigned long long)((hw & 0xfffffu) | 0x100000u) << 32) | (unsigned)__double2loint(X);
+  const long long v = (int)hw < 0 ? -(long long)mant : (long long)mant;  // X 2^(52 - e)
+  const int s = 52 - e;                                                   // 22 .. 60
+  c = (int)(v >> s);
+  const unsigned long long q = (unsigned long long)v << (64 - s);  // fraction, 2^-64 units
+  // one rounding: normalised to 32 significant bits, with a sticky bit for
+  // the rest (an FP32 significand has 24)
+  const int z = min(__clzll((long long)q), 64 - 32);
+  const unsigned long long t = q << z;
+  const unsigned h = (unsigned)(t >> 32) | ((unsigned)t != 0u ? 1u : 0u);
+  f = __uint2float_rn(h) * __int_as_float((127 - 32 - z) << 23);
+}
+
 // Stencil cache of one marker coordinate: floor and fractional part.
 __device__ __forceinline__ void cache_coord(const MarkersDev& m, size_t off, double X) {
-  const double f = floor(X);
-  m.cell[off] = (int)f;
-  m.frac[off] = (float)(X - f);
+  int c;
+  float f;
+  split_coord(X, c, f);
+  m.cell[off] = c;
+  m.frac[off] = f;
 }
 
 }  // namespace ibm

@@ -79,7 +79,7 @@ __device__ __forceinline__ void smem_cell(const MembraneSmem& S, int nv, int v, 
 template <int GEOM>
 __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_next, const MarkersDev& m, BodyDev* B,
                                                 const MarkerGroup G, int4* box, unsigned char* orec,
-                                                const MeshDev& mesh, unsigned char* smem, double* red) {
+                                                const MeshDev& mesh, unsigned char* smem) {
   __shared__ int s_lo[3], s_hi[3];
   __shared__ unsigned s_fmax;
   const size_t M = (size_t)m.M;
@@ -170,9 +170,9 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
       for (int a = 0; a < 3; ++a) {
         const double Xn = Xo[q][a] + (double)ua[a];
         m.X[a * M + k] = Xn;
-        const double fl = floor(Xn);
-        const int c = (int)fl;
-        const float f = (float)(Xn - fl);
+        int c;
+        float f;
+        split_coord(Xn, c, f);
         m.cell[a * M + k] = c;
         m.frac[a * M + k] = f;
         S.sI[a * nv + j] = (float)(c - oa[a]);
@@ -214,7 +214,7 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
   }
 
   // ---- 2. membrane forces at X^{n+1} ---------------------------------------
-  const ForceSums sF = membrane_core(B, mesh, S, red);  // ends synchronised
+  const ForceSums sF = membrane_core(B, mesh, S);  // ends synchronised
   {
     float fm = 0.f;
     for (int v = threadIdx.x; v < nv; v += blockDim.x) {
@@ -307,12 +307,11 @@ __global__ void __launch_bounds__(COUPLE_THREADS, 2)
     k_couple(LatticeDev L, float4* g_next, MarkersDev m, BodyDev* __restrict__ bodies, const int2* __restrict__ items,
              const MarkerGroup* __restrict__ groups, int4* boxes, unsigned char* orders, MeshDev mesh) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[2 * 32];
   // items[b] = (body, group b): the items follow the group order, so the
   // group and its box are read without waiting for the item
   const int b = blockIdx.x;
   couple_membrane<GEOM>(L, g_next, m, bodies + items[b].x, groups[b], boxes + 2 * b,
-                        orders + (size_t)b * couple_order_stride(mesh.nv), mesh, smem, red);
+                        orders + (size_t)b * couple_order_stride(mesh.nv), mesh, smem);
 }
 
 }  // namespace

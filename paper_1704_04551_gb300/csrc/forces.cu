@@ -10,8 +10,7 @@ namespace ibm {
 __global__ void __launch_bounds__(MEMBRANE_THREADS, 4)
     k_membranes(MarkersDev m, BodyDev* __restrict__ bodies, const int* __restrict__ list, MeshDev mesh) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[2 * 32];
-  membrane_block(m, bodies + list[blockIdx.x], mesh, smem, red);
+  membrane_block(m, bodies + list[blockIdx.x], mesh, smem);
 }
 
 __global__ void __launch_bounds__(RIGID_THREADS) k_rigid(MarkersDev m, BodyDev* __restrict__ bodies,

@@ -75,6 +75,90 @@ __device__ __forceinline__ Topo topo_at(const unsigned char* base, const MeshDev
   return T;
 }
 
+// The body's area and volume are sums of FP32 values of which only a small
+// difference from the rest value matters. They are added exactly, in fixed
+// point: a value v is hi + lo with hi = round(v s) (s a power of two, the
+// whole sum about 2^20 of its units) and lo the rest in units 2^22 finer, each
+// summed over a warp by one integer reduction. A tree of FP64 adds keeps an
+// SM's FP64 pipe (2 lanes a cycle) busy for ~1 us per body, and its last
+// serial sum of the warps for as long again.
+struct MembraneScale {
+  float sa, sv;    // units of hi per area, volume
+  double qa, qv;   // area, volume per unit of lo
+};
+__device__ __forceinline__ MembraneScale membrane_scale(const MeshDev& mesh) {
+  MembraneScale K;
+  K.sa = mesh.fix_a;
+  K.sv = mesh.fix_v;
+  K.qa = (double)(0x1p-22f / mesh.fix_a);
+  K.qv = (double)(0x1p-22f / mesh.fix_v);
+  return K;
+}
+__device__ __forceinline__ long long warp_fixed(float v, float s) {
+  const int hi = __float2int_rn(v * s);
+  const int lo = __float2int_rn(fmaf(v, s, -(float)hi) * 4194304.0f);
+  return ((long long)__reduce_add_sync(0xffffffffu, hi) << 22) + __reduce_add_sync(0xffffffffu, lo);
+}
+// Adds the warp's values to sum[0] (area) and sum[1] (volume) in shared memory.
+__device__ __forceinline__ void warp_fixed_sum(float area, float volume, const MembraneScale& K, long long* sum) {
+  const long long a = warp_fixed(area, K.sa), v = warp_fixed(volume, K.sv);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(reinterpret_cast<unsigned long long*>(sum), (unsigned long long)a);
+    atomicAdd(reinterpret_cast<unsigned long long*>(sum + 1), (unsigned long long)v);
+  }
+}
+
+// Stretching and bending forces of one edge E = (a, b, c, d) with triangles
+// ET: dv(a, b) = x_a - x_b, normal(t) the doubled-area normal, rest = (l0,
+// cos theta0, sin theta0, -); each contribution is handed to add(vertex, force).
+template <class Diff, class Normal, class Add>
+__device__ __forceinline__ void edge_forces(const ushort4 E, const ushort2 ET, const float4 rest, float kBT_p, float k_b,
+                                            Diff&& dv, Normal&& normal, Add&& add) {
+  const float3 ev = dv(E.y, E.x);  // b - a
+  const float L2 = dot(ev, ev), l = sqrtf(L2);
+  const float rL2 = __fdividef(1.0f, L2), rl = l * rL2;
+  const float l0 = rest.x, x = __fdividef(l, 2.0f * l0);
+  const float kp = 1.25f * kBT_p * l0 * l0;  // zero bond force at x = 1/2
+  const float dUdl = kBT_p * (__fdividef(0.25f, (1.0f - x) * (1.0f - x)) - 0.25f + x) - kp * rL2;
+  const float3 fs = (dUdl * rl) * ev;  // F_a = (dU/dl)/l (b - a), F_b = -F_a
+  if (k_b == 0.f) {
+    add(E.x, fs);
+    add(E.y, (-1.0f) * fs);
+    return;
+  }
+  // bending: F_v = -s dtheta/dv with dtheta/dc = -L n1/|n1|^2,
+  // dtheta/dd = -L n2/|n2|^2, dtheta/da = -(1-t1) g_c - (1-t2) g_d,
+  // dtheta/db = -t1 g_c - t2 g_d, t1,2 = (c,d - a).(b - a)/L^2
+  const float3 n1 = normal(ET.x), n2 = normal(ET.y);
+  // sin(theta - theta0) = sin(theta) cos(theta0) - cos(theta) sin(theta0), with
+  // cos(theta), sin(theta) from the normals (no inverse trigonometry)
+  const float inv = rsqrtf(dot(n1, n1) * dot(n2, n2));
+  const float cth = dot(n1, n2) * inv, sth = dot(cross(n1, n2), ev) * rl * inv;
+  const float sb = k_b * (sth * rest.y - cth * rest.z);
+  const float3 gc = __fdividef(-l, dot(n1, n1)) * n1, gd = __fdividef(-l, dot(n2, n2)) * n2;
+  const float t1 = dot(dv(E.z, E.x), ev) * rL2, t2 = dot(dv(E.w, E.x), ev) * rL2;
+  add(E.x, fs + (sb * (1.0f - t1)) * gc + (sb * (1.0f - t2)) * gd);
+  add(E.y, (-1.0f) * fs + (sb * t1) * gc + (sb * t2) * gd);
+  add(E.z, (-sb) * gc);
+  add(E.w, (-sb) * gd);
+}
+
+// Area and volume forces of one triangle (normal N, area At):
+// F_v = -coef dA_t/dx_v - (k_v (V - V0)/V0) N_t / 6, dA_t/dx_v = 1/2 n x (x_{v+2} - x_{v+1}).
+template <class Diff, class Add>
+__device__ __forceinline__ void triangle_forces(const ushort4 Tr, float3 N, float At, float At0, float k_l, float cg,
+                                                float cv, Diff&& dv, Add&& add) {
+  const int vv[3] = {Tr.x, Tr.y, Tr.z};
+  const float coef = k_l * __fdividef(At - At0, At0) + cg;
+  const float3 nh = __fdividef(0.5f, At) * N;
+  const float3 fV = (-cv / 6.0f) * N;
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    const float3 gA = cross(nh, dv(vv[(q + 2) % 3], vv[(q + 1) % 3]));
+    add(vv[q], (-0.5f * coef) * gA + fV);
+  }
+}
+
 }  // namespace forces_detail
 using namespace forces_detail;
 
@@ -109,12 +193,10 @@ struct ForceSums {
   }
 };
 
-__device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& mesh, const MembraneSmem& S,
-                                                   double* red);
+__device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& mesh, const MembraneSmem& S);
 
 // Membrane forces of one body by the whole thread block. smem: [9 nv + 4 nt]
-// words (positions as floor + fraction, force sums, normals, areas);
-// red: [2 * 32] doubles.
+// words (positions as floor + fraction, force sums, normals, areas).
 //
 // The force sums are scattered with shared-memory integer atomics in fixed
 // point (native and order-independent; float atomics on shared memory are
@@ -125,7 +207,7 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
 // or has no previous step, redoes the scatter with float atomics. The
 // quantum 1/Sq is ~3e-8 q, below the FP32 rounding of the sums.
 __device__ __forceinline__ void membrane_block(const MarkersDev& m, BodyDev* Bp, const MeshDev& mesh,
-                                               unsigned char* smem, double* red) {
+                                               unsigned char* smem) {
   const size_t M = (size_t)m.M;
   const int nv = mesh.nv;
   const MembraneSmem S = MembraneSmem::at(smem, nv, mesh.nt);
@@ -139,7 +221,7 @@ __device__ __forceinline__ void membrane_block(const MarkersDev& m, BodyDev* Bp,
     }
   }
   __syncthreads();
-  const ForceSums F = membrane_core(Bp, mesh, S, red);
+  const ForceSums F = membrane_core(Bp, mesh, S);
   for (int v = threadIdx.x; v < nv; v += blockDim.x) m.F[first + v] = make_float4(F(v), F(nv + v), F(2 * nv + v), 0.f);
 }
 
@@ -147,8 +229,7 @@ __device__ __forceinline__ void membrane_block(const MarkersDev& m, BodyDev* Bp,
 // synchronised after writing them): S.sQ receives the per-vertex sums
 // [3][nv] (read through the returned ForceSums), Bp->qmax the scale for the
 // next step; ends synchronised.
-__device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& mesh, const MembraneSmem& S,
-                                                   double* red) {
+__device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& mesh, const MembraneSmem& S) {
   const Topo T = topo_at(mesh.packed, mesh);
   const int nv = mesh.nv, nt = mesh.nt, ne = mesh.ne;
   const float kBT_p = Bp->kBT_p, k_b = Bp->k_b, k_l = Bp->k_l, k_g = Bp->k_g, k_v = Bp->k_v;
@@ -159,9 +240,15 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
   float* sN = S.sN;
   float* sA = S.sA;
   __shared__ float s_dev[2];
+  __shared__ long long s_fix[2];
   __shared__ unsigned s_qmax;
+  const MembraneScale K = membrane_scale(mesh);
   for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) sQ[i] = 0;
-  if (threadIdx.x == 0) s_qmax = 0u;
+  if (threadIdx.x == 0) {
+    s_qmax = 0u;
+    s_fix[0] = s_fix[1] = 0;
+  }
+  __syncthreads();  // the sums are cleared before the first warp adds to them
   // x_a - x_b, exact in the integer part, one FP32 rounding in the fraction
   auto dv = [&](int a, int b) {
     return make_float3((sI[a] - sI[b]) + (sR[a] - sR[b]), (sI[nv + a] - sI[nv + b]) + (sR[nv + a] - sR[nv + b]),
@@ -182,27 +269,11 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
     // triangle's first vertex from vertex 0
     v_part += dot(dv(Tr.x, 0), N) * (1.0f / 6.0f);
   }
-  double s0 = a_part, s1 = v_part;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    s0 += __shfl_xor_sync(0xffffffffu, s0, o);
-    s1 += __shfl_xor_sync(0xffffffffu, s1, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    red[2 * (threadIdx.x >> 5)] = s0;
-    red[2 * (threadIdx.x >> 5) + 1] = s1;
-  }
-  __syncthreads();  // normals, areas and partial sums are visible
-  if (threadIdx.x == 0) {
-    // A - A0 and V - V0 in FP64 (small differences of large sums)
-    double A = 0.0, V = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) {
-      A += red[2 * w];
-      V += red[2 * w + 1];
-    }
-    s_dev[0] = (float)(A - (double)mesh.A0) / mesh.A0;
-    s_dev[1] = (float)(V - (double)mesh.V0) / mesh.V0;
-  }
+  warp_fixed_sum(a_part, v_part, K, s_fix);
+  __syncthreads();  // normals, areas and sums are visible
+  // A - A0 and V - V0 in FP64 (small differences of large sums)
+  if (threadIdx.x == 0) s_dev[0] = (float)((double)s_fix[0] * K.qa - (double)mesh.A0) / mesh.A0;
+  if (threadIdx.x == 32) s_dev[1] = (float)((double)s_fix[1] * K.qv - (double)mesh.V0) / mesh.V0;
   __syncthreads();
   const float cg = k_g * s_dev[0];
   const float cv = k_v * s_dev[1];
@@ -229,33 +300,7 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
         rn = T.edge_rest[e + blockDim.x];
         ETn = T.edge_tris[e + blockDim.x];
       }
-      const float3 ev = dv(E.y, E.x);  // b - a
-      const float L2 = dot(ev, ev), l = sqrtf(L2);
-      const float rL2 = __fdividef(1.0f, L2), rl = l * rL2;
-      const float l0 = rest.x, x = __fdividef(l, 2.0f * l0);
-      const float kp = 1.25f * kBT_p * l0 * l0;  // zero bond force at x = 1/2
-      const float dUdl = kBT_p * (__fdividef(0.25f, (1.0f - x) * (1.0f - x)) - 0.25f + x) - kp * rL2;
-      const float3 fs = (dUdl * rl) * ev;  // F_a = (dU/dl)/l (b - a), F_b = -F_a
-      if (k_b == 0.f) {
-        add(E.x, fs);
-        add(E.y, (-1.0f) * fs);
-        continue;
-      }
-      // bending: F_v = -s dtheta/dv with dtheta/dc = -L n1/|n1|^2,
-      // dtheta/dd = -L n2/|n2|^2, dtheta/da = -(1-t1) g_c - (1-t2) g_d,
-      // dtheta/db = -t1 g_c - t2 g_d, t1,2 = (c,d - a).(b - a)/L^2
-      const float3 n1 = normal(ET.x), n2 = normal(ET.y);
-      // sin(theta - theta0) = sin(theta) cos(theta0) - cos(theta) sin(theta0), with
-      // cos(theta), sin(theta) from the normals (no inverse trigonometry)
-      const float inv = rsqrtf(dot(n1, n1) * dot(n2, n2));
-      const float cth = dot(n1, n2) * inv, sth = dot(cross(n1, n2), ev) * rl * inv;
-      const float sb = k_b * (sth * rest.y - cth * rest.z);
-      const float3 gc = __fdividef(-l, dot(n1, n1)) * n1, gd = __fdividef(-l, dot(n2, n2)) * n2;
-      const float t1 = dot(dv(E.z, E.x), ev) * rL2, t2 = dot(dv(E.w, E.x), ev) * rL2;
-      add(E.x, fs + (sb * (1.0f - t1)) * gc + (sb * (1.0f - t2)) * gd);
-      add(E.y, (-1.0f) * fs + (sb * t1) * gc + (sb * t2) * gd);
-      add(E.z, (-sb) * gc);
-      add(E.w, (-sb) * gd);
+      edge_forces(E, ET, rest, kBT_p, k_b, dv, normal, add);
     }
     ushort4 Trn = make_ushort4(0, 0, 0, 0);
     float A0n = 1.f;
@@ -270,18 +315,7 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
         Trn = T.tris[t + blockDim.x];
         A0n = T.area0[t + blockDim.x];
       }
-      const int vv[3] = {Tr.x, Tr.y, Tr.z};
-      const float3 N = normal(t);
-      const float At = sA[t];
-      const float coef = k_l * __fdividef(At - At0, At0) + cg;
-      const float3 nh = __fdividef(0.5f, At) * N;
-      const float3 fV = (-cv / 6.0f) * N;
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        // F_v = -coef dA_t/dx_v - (k_v (V - V0)/V0) N_t / 6, dA_t/dx_v = 1/2 n x (x_{v+2} - x_{v+1})
-        const float3 gA = cross(nh, dv(vv[(q + 2) % 3], vv[(q + 1) % 3]));
-        add(vv[q], (-0.5f * coef) * gA + fV);
-      }
+      triangle_forces(Tr, normal(t), sA[t], At0, k_l, cg, cv, dv, add);
     }
   };
   const float Sq = q_prev > 0.f ? mesh.qcap / (4.0f * q_prev) : 0.f;

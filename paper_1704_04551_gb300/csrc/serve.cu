@@ -106,11 +106,10 @@ __global__ void __launch_bounds__(RIGID_THREADS) k_rigid_b(const CaseDev* cases,
 
 __global__ void __launch_bounds__(MEMBRANE_THREADS, 4) k_membranes_b(const CaseDev* cases, const Item* items) {
   extern __shared__ __align__(16) unsigned char smem[];
-  __shared__ double red[2 * 32];
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
   if (!C.active) return;
-  membrane_block(C.m, C.bodies + it.i, C.mesh, smem, red);
+  membrane_block(C.m, C.bodies + it.i, C.mesh, smem);
 }
 
 __global__ void __launch_bounds__(SERVE_XFER_THREADS, 2) k_spread_b(const CaseDev* cases, const Item* items) {
