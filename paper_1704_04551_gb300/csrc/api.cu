@@ -17,6 +17,7 @@
 #include <vector>
 
 #include "../../include/ibm_lbm.h"
+#include "cluster_body.cuh"
 #include "common.cuh"
 #include "handle.h"
 #include "internal.h"
@@ -139,7 +140,7 @@ void drop_graphs(ibm_lbm_t* h) {
       if (g) cudaGraphExecDestroy(g);
       g = nullptr;
     }
-  for (auto& g : h->g_fused) {
+  for (auto& g : h->g_mid) {
     if (g) cudaGraphExecDestroy(g);
     g = nullptr;
   }
@@ -154,28 +155,101 @@ LatticeDev lat(const ibm_lbm_t* h, bool odd) {
   return h->L;
 }
 
+// How the markers and the lattice exchange velocities and forces. SEPARATE:
+// forces, spreading and interpolation as kernels of their own. FUSED (many
+// membranes) and CLUSTER (few bodies, rigid or membranes): one kernel between
+// two collisions does the interpolation and advection of a step and the forces
+// and spreading of the next, into the force density (and, for CLUSTER, the
+// tile flags) that the next collision reads; the buffers alternate.
+enum Path { SEPARATE, FUSED, CLUSTERED };
+
+// Membranes take clusters up to this many bodies. One block per body
+// (couple.cu) does less work in all, but its latency decides while the
+// bodies do not fill the chip.
+constexpr int CLUSTER_MEMBRANES_MAX = 38;
+
+Path path_of(const ibm_lbm_t* h) {
+  if (h->m.M == 0 || h->morse_rc > 0.0) return SEPARATE;
+  if (h->cluster_boxes) return CLUSTERED;
+  return h->n_couple > 0 ? FUSED : SEPARATE;
+}
+
+// Lattice view of a step that uses force-density buffer k (0 or 1).
+LatticeDev lattice_of(const ibm_lbm_t* h, Path p, int k) {
+  LatticeDev L = h->L;
+  if (p != SEPARATE && k) L.g = h->gbuf2;
+  if (p == CLUSTERED && k) L.flags = h->fbuf2;
+  return L;
+}
+
+void enqueue_cluster(ibm_lbm_t* h, int k, int next, bool interp, bool forces, bool spread) {
+  const LatticeDev L = lattice_of(h, CLUSTERED, k), Ln = lattice_of(h, CLUSTERED, next);
+  launch_couple_cluster(L, Ln.g, Ln.flags, h->m, h->d_bodies, h->rigid_list, h->n_rigids, false, h->cluster_max,
+                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, h->stream);
+  launch_couple_cluster(L, Ln.g, Ln.flags, h->m, h->d_bodies, h->membrane_list, h->n_membranes, true, h->mesh.nv,
+                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, h->stream);
+}
+
 // Marker forces: each body's own forces (membranes, rigid tethers,
 // filaments), then the Morse excluded volume between bodies.
 void enqueue_forces(ibm_lbm_t* h, cudaStream_t st) {
   if (h->m.M == 0) return;
   if (h->need_zero_F) cudaMemsetAsync(h->m.F, 0, sizeof(float4) * (size_t)h->m.M, st);
-  launch_forces(h->m, h->d_bodies, h->membrane_list, h->n_membranes, h->rigid_list, h->n_rigids, h->mesh, st);
+  if (h->cluster_boxes)
+    enqueue_cluster(h, 0, 0, false, true, false);
+  else
+    launch_forces(h->m, h->d_bodies, h->membrane_list, h->n_membranes, h->rigid_list, h->n_rigids, h->mesh, st);
   launch_filaments(h->m, h->d_bodies, h->filament_list, h->n_filaments, st);
   if (h->morse_rc > 0.0 && h->morse_ready)
     launch_morse(h->morse, h->m, h->cfg.nx, h->cfg.ny, h->cfg.nz, h->cfg.geometry, st);
 }
 
-// One coupled step on the handle's stream (also used under capture).
-void enqueue_step(ibm_lbm_t* h, bool odd, bool dense) {
+// Forces and spreading of the first step into buffer k.
+void couple_begin(ibm_lbm_t* h, Path p, int k) {
   cudaStream_t st = h->stream;
-  const LatticeDev L = lat(h, odd);
-  cudaMemsetAsync(L.flags, 0, (size_t)tiles(L), st);
-  if (h->m.M > 0) {
-    enqueue_forces(h, st);
-    launch_spread(L, h->m, h->groups, h->n_groups, h->boxes, st);
+  const LatticeDev L = lattice_of(h, p, k);
+  cudaMemsetAsync(h->fbuf, 0, (size_t)tiles(L), st);
+  if (h->m.M == 0) return;
+  if (p == CLUSTERED) {
+    cudaMemsetAsync(h->fbuf2, 0, (size_t)tiles(L), st);
+    enqueue_cluster(h, k, k, false, true, true);
+    return;
   }
-  launch_collide(L, h->rows, h->n_rows, h->cfg.storage, odd, dense, st);
-  if (h->m.M > 0) launch_interpolate(L, h->m, h->groups, h->n_groups, h->boxes, st);
+  enqueue_forces(h, st);
+  launch_spread(L, h->m, h->groups, h->n_groups, h->boxes, st);
+}
+
+// Interpolation and advection of the step that used buffer k, forces and
+// spreading of the next into the other one.
+void couple_mid(ibm_lbm_t* h, Path p, int k) {
+  if (p == CLUSTERED) {
+    enqueue_cluster(h, k, k ^ 1, true, true, true);
+    return;
+  }
+  const LatticeDev L = lattice_of(h, p, k);
+  cudaMemsetAsync(L.flags, 0, (size_t)tiles(L), h->stream);
+  launch_couple(L, k ? h->gbuf : h->gbuf2, h->m, h->d_bodies, h->couple_items, h->n_couple, h->groups, h->boxes,
+                h->couple_order, h->mesh, h->stream);
+}
+
+// Interpolation and advection of the last step.
+void couple_end(ibm_lbm_t* h, Path p, int k) {
+  if (h->m.M == 0) return;
+  if (p == CLUSTERED) enqueue_cluster(h, k, k, true, false, false);
+  else launch_interpolate(lattice_of(h, p, k), h->m, h->groups, h->n_groups, h->boxes, h->stream);
+}
+
+void collide(ibm_lbm_t* h, Path p, int k, bool odd, bool dense) {
+  launch_collide(lattice_of(h, p, k), h->rows, h->n_rows, h->cfg.storage, odd, dense, h->stream);
+}
+
+// One coupled step by itself on the handle's stream (also used under
+// capture); it needs the first buffers only.
+void enqueue_step(ibm_lbm_t* h, bool odd, bool dense) {
+  const Path p = path_of(h);
+  couple_begin(h, p, 0);
+  collide(h, p, 0, odd, dense);
+  couple_end(h, p, 0);
 }
 
 // One step with an event before each stage and after the last.
@@ -204,14 +278,8 @@ void enqueue_timed_step(ibm_lbm_t* h, bool odd, bool dense) {
   }
 }
 
-int capture(ibm_lbm_t* h, cudaGraphExec_t* out, int n, bool odd0, bool dense_last) {
+int end_capture(ibm_lbm_t* h, cudaGraphExec_t* out) {
   cudaGraph_t g = nullptr;
-  CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-  bool odd = odd0;
-  for (int s = 0; s < n; ++s) {
-    enqueue_step(h, odd, dense_last && s == n - 1);
-    odd = !odd;
-  }
   CUDA_TRY(h, cudaStreamEndCapture(h->stream, &g));
   cudaError_t e = cudaGraphInstantiate(out, g, 0);
   cudaGraphDestroy(g);
@@ -219,64 +287,74 @@ int capture(ibm_lbm_t* h, cudaGraphExec_t* out, int n, bool odd0, bool dense_las
   return IBM_LBM_OK;
 }
 
-// The fused path: n (even) coupled steps starting at an even AA step. The
-// first step's forces and spreading run as separate kernels into the first
-// force-density buffer; then every step is the collision (reading the
-// buffer of its parity) followed by the fused kernel, which interpolates and
-// advects, computes the forces at the new positions and spreads them into
-// the other buffer; the last step's interpolation runs alone. The tile flags
-// are cleared between a collision and the spreading that follows it.
-bool fused_applies(const ibm_lbm_t* h) {
-  return h->n_couple > 0 && (!h->timing || h->timing_fused) && !(h->morse_rc > 0.0) && h->gbuf2 != nullptr;
+int capture(ibm_lbm_t* h, cudaGraphExec_t* out, int n, bool odd0, bool dense_last) {
+  CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
+  bool odd = odd0;
+  for (int s = 0; s < n; ++s) {
+    enqueue_step(h, odd, dense_last && s == n - 1);
+    odd = !odd;
+  }
+  return end_capture(h, out);
 }
 
-// With timed, the steps that launch the fused kernel record the events
-// around the collision and around the tile-flag clear and the fused kernel
-// (the forces and spreading slots of such a step are not read); the first
-// step's forces and spreading and the last step's interpolation lie outside
-// the timed intervals.
-void enqueue_fused_chunk(ibm_lbm_t* h, int n, bool timed) {
-  cudaStream_t st = h->stream;
-  LatticeDev L0 = h->L;
-  L0.g = h->gbuf;
-  cudaMemsetAsync(L0.flags, 0, (size_t)tiles(L0), st);
-  enqueue_forces(h, st);
-  launch_spread(L0, h->m, h->groups, h->n_groups, h->boxes, st);
+// n times (even) collision and coupling into the next step, from an even
+// step on: step parity and buffer alternate together.
+int capture_mid(ibm_lbm_t* h, Path p, cudaGraphExec_t* out, int n) {
+  CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
   for (int s = 0; s < n; ++s) {
-    const size_t base = 5 * h->timed_steps;
-    const bool rec = timed && s + 1 < n && base + 5 <= h->events.size();
-    auto mark = [&](int k) {
-      if (rec) cudaEventRecord(h->events[base + k], st);
-    };
-    LatticeDev Ls = h->L;
-    Ls.g = (s & 1) ? h->gbuf2 : h->gbuf;
-    mark(2);
-    launch_collide(Ls, h->rows, h->n_rows, h->cfg.storage, (s & 1) != 0, false, st);
-    mark(3);
-    if (s + 1 < n) {
-      cudaMemsetAsync(Ls.flags, 0, (size_t)tiles(Ls), st);
-      launch_couple(Ls, (s & 1) ? h->gbuf : h->gbuf2, h->m, h->d_bodies, h->couple_items, h->n_couple, h->groups,
-                    h->boxes, h->couple_order, h->mesh, st);
-    } else {
-      launch_interpolate(Ls, h->m, h->groups, h->n_groups, h->boxes, st);
+    collide(h, p, s & 1, (s & 1) != 0, false);
+    couple_mid(h, p, s & 1);
+  }
+  return end_capture(h, out);
+}
+
+// Whether a call of n steps couples two steps with one kernel.
+bool fused_applies(const ibm_lbm_t* h) {
+  return path_of(h) != SEPARATE && (!h->timing || h->timing_fused) && h->gbuf2 != nullptr;
+}
+
+// n coupled steps on a fused path, the last one with the moments of every
+// cell if dense: the first step's forces and spreading, then collision and
+// coupling by turns, the last step's interpolation alone. With timed, the
+// steps that launch the coupling kernel record events around the collision
+// and around the coupling (the forces and spreading slots of such a step are
+// not read); kernels are then launched directly.
+int enqueue_fused(ibm_lbm_t* h, int64_t n, bool dense, bool timed) {
+  cudaStream_t st = h->stream;
+  const Path p = path_of(h);
+  int k = h->odd_next ? 1 : 0;  // the buffer goes with the AA parity
+  couple_begin(h, p, k);
+  int64_t mids = n - 1;
+  while (mids > 0) {
+    const int which = mids >= FUSED_LONG ? 0 : 1, len = which == 0 ? FUSED_LONG : CHUNK;
+    if (!timed && k == 0 && mids >= len) {
+      if (!h->g_mid[which]) {
+        const int rc = capture_mid(h, p, &h->g_mid[which], len);
+        if (rc) return rc;
+      }
+      CUDA_TRY(h, cudaGraphLaunch(h->g_mid[which], st));
+      mids -= len;
+      continue;
     }
-    mark(4);
+    const size_t base = 5 * h->timed_steps;
+    const bool rec = timed && base + 5 <= h->events.size();
+    if (rec) cudaEventRecord(h->events[base + 2], st);
+    collide(h, p, k, k != 0, false);
+    if (rec) cudaEventRecord(h->events[base + 3], st);
+    couple_mid(h, p, k);
     if (rec) {
-      h->timed_odd.push_back((s & 1) ? 1 : 0);
+      cudaEventRecord(h->events[base + 4], st);
+      h->timed_odd.push_back(k != 0 ? 1 : 0);
       h->timed_fused.push_back(1);
       h->timed_steps++;
     }
+    k ^= 1;
+    --mids;
   }
-}
-
-int capture_fused(ibm_lbm_t* h, cudaGraphExec_t* out, int n) {
-  cudaGraph_t g = nullptr;
-  CUDA_TRY(h, cudaStreamBeginCapture(h->stream, cudaStreamCaptureModeThreadLocal));
-  enqueue_fused_chunk(h, n, false);
-  CUDA_TRY(h, cudaStreamEndCapture(h->stream, &g));
-  cudaError_t e = cudaGraphInstantiate(out, g, 0);
-  cudaGraphDestroy(g);
-  if (e != cudaSuccess) return fail(h, IBM_LBM_E_CUDA, std::string("cudaGraphInstantiate: ") + cudaGetErrorString(e));
+  collide(h, p, k, k != 0, dense);
+  couple_end(h, p, k);
+  h->steps += n;
+  if (n & 1) h->odd_next = !h->odd_next;
   return IBM_LBM_OK;
 }
 
@@ -313,24 +391,22 @@ int enqueue_steps(ibm_lbm_t* h, int64_t n) {
   if (n == 0) return IBM_LBM_OK;
   h->boxes_valid = false;  // the last interpolation moves the markers
   int64_t left = n;
-  if (h->n_couple > 0 && !h->gbuf2 && (h->timing ? h->timing_fused && left > 2 : left > CHUNK)) {
-    // second force-density buffer of the fused path, zero like the first
+  if (path_of(h) != SEPARATE && !h->gbuf2 && (h->timing ? h->timing_fused && left > 2 : left > 1)) {
+    // second force-density buffer of the fused paths, zero like the first
     h->gbuf2 = (float4*)dalloc(h, h->lattice_mem, sizeof(float4) * (size_t)h->L.N);
     if (h->gbuf2) CUDA_TRY(h, cudaMemsetAsync(h->gbuf2, 0, sizeof(float4) * (size_t)h->L.N, h->stream));
   }
+  const bool fused = fused_applies(h);
   if (h->timing) {
-    // with timing_fused, a handle on the fused path times only its fused
-    // steps; every other handle is timed stage by stage
-    const bool fused = h->timing_fused && fused_applies(h);
+    // with timing_fused, a handle on a fused path times only its coupled
+    // steps, the last one of the call apart; every other handle is timed
+    // stage by stage
     while (left > 0) {
       if (fused && !h->odd_next && left > 2) {
-        // the fused path with direct launches; the last step stays separate
-        // (it writes the velocity of every cell)
         const int m = (int)std::min<int64_t>(left - 1, 1 << 22);
-        enqueue_fused_chunk(h, m, true);
+        const int rc = enqueue_fused(h, m, false, true);
+        if (rc) return rc;
         left -= m;
-        h->steps += m;
-        if (m & 1) h->odd_next = !h->odd_next;
         continue;
       }
       if (fused) enqueue_step(h, h->odd_next, left == 1);
@@ -342,18 +418,14 @@ int enqueue_steps(ibm_lbm_t* h, int64_t n) {
     CUDA_TRY(h, cudaGetLastError());
     return enqueue_diagnostics(h);
   }
+  if (fused && left > 1) {
+    const int rc = enqueue_fused(h, left, true, false);
+    if (rc) return rc;
+    CUDA_TRY(h, cudaGetLastError());
+    return enqueue_diagnostics(h);
+  }
   while (left > 0) {
-    if (fused_applies(h) && !h->odd_next && left > CHUNK) {
-      const int which = left > FUSED_LONG ? 0 : 1;
-      const int n = which == 0 ? FUSED_LONG : CHUNK;
-      if (!h->g_fused[which]) {
-        int rc = capture_fused(h, &h->g_fused[which], n);
-        if (rc) return rc;
-      }
-      CUDA_TRY(h, cudaGraphLaunch(h->g_fused[which], h->stream));
-      left -= n;
-      h->steps += n;
-    } else if (!h->odd_next && left > CHUNK) {
+    if (!h->odd_next && left > CHUNK) {
       if (!h->g_chunk) {
         int rc = capture(h, &h->g_chunk, CHUNK, false, false);
         if (rc) return rc;
@@ -454,6 +526,62 @@ void order_for_banks(HostMesh& m) {
   }
   m.edges.swap(edges);
   m.edge_tris.swap(et);
+}
+
+// The part of a template that the vertices [v0, v1) need: every edge that has
+// one of them among its four, with both its triangles (the forces on c and d
+// need their normals), and every triangle that has one of them; those first.
+struct MeshPartHost {
+  std::vector<ushort4> edges, tris;
+  std::vector<ushort2> edge_tris;
+  std::vector<float4> edge_rest;
+  std::vector<float> area0;
+  int nt_own = 0;
+};
+MeshPartHost mesh_part_of(const HostMesh& m, int v0, int v1) {
+  auto own = [&](int v) { return v >= v0 && v < v1; };
+  MeshPartHost P;
+  std::vector<int> touching, ghosts, edges;
+  std::vector<int> local(m.tris.size(), -1);
+  for (size_t t = 0; t < m.tris.size(); ++t)
+    if (own(m.tris[t].x) || own(m.tris[t].y) || own(m.tris[t].z)) {
+      touching.push_back((int)t);
+      local[t] = 0;
+    }
+  for (size_t e = 0; e < m.edges.size(); ++e) {
+    const int4 E = m.edges[e];
+    if (!own(E.x) && !own(E.y) && !own(E.z) && !own(E.w)) continue;
+    edges.push_back((int)e);
+    for (int t : {m.edge_tris[e].x, m.edge_tris[e].y})
+      if (local[t] < 0) {
+        local[t] = 0;
+        ghosts.push_back(t);
+      }
+  }
+  std::vector<std::array<int, 3>> tk;
+  for (int t : touching) tk.push_back({m.tris[t].x, m.tris[t].y, m.tris[t].z});
+  P.nt_own = (int)touching.size();
+  std::vector<int> order;
+  for (int i : bank_order<3>(tk)) order.push_back(touching[i]);
+  order.insert(order.end(), ghosts.begin(), ghosts.end());
+  for (size_t i = 0; i < order.size(); ++i) {
+    const int t = order[i];
+    local[t] = (int)i;
+    P.tris.push_back(make_ushort4(m.tris[t].x, m.tris[t].y, m.tris[t].z, own(m.tris[t].x) ? 1 : 0));
+    P.area0.push_back(m.area0[t]);
+  }
+  std::vector<std::array<int, 6>> ek;
+  for (int e : edges) {
+    const int4 E = m.edges[e];
+    ek.push_back({E.x, E.y, E.z, E.w, local[m.edge_tris[e].x], local[m.edge_tris[e].y]});
+  }
+  for (int i : bank_order<6>(ek)) {
+    const int e = edges[i];
+    P.edges.push_back(make_ushort4(ek[i][0], ek[i][1], ek[i][2], ek[i][3]));
+    P.edge_tris.push_back(make_ushort2(ek[i][4], ek[i][5]));
+    P.edge_rest.push_back(m.edge_rest[e]);
+  }
+  return P;
 }
 
 bool build_mesh(const ibm_lbm_mesh* mesh, HostMesh& out, std::string& why) {
@@ -725,12 +853,13 @@ static int impl_ibm_lbm_create(const ibm_lbm_config* cfg, const ibm_lbm_allocato
   L.uw = (float4*)dalloc(h, h->lattice_mem, sizeof(float4) * N);
   h->gbuf = (float4*)dalloc(h, h->lattice_mem, sizeof(float4) * N);
   h->fbuf = (uint8_t*)dalloc(h, h->lattice_mem, (size_t)tiles(L));
+  h->fbuf2 = (uint8_t*)dalloc(h, h->lattice_mem, (size_t)tiles(L));
   L.g = h->gbuf;  // every view of the lattice (steps, stages, server) carries them
   L.flags = h->fbuf;
   L.status = (int*)dalloc(h, h->lattice_mem, 256);
   h->d_diag = (double*)dalloc(h, h->lattice_mem, 8 * sizeof(double));
   h->d_umax = (unsigned*)dalloc(h, h->lattice_mem, 256);
-  if (!L.pop || !L.uw || !h->gbuf || !h->fbuf || !L.status || !h->d_diag ||
+  if (!L.pop || !L.uw || !h->gbuf || !h->fbuf || !h->fbuf2 || !L.status || !h->d_diag ||
       !h->d_umax) {
     h->err = "device allocation failed";
     return bail(IBM_LBM_E_NOMEM);
@@ -742,7 +871,8 @@ static int impl_ibm_lbm_create(const ibm_lbm_config* cfg, const ibm_lbm_allocato
   }
   if (cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess)
     return bail(IBM_LBM_E_CUDA);
-  if (transfer_configure() != cudaSuccess || couple_configure() != cudaSuccess) {
+  if (transfer_configure() != cudaSuccess || couple_configure() != cudaSuccess ||
+      cluster_configure() != cudaSuccess) {
     cudaGetLastError();
     return bail(IBM_LBM_E_CUDA);
   }
@@ -873,6 +1003,8 @@ static void clear_markers(ibm_lbm_t* h) {
   h->couple_items = nullptr;
   h->n_couple = 0;
   h->couple_order = nullptr;
+  h->cluster_boxes = nullptr;
+  h->cluster_max = 0;
   h->need_zero_F = false;
 }
 
@@ -962,9 +1094,12 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.count = (int)B.count;
     D.kBT_p = (float)B.kBT_p; D.k_b = (float)B.k_b; D.k_l = (float)B.k_l; D.k_g = (float)B.k_g; D.k_v = (float)B.k_v;
     D.kappa = B.kappa; D.mass = B.mass;
+    D.inv_mass = B.mass > 0 ? 1.0 / B.mass : 0.0;
     D.l0 = (float)B.l0;
     for (int a = 0; a < 3; ++a) {
-      D.inertia[a] = B.inertia[a]; D.center[a] = B.center[a]; D.vel[a] = B.vel[a]; D.omega[a] = B.omega[a];
+      D.inertia[a] = B.inertia[a];
+      D.inv_inertia[a] = B.inertia[a] > 0 ? 1.0 / B.inertia[a] : 0.0;
+      D.center[a] = B.center[a]; D.vel[a] = B.vel[a]; D.omega[a] = B.omega[a];
     }
     for (int a = 0; a < 4; ++a) D.quat[a] = B.quat[a];
     h->h_bodies.push_back(B);
@@ -1019,6 +1154,24 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.off_ve = section(vel.data(), vel.size() * 2);
     D.off_vt_start = section(vts.data(), vts.size() * 2);
     D.off_vt = section(vtl.data(), vtl.size() * 2);
+    {
+      // parts of consecutive vertices (cluster_body.cuh)
+      int table[CLUSTER][8] = {};
+      D.part_tris = 0;
+      const int per = cluster_per(mesh->n_vertices);
+      for (int p = 0; p < CLUSTER; ++p) {
+        const MeshPartHost P = mesh_part_of(hm, p * per, std::min(mesh->n_vertices, (p + 1) * per));
+        const int t[8] = {(int)P.edges.size(), (int)P.tris.size(), P.nt_own,
+                          section(P.edges.data(), P.edges.size() * sizeof(ushort4)),
+                          section(P.edge_tris.data(), P.edge_tris.size() * sizeof(ushort2)),
+                          section(P.edge_rest.data(), P.edge_rest.size() * sizeof(float4)),
+                          section(P.tris.data(), P.tris.size() * sizeof(ushort4)),
+                          section(P.area0.data(), P.area0.size() * sizeof(float))};
+        std::copy(t, t + 8, table[p]);
+        D.part_tris = std::max(D.part_tris, t[1]);
+      }
+      D.off_parts = section(table, sizeof(table));
+    }
     D.packed_bytes = (int)buf.size();
     unsigned char* dpk = nullptr;
     if ((rc = upload<unsigned char>(h, h->marker_mem, &dpk, buf.data(), buf.size()))) return rc;
@@ -1126,6 +1279,26 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     // no box until the first spreading: an interpolation run before it (the
     // stage interface allows that) takes the per-marker path
     CUDA_TRY(h, cudaMemset(h->boxes, 0, sizeof(int4) * 2 * std::max<size_t>(1, groups.size())));
+  }
+  // clusters: bodies of a size one cluster takes, nothing else
+  {
+    bool few = n_bodies > 0 && covered == n_markers && h->n_filaments == 0 && h->n_membranes <= CLUSTER_MEMBRANES_MAX;
+    for (int b = 0; b < n_bodies && few; ++b) {
+      few = bodies[b].count <= CLUSTER_MAX_COUNT;
+      h->cluster_max = std::max(h->cluster_max, (int)bodies[b].count);
+    }
+    few = few && (h->n_rigids == 0 ||
+                  cluster_box_cells(cluster_fixed_words(h->cluster_max, 0, 0), h->n_rigids, h->n_sm) > 0);
+    few = few && (h->n_membranes == 0 ||
+                  cluster_box_cells(cluster_fixed_words(h->mesh.nv, h->mesh.nv, h->mesh.part_tris), h->n_membranes,
+                                    h->n_sm) > 0);
+    if (few) {
+      const size_t bytes = sizeof(int4) * 2 * CLUSTER * (size_t)n_bodies;
+      int4* boxes = (int4*)dalloc(h, h->marker_mem, bytes);
+      if (!boxes) return fail(h, IBM_LBM_E_NOMEM, "device allocation failed");
+      CUDA_TRY(h, cudaMemset(boxes, 0, bytes));
+      h->cluster_boxes = boxes;
+    }
   }
   h->need_zero_F = covered < n_markers;
   if (h->morse_rc > 0.0) return prepare_morse(h);

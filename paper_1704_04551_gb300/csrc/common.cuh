@@ -11,6 +11,10 @@ namespace ibm {
 
 constexpr int Q = 19;
 
+// Thread blocks that share one body's coupling where there are few bodies
+// (cluster_body.cuh; the portable cluster size).
+constexpr int CLUSTER = 8;
+
 // Velocities in the public D3Q19 order: rest, +-x, +-y, +-z, then the face
 // diagonals in opposite pairs, so that opposite(i) = i + 1 for odd i and
 // i - 1 for even i > 0.
@@ -132,6 +136,7 @@ struct BodyDev {
   int first, count;
   float kBT_p, k_b, k_l, k_g, k_v;
   double kappa, mass, inertia[3];
+  double inv_mass, inv_inertia[3];
   double center[3], quat[4], vel[3], omega[3];
   float qmax;  // membranes: largest force contribution component of the last step (0: none yet)
   float l0;    // filaments: rest bond length
@@ -148,6 +153,11 @@ struct MeshDev {
   const unsigned char* packed;
   int packed_bytes;  // multiple of 16
   int off_edges, off_edge_tris, off_edge_rest, off_tris, off_area0, off_ve_start, off_ve, off_vt_start, off_vt;
+  // The template in CLUSTER parts of consecutive vertices (cluster_body.cuh):
+  // a table [CLUSTER][8] of (edges, triangles, triangles that touch the part,
+  // offsets of edges, edge_tris, edge_rest, tris, area0), each part with its
+  // own copy of the edges that touch its vertices and of their triangles.
+  int off_parts, part_tris;  // part_tris: largest triangle count of a part
   int work_floats;   // per-body shared work area: 9 nv + 4 nt words
   float A0, V0;
   float fix_a, fix_v;  // powers of two: fixed-point scales of the area and volume sums

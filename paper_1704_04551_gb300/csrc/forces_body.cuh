@@ -159,6 +159,31 @@ __device__ __forceinline__ void triangle_forces(const ushort4 Tr, float3 N, floa
   }
 }
 
+// One part of the template (MeshDev::off_parts): the edges that touch its
+// vertices and their triangles, those that touch its vertices (nt_own) first;
+// tris.w is set where the triangle counts for the body's area and volume.
+struct MeshPart {
+  int ne, nt, nt_own;
+  const ushort4* edges;
+  const ushort2* edge_tris;  // indices into the part's triangles
+  const float4* edge_rest;
+  const ushort4* tris;
+  const float* area0;
+};
+__device__ __forceinline__ MeshPart mesh_part(const MeshDev& mesh, int p) {
+  const int* t = reinterpret_cast<const int*>(mesh.packed + mesh.off_parts) + 8 * p;
+  MeshPart P;
+  P.ne = t[0];
+  P.nt = t[1];
+  P.nt_own = t[2];
+  P.edges = reinterpret_cast<const ushort4*>(mesh.packed + t[3]);
+  P.edge_tris = reinterpret_cast<const ushort2*>(mesh.packed + t[4]);
+  P.edge_rest = reinterpret_cast<const float4*>(mesh.packed + t[5]);
+  P.tris = reinterpret_cast<const ushort4*>(mesh.packed + t[6]);
+  P.area0 = reinterpret_cast<const float*>(mesh.packed + t[7]);
+  return P;
+}
+
 }  // namespace forces_detail
 using namespace forces_detail;
 

@@ -73,6 +73,11 @@ struct ibm_lbm {
   // vertices' residue counters and order (couple_order_bytes each)
   unsigned char* couple_order = nullptr;
   float4* gbuf2 = nullptr;        // second force density (allocated on first use)
+  // Few bodies, all rigid or membranes: a cluster of thread blocks per body
+  // does the same (cluster_body.cuh); boxes of its blocks [n_bodies][CLUSTER][2].
+  int4* cluster_boxes = nullptr;  // set: the path applies to these markers
+  int cluster_max = 0;            // largest marker count of a body
+  uint8_t* fbuf2 = nullptr;       // second tile flags (beside gbuf2)
   bool boxes_valid = false;       // boxes match the markers' current positions (stage interface)
   bool need_zero_F = false;
   // state
@@ -93,7 +98,8 @@ struct ibm_lbm {
   bool timing_fused = false;  // time the fused path where it applies
   // graphs
   cudaGraphExec_t g_chunk = nullptr;
-  cudaGraphExec_t g_fused[2] = {nullptr, nullptr};  // fused chunks of FUSED_LONG and CHUNK steps
+  // FUSED_LONG and CHUNK times (collision, coupling into the next step), from an even step on
+  cudaGraphExec_t g_mid[2] = {nullptr, nullptr};
   cudaGraphExec_t g_single[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   std::string err;
 };

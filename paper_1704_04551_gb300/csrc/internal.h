@@ -42,6 +42,14 @@ void launch_couple(const LatticeDev& L, float4* g_next, const MarkersDev& m, Bod
                    int n_items, const MarkerGroup* groups, int4* boxes, unsigned char* orders, const MeshDev& mesh,
                    cudaStream_t st);
 
+// cluster.cu (few bodies: a cluster of thread blocks per body)
+cudaError_t cluster_configure();
+int cluster_box_cells(size_t fixed_words, int n_clusters, int n_sm);
+void launch_couple_cluster(const LatticeDev& L, float4* g_next, uint8_t* flags_next, const MarkersDev& m,
+                           BodyDev* bodies, const int* list, int n, bool membranes, int max_count,
+                           const MeshDev& mesh, int4* boxes, int n_sm, bool interp, bool forces, bool spread,
+                           cudaStream_t st);
+
 // solid.cu
 void launch_solid_half(const MarkersDev& m, double* v, const double* fext, double dt, double gamma, double mass,
                        bool first, cudaStream_t st);

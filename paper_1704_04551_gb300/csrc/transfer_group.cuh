@@ -137,7 +137,8 @@ __device__ __forceinline__ int axis_tiles(int b, int n, int sh, int t[2]) {
 // equals that of the previous lane's marker skips its stores. All 32 lanes
 // of the warp call this.
 template <int GEOM>
-__device__ __forceinline__ void mark_tiles(const LatticeDev& L, int bx, int by, int bz, bool active) {
+__device__ __forceinline__ void mark_tiles(const LatticeDev& L, int bx, int by, int bz, bool active,
+                                           uint8_t value = 1) {
   int tx[2] = {-1, -1}, ty[2] = {-1, -1}, tz[2] = {-1, -1};
   const int nx_ = axis_tiles<true>(bx, L.nx, TILE_X_SHIFT, tx);
   const int ny_ = GEOM == GEOM_PERIODIC ? axis_tiles<true>(by, L.ny, TILE_Y_SHIFT, ty)
@@ -155,7 +156,7 @@ __device__ __forceinline__ void mark_tiles(const LatticeDev& L, int bx, int by, 
   if (!active || same) return;
   for (int c = 0; c < nz_; ++c)
     for (int b = 0; b < ny_; ++b)
-      for (int a = 0; a < nx_; ++a) L.flags[tx[a] + L.ntx * (ty[b] + L.nty * tz[c])] = 1;
+      for (int a = 0; a < nx_; ++a) L.flags[tx[a] + L.ntx * (ty[b] + L.nty * tz[c])] = value;
 }
 
 // Tiles covered by nodes lo .. lo + n - 1 (unwrapped) of an axis of `size`
@@ -183,11 +184,12 @@ __device__ __forceinline__ int axis_tile_ranges(int lo, int n, int size, int sh,
   return 1;
 }
 
-// Mark every tile that intersects the box [lo, lo + dims) by the whole
-// block: a superset of the tiles the group's stencils touch, at a cost of a
+// Set the flags of every tile that intersects the box [lo, lo + dims) by
+// `threads` threads (by default the whole block sets them): a superset of the tiles the group's stencils touch, at a cost of a
 // few stores per group.
 template <int GEOM>
-__device__ __forceinline__ void mark_box_tiles(const LatticeDev& L, int4 lo, int4 dims) {
+__device__ __forceinline__ void mark_box_tiles(const LatticeDev& L, int4 lo, int4 dims, int tid, int threads,
+                                               uint8_t value) {
   int2 rx[2], ry[2], rz[2];
   const int nrx = axis_tile_ranges<true>(lo.x, dims.x, L.nx, TILE_X_SHIFT, rx);
   const int nry = GEOM == GEOM_PERIODIC ? axis_tile_ranges<true>(lo.y, dims.y, L.ny, TILE_Y_SHIFT, ry)
@@ -198,11 +200,15 @@ __device__ __forceinline__ void mark_box_tiles(const LatticeDev& L, int4 lo, int
     for (int iy = 0; iy < nry; ++iy)
       for (int ix = 0; ix < nrx; ++ix) {
         const int ax = rx[ix].y - rx[ix].x + 1, ay = ry[iy].y - ry[iy].x + 1, az = rz[iz].y - rz[iz].x + 1;
-        for (int i = threadIdx.x; i < ax * ay * az; i += blockDim.x) {
+        for (int i = tid; i < ax * ay * az; i += threads) {
           const int tx = rx[ix].x + i % ax, ty = ry[iy].x + (i / ax) % ay, tz = rz[iz].x + i / (ax * ay);
-          L.flags[tx + L.ntx * (ty + L.nty * tz)] = 1;
+          L.flags[tx + L.ntx * (ty + L.nty * tz)] = value;
         }
       }
+}
+template <int GEOM>
+__device__ __forceinline__ void mark_box_tiles(const LatticeDev& L, int4 lo, int4 dims) {
+  mark_box_tiles<GEOM>(L, lo, dims, threadIdx.x, blockDim.x, 1);
 }
 
 // Bounding box of the group's stencil nodes (unwrapped coordinates) and the
