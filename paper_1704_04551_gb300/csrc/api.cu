@@ -392,9 +392,7 @@ int enqueue_steps(ibm_lbm_t* h, int64_t n) {
   h->boxes_valid = false;  // the last interpolation moves the markers
   int64_t left = n;
   if (path_of(h) != SEPARATE && !h->gbuf2 && (h->timing ? h->timing_fused && left > 2 : left > 1)) {
-    // second force-density buffer of the fused paths, zero like the first
-    h->gbuf2 = (float4*)dalloc(h, h->lattice_mem, sizeof(float4) * (size_t)h->L.N);
-    if (h->gbuf2) CUDA_TRY(h, cudaMemsetAsync(h->gbuf2, 0, sizeof(float4) * (size_t)h->L.N, h->stream));
+    if (!ensure_second_buffer(h)) CUDA_TRY(h, cudaGetLastError());  // (no memory: separate kernels)
   }
   const bool fused = fused_applies(h);
   if (h->timing) {
@@ -793,6 +791,15 @@ int prepare_morse(ibm_lbm_t* h) {
 }
 
 }  // namespace
+
+bool ibm::ensure_second_buffer(ibm_lbm* h) {
+  if (h->gbuf2) return true;
+  const size_t bytes = sizeof(float4) * (size_t)h->L.N;
+  float4* g = (float4*)dalloc(h, h->lattice_mem, bytes);
+  if (!g || cudaMemsetAsync(g, 0, bytes, h->stream) != cudaSuccess) return false;  // (freed with the lattice)
+  h->gbuf2 = g;
+  return true;
+}
 
 extern "C" {
 

@@ -50,6 +50,8 @@ constexpr int CLUSTER_MAX_COUNT = 4096;  // markers per body
 constexpr int CLUSTER_BOX_MAX = 12288;   // cells of a block's box
 constexpr int CLUSTER_PER_SM = 2;        // resident blocks the registers are sized for
 constexpr int CLUSTER_SMEM_SM = 227 * 1024, CLUSTER_SMEM_MAX = 220 * 1024;
+// dynamic shared memory of a block at CLUSTER_PER_SM blocks
+constexpr int CLUSTER_SHARE = CLUSTER_SMEM_SM / CLUSTER_PER_SM - 5 * 1024;
 
 // Shared memory of one block, in this order (floats / ints, 16-byte aligned
 // sections): own markers' cells [3][per], fractions [3][per], forces [3][per]

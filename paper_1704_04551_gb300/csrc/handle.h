@@ -104,3 +104,8 @@ struct ibm_lbm {
   std::string err;
 };
 
+namespace ibm {
+// The second force-density buffer, zero like the first; false if the
+// allocator has no memory for it (api.cu).
+bool ensure_second_buffer(ibm_lbm* h);
+}  // namespace ibm

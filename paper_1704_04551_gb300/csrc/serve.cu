@@ -8,8 +8,11 @@
 //   rows   (case, fluid row)      -> collide-stream-force
 //   groups (case, marker group)   -> spreading, interpolation
 //   bodies (case, body)           -> marker forces
-// and a device-side case table holding each case's arrays, step count and
-// this step's flags (active, AA parity, dense moments on the last step). A
+// and a device-side case table holding each case's arrays and step counts,
+// from which a kernel derives whether a case takes part in a step of the chunk
+// and whether it is its last one (dense moments). Cases whose bodies take
+// clusters (cluster_body.cuh) need two launches a step, collision and coupling;
+// the others, with tracers or large suspensions, run the separate stages. A
 // chunk of steps is captured once per set of admitted cases and replayed as
 // a CUDA graph; a case that reaches its step count mid-chunk is skipped for
 // the rest of it. Between chunks finished cases are retired (results copied
@@ -31,6 +34,7 @@
 #include <vector>
 
 #include "../../include/ibm_lbm.h"
+#include "cluster_body.cuh"
 #include "common.cuh"
 #include "forces_body.cuh"
 #include "handle.h"
@@ -42,9 +46,15 @@ namespace ibm {
 namespace {
 
 struct CaseDev {
-  LatticeDev L;  // g / flags are taken from gbuf / fbuf by parity
-  float4* gbuf;
-  uint8_t* fbuf;
+  LatticeDev L;  // g / flags are taken from gbuf / fbuf (gbuf2 / fbuf2 in odd steps of the cluster path)
+  float4 *gbuf, *gbuf2;
+  uint8_t *fbuf, *fbuf2;
+  int4* cluster_boxes;
+  // Bodies coupled by clusters (cluster_body.cuh; fixed at admission): two
+  // launches a step, collision and coupling. primed: the next step's forces
+  // are spread already.
+  int clustered, primed;
+  int cap;           // cells of a cluster block's box
   const RowInfo* rows;
   MarkersDev m;
   const MarkerGroup* groups;
@@ -53,70 +63,119 @@ struct CaseDev {
   MeshDev mesh;
   long long target;  // steps to run
   long long done;    // steps completed
-  int active, odd, dense, ntiles, zero_F;
+  int ntiles, zero_F;
 };
 
 struct Item {
   int c, i;  // case, row / group / body
 };
 
-__device__ __forceinline__ LatticeDev case_lattice(const CaseDev& C) {
+__device__ __forceinline__ LatticeDev case_lattice(const CaseDev& C, bool second = false) {
   LatticeDev L = C.L;
-  L.g = C.gbuf;
-  L.flags = C.fbuf;
+  L.g = second ? C.gbuf2 : C.gbuf;
+  L.flags = second ? C.fbuf2 : C.fbuf;
   return L;
+}
+
+// Kernels know the step's index s in the chunk; done counts the steps before
+// the chunk.
+struct ChunkStep {
+  bool active, last;
+};
+__device__ __forceinline__ ChunkStep chunk_step(const CaseDev& C, int s) {
+  const long long left = C.target - C.done - s;
+  return {left > 0, left == 1};
+}
+
+// One cluster per (case, body): after the collision of step s (s < 0: before
+// the first step of a case just admitted, forces and spreading only).
+template <int KIND>
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(CLUSTER_THREADS, CLUSTER_PER_SM)
+    k_couple_cluster_b(const CaseDev* __restrict__ cases, const Item* __restrict__ items, int s) {
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ ClusterShare S;
+  const Item it = items[blockIdx.x / CLUSTER];
+  const CaseDev& C = cases[it.c];
+  ClusterArgs A;
+  bool second;  // the finished step's buffers
+  if (s < 0) {
+    if (C.primed || C.done >= C.target) return;
+    second = false;
+    A.interp = false;
+    A.forces = A.spread = true;
+  } else {
+    const ChunkStep st = chunk_step(C, s);
+    if (!st.active) return;
+    second = (s & 1) != 0;  // chunks are even: parity and buffers go with s
+    A.interp = true;
+    A.forces = A.spread = !st.last;
+  }
+  A.L = case_lattice(C, second);
+  const LatticeDev Ln = case_lattice(C, s < 0 ? second : !second);
+  A.g_next = Ln.g;
+  A.flags_next = Ln.flags;
+  A.m = C.m;
+  A.body = C.bodies + it.i;
+  A.mesh = C.mesh;
+  A.boxes = C.cluster_boxes + (size_t)it.i * 2 * CLUSTER;
+  A.cap = C.cap;
+  switch (A.L.geometry) {
+    case GEOM_PERIODIC: cluster_couple<GEOM_PERIODIC, KIND>(A, S, smem); break;
+    case GEOM_YWALLS: cluster_couple<GEOM_YWALLS, KIND>(A, S, smem); break;
+    default: cluster_couple<GEOM_TUBE, KIND>(A, S, smem); break;
+  }
+}
+
+// Start of a chunk: both buffers' tile flags of the cases with clusters that
+// are not primed.
+__global__ void k_chunk_begin(const CaseDev* cases) {
+  const CaseDev& C = cases[blockIdx.x];
+  if (!C.clustered || C.primed) return;
+  for (int i = threadIdx.x; i < C.ntiles; i += blockDim.x) C.fbuf[i] = C.fbuf2[i] = 0;
+}
+__global__ void k_chunk_end(CaseDev* cases, int n, int steps) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  CaseDev& C = cases[t];
+  C.done = C.done + steps < C.target ? C.done + steps : C.target;
+  C.primed = C.clustered;
 }
 
 constexpr int SERVE_XFER_THREADS = XFER_THREADS;
 constexpr int SERVE_COLLIDE_TX = 32, SERVE_COLLIDE_TY = 4;
 
-__global__ void k_book_begin(CaseDev* cases, int n) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  CaseDev& C = cases[t];
-  C.active = C.done < C.target ? 1 : 0;
-  C.odd = (int)(C.done & 1);
-  C.dense = (C.done + 1 == C.target) ? 1 : 0;
-}
-
-__global__ void k_book_end(CaseDev* cases, int n) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= n) return;
-  if (cases[t].active) cases[t].done += 1;
-}
-
-// Start of a step: clear the tile flags this step's spreading marks and,
-// for cases with markers outside every body, the marker forces.
-__global__ void k_clear_flags(const CaseDev* cases) {
+// Start of a step of the cases without clusters: clear the tile flags this
+// step's spreading marks and, for markers outside every body, the forces.
+__global__ void k_clear_flags(const CaseDev* cases, int s) {
   const CaseDev& C = cases[blockIdx.x];
-  if (!C.active) return;
+  if (C.clustered || !chunk_step(C, s).active) return;
   uint8_t* f = C.fbuf;
   for (int i = threadIdx.x; i < C.ntiles; i += blockDim.x) f[i] = 0;
   if (C.zero_F)
     for (int k = threadIdx.x; k < C.m.M; k += blockDim.x) C.m.F[k] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-__global__ void __launch_bounds__(RIGID_THREADS) k_rigid_b(const CaseDev* cases, const Item* items) {
+__global__ void __launch_bounds__(RIGID_THREADS) k_rigid_b(const CaseDev* cases, const Item* items, int s) {
   __shared__ double sh[6 * 32];
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
-  if (!C.active) return;
+  if (!chunk_step(C, s).active) return;
   rigid_block(C.m, C.bodies + it.i, sh);
 }
 
-__global__ void __launch_bounds__(MEMBRANE_THREADS, 4) k_membranes_b(const CaseDev* cases, const Item* items) {
+__global__ void __launch_bounds__(MEMBRANE_THREADS, 4) k_membranes_b(const CaseDev* cases, const Item* items, int s) {
   extern __shared__ __align__(16) unsigned char smem[];
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
-  if (!C.active) return;
+  if (!chunk_step(C, s).active) return;
   membrane_block(C.m, C.bodies + it.i, C.mesh, smem);
 }
 
-__global__ void __launch_bounds__(SERVE_XFER_THREADS, 2) k_spread_b(const CaseDev* cases, const Item* items) {
+__global__ void __launch_bounds__(SERVE_XFER_THREADS, 2) k_spread_b(const CaseDev* cases, const Item* items, int s) {
   extern __shared__ __align__(16) unsigned char ibox[];
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
-  if (!C.active) return;
+  if (!chunk_step(C, s).active) return;
   const LatticeDev L = case_lattice(C);
   int4* box = C.boxes + 2 * it.i;
   switch (L.geometry) {
@@ -126,11 +185,11 @@ __global__ void __launch_bounds__(SERVE_XFER_THREADS, 2) k_spread_b(const CaseDe
   }
 }
 
-__global__ void __launch_bounds__(SERVE_XFER_THREADS, 2) k_interpolate_b(const CaseDev* cases, const Item* items) {
+__global__ void __launch_bounds__(SERVE_XFER_THREADS, 2) k_interpolate_b(const CaseDev* cases, const Item* items, int s) {
   extern __shared__ __align__(16) unsigned char fbox[];
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
-  if (!C.active) return;
+  if (!chunk_step(C, s).active) return;
   const LatticeDev L = case_lattice(C);
   const int4* box = C.boxes + 2 * it.i;
   switch (L.geometry) {
@@ -142,11 +201,11 @@ __global__ void __launch_bounds__(SERVE_XFER_THREADS, 2) k_interpolate_b(const C
 
 // The same for chunks of fewer than LANE_MAX_GROUPS groups (four lanes per
 // marker).
-__global__ void __launch_bounds__(LANE_THREADS, 1) k_spread_bl(const CaseDev* cases, const Item* items) {
+__global__ void __launch_bounds__(LANE_THREADS, 1) k_spread_bl(const CaseDev* cases, const Item* items, int s) {
   extern __shared__ __align__(16) int ibox_l[];
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
-  if (!C.active) return;
+  if (!chunk_step(C, s).active) return;
   const LatticeDev L = case_lattice(C);
   int4* box = C.boxes + 2 * it.i;
   switch (L.geometry) {
@@ -156,11 +215,11 @@ __global__ void __launch_bounds__(LANE_THREADS, 1) k_spread_bl(const CaseDev* ca
   }
 }
 
-__global__ void __launch_bounds__(LANE_THREADS, 1) k_interpolate_bl(const CaseDev* cases, const Item* items) {
+__global__ void __launch_bounds__(LANE_THREADS, 1) k_interpolate_bl(const CaseDev* cases, const Item* items, int s) {
   extern __shared__ __align__(16) unsigned char fbox_l[];
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
-  if (!C.active) return;
+  if (!chunk_step(C, s).active) return;
   const LatticeDev L = case_lattice(C);
   const int4* box = C.boxes + 2 * it.i;
   switch (L.geometry) {
@@ -178,18 +237,19 @@ __global__ void __launch_bounds__(LANE_THREADS, 1) k_interpolate_bl(const CaseDe
 // single-lattice collide (64-case stream: 17,610 -> 18,150 MLUPS against 6).
 template <int ODD, int GEOM>
 __global__ void __launch_bounds__(SERVE_COLLIDE_TX * SERVE_COLLIDE_TY, ODD ? 9 : 10)
-    k_collide_b(const CaseDev* cases, const Item* items, int n_items, int nxb) {
+    k_collide_b(const CaseDev* cases, const Item* items, int n_items, int nxb, int s) {
   const int ib = blockIdx.x / nxb, xb = blockIdx.x - ib * nxb;  // one-dimensional grid, x chunks fastest
   const int item = ib * blockDim.y + threadIdx.y;
   if (item >= n_items) return;
   const Item it = items[item];
   const CaseDev& C = cases[it.c];
   const int x = xb * blockDim.x + threadIdx.x;
-  if (!C.active || x >= C.L.nx) return;
-  const LatticeDev L = case_lattice(C);
+  const ChunkStep st = chunk_step(C, s);
+  if (!st.active || x >= C.L.nx) return;
+  const LatticeDev L = case_lattice(C, ODD == 1 && C.clustered != 0);
   const RowInfo R = C.rows[it.i];
   // served lattices are far below 2^32 / 19 cells (checked at submission)
-  if (C.dense) collide_cell<STORE_F32, ODD, GEOM, true, ODD == 1>(L, R, x);
+  if (st.last) collide_cell<STORE_F32, ODD, GEOM, true, ODD == 1>(L, R, x);
   else collide_cell<STORE_F32, ODD, GEOM, false, ODD == 1>(L, R, x);
 }
 
@@ -206,6 +266,8 @@ struct ibm_lbm_server {
     long long target = 0, steps = 0;
     size_t estimate = 0, held = 0;
     int unstable = 0;
+    int cluster_cap = 0;  // > 0: its bodies are coupled by clusters (cells of a block's box)
+    bool primed = false;  // then: the next step's forces are spread already
     // inputs
     ibm_lbm_config lat{};
     std::vector<double> rho0, u0, X;
@@ -232,7 +294,8 @@ struct ibm_lbm_server {
   std::vector<Alloc> mem;
   CaseDev* d_cases = nullptr;
   Item *d_rows = nullptr, *d_groups = nullptr, *d_rigid = nullptr, *d_membranes = nullptr;
-  size_t cap_rows = 0, cap_groups = 0, cap_rigid = 0, cap_membranes = 0;
+  Item *d_cl_rigid = nullptr, *d_cl_membranes = nullptr;  // bodies coupled by clusters
+  size_t cap_rows = 0, cap_groups = 0, cap_rigid = 0, cap_membranes = 0, cap_cl_rigid = 0, cap_cl_membranes = 0;
   int n_rows = 0, n_groups = 0, n_rigid = 0, n_membranes = 0, max_xblocks = 0;
   int geom_first[4] = {0, 0, 0, 0};  // rows of geometry g: [geom_first[g], geom_first[g + 1])
   size_t membrane_smem = 0;
@@ -359,6 +422,14 @@ int admit(ibm_lbm_server_t* s) {
       if (rc == IBM_LBM_E_NOMEM) break;  // retry after retirements
       return sfail(s, rc, "server: admission failed: " + why);
     }
+    // Clusters where they apply and the second force-density buffer is to be
+    // had (part of the estimate). The boxes' size is that of two blocks per SM
+    // whatever else is served, so that a case's path does not depend on it.
+    if (h->cluster_boxes && ensure_second_buffer(h)) {
+      const int words = std::max(h->n_rigids ? cluster_fixed_words(h->cluster_max, 0, 0) : 0,
+                                 h->n_membranes ? cluster_fixed_words(h->mesh.nv, h->mesh.nv, h->mesh.part_tris) : 0);
+      c->cluster_cap = cluster_box_cells(words, 1 << 20, h->n_sm);
+    }
     c->h = h;
     c->held = ibm_lbm_device_bytes(h);
     s->used += c->held;
@@ -371,9 +442,30 @@ int admit(ibm_lbm_server_t* s) {
   return IBM_LBM_OK;
 }
 
+// The collision of step `step` of the chunk for all cases, one launch per
+// geometry present.
+void launch_collide_b(ibm_lbm_server_t* s, bool odd, int step) {
+  for (int g = 0; g < 3; ++g) {
+    const int first = s->geom_first[g], n_items = s->geom_first[g + 1] - first;
+    if (n_items == 0) continue;
+    const dim3 block(SERVE_COLLIDE_TX, SERVE_COLLIDE_TY);
+    const int nxb = s->max_xblocks;
+    const dim3 grid((unsigned)nxb * (unsigned)((n_items + SERVE_COLLIDE_TY - 1) / SERVE_COLLIDE_TY));
+    const Item* items = s->d_rows + first;
+    switch (g * 2 + (odd ? 1 : 0)) {
+      case 0: k_collide_b<0, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
+      case 1: k_collide_b<1, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
+      case 2: k_collide_b<0, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
+      case 3: k_collide_b<1, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
+      case 4: k_collide_b<0, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
+      default: k_collide_b<1, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
+    }
+  }
+}
+
 int rebuild(ibm_lbm_server_t* s) {
   const int n = (int)s->running.size();
-  std::vector<Item> rows, groups, rigid, membranes;
+  std::vector<Item> rows, groups, rigid, membranes, cl_rigid, cl_membranes;
   std::vector<Item> rows_g[3];
   s->h_cases.assign(n, CaseDev{});
   s->max_xblocks = 0;
@@ -383,7 +475,13 @@ int rebuild(ibm_lbm_server_t* s) {
     CaseDev& C = s->h_cases[i];
     C.L = h->L;
     C.gbuf = h->gbuf;
+    C.gbuf2 = h->gbuf2;
     C.fbuf = h->fbuf;
+    C.fbuf2 = h->fbuf2;
+    C.cluster_boxes = h->cluster_boxes;
+    C.clustered = s->running[i]->cluster_cap > 0 ? 1 : 0;
+    C.cap = s->running[i]->cluster_cap;
+    C.primed = s->running[i]->primed ? 1 : 0;
     C.rows = h->rows;
     C.m = h->m;
     C.groups = h->groups;
@@ -396,14 +494,14 @@ int rebuild(ibm_lbm_server_t* s) {
     C.zero_F = h->need_zero_F ? 1 : 0;
     const int geom = std::min(std::max(h->L.geometry, 0), 2);
     for (int r = 0; r < h->n_rows; ++r) rows_g[geom].push_back({i, r});
-    if (h->m.M > 0)
+    if (h->m.M > 0 && !C.clustered)
       for (int g = 0; g < h->n_groups; ++g) groups.push_back({i, g});
     for (int b = 0; b < h->n_bodies; ++b) {
       const int kind = h->h_bodies[b].kind;
-      if (kind == IBM_LBM_BODY_RIGID || kind == IBM_LBM_BODY_RIGID_DIRECT) rigid.push_back({i, b});
-      else membranes.push_back({i, b});
+      const bool is_rigid = kind == IBM_LBM_BODY_RIGID || kind == IBM_LBM_BODY_RIGID_DIRECT;
+      (C.clustered ? (is_rigid ? cl_rigid : cl_membranes) : (is_rigid ? rigid : membranes)).push_back({i, b});
     }
-    if (h->n_membranes > 0)
+    if (h->n_membranes > 0 && !C.clustered)
       s->membrane_smem = std::max(s->membrane_smem, sizeof(float) * (size_t)h->mesh.work_floats);
     s->max_xblocks = std::max(s->max_xblocks, (h->L.nx + SERVE_COLLIDE_TX - 1) / SERVE_COLLIDE_TX);
   }
@@ -417,6 +515,8 @@ int rebuild(ibm_lbm_server_t* s) {
   if ((rc = ensure(s, &s->d_groups, &s->cap_groups, groups.size()))) return rc;
   if ((rc = ensure(s, &s->d_rigid, &s->cap_rigid, rigid.size()))) return rc;
   if ((rc = ensure(s, &s->d_membranes, &s->cap_membranes, membranes.size()))) return rc;
+  if ((rc = ensure(s, &s->d_cl_rigid, &s->cap_cl_rigid, cl_rigid.size()))) return rc;
+  if ((rc = ensure(s, &s->d_cl_membranes, &s->cap_cl_membranes, cl_membranes.size()))) return rc;
   s->n_rows = (int)rows.size();
   s->n_groups = (int)groups.size();
   s->n_rigid = (int)rigid.size();
@@ -432,6 +532,12 @@ int rebuild(ibm_lbm_server_t* s) {
   if (!membranes.empty())
     SCUDA(s, cudaMemcpyAsync(s->d_membranes, membranes.data(), sizeof(Item) * membranes.size(),
                              cudaMemcpyHostToDevice, s->stream));
+  if (!cl_rigid.empty())
+    SCUDA(s, cudaMemcpyAsync(s->d_cl_rigid, cl_rigid.data(), sizeof(Item) * cl_rigid.size(), cudaMemcpyHostToDevice,
+                             s->stream));
+  if (!cl_membranes.empty())
+    SCUDA(s, cudaMemcpyAsync(s->d_cl_membranes, cl_membranes.data(), sizeof(Item) * cl_membranes.size(),
+                             cudaMemcpyHostToDevice, s->stream));
   if (s->membrane_smem > 48 * 1024)
     SCUDA(s, cudaFuncSetAttribute(k_membranes_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s->membrane_smem));
   SCUDA(s, cudaStreamSynchronize(s->stream));
@@ -443,39 +549,34 @@ int rebuild(ibm_lbm_server_t* s) {
   cudaGraph_t g = nullptr;
   const bool lanes = s->n_groups < LANE_MAX_GROUPS;
   SCUDA(s, cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
+  const int n_cr = (int)cl_rigid.size(), n_cm = (int)cl_membranes.size();
+  auto couple = [&](int step) {
+    if (n_cr)
+      k_couple_cluster_b<0><<<n_cr * CLUSTER, CLUSTER_THREADS, CLUSTER_SHARE, s->stream>>>(s->d_cases, s->d_cl_rigid, step);
+    if (n_cm)
+      k_couple_cluster_b<1>
+          <<<n_cm * CLUSTER, CLUSTER_THREADS, CLUSTER_SHARE, s->stream>>>(s->d_cases, s->d_cl_membranes, step);
+  };
+  const bool separate = n_cr + n_cm == 0 || s->n_groups + s->n_rigid + s->n_membranes > 0;
+  if (n_cr + n_cm) k_chunk_begin<<<n, 256, 0, s->stream>>>(s->d_cases);
+  couple(-1);
   for (int step = 0; step < s->cfg.chunk_steps; ++step) {
-    k_book_begin<<<(n + 127) / 128, 128, 0, s->stream>>>(s->d_cases, n);
-    k_clear_flags<<<n, 256, 0, s->stream>>>(s->d_cases);
-    if (s->n_rigid) k_rigid_b<<<s->n_rigid, RIGID_THREADS, 0, s->stream>>>(s->d_cases, s->d_rigid);
+    if (separate) k_clear_flags<<<n, 256, 0, s->stream>>>(s->d_cases, step);
+    if (s->n_rigid) k_rigid_b<<<s->n_rigid, RIGID_THREADS, 0, s->stream>>>(s->d_cases, s->d_rigid, step);
     if (s->n_membranes)
-      k_membranes_b<<<s->n_membranes, MEMBRANE_THREADS, s->membrane_smem, s->stream>>>(s->d_cases, s->d_membranes);
+      k_membranes_b<<<s->n_membranes, MEMBRANE_THREADS, s->membrane_smem, s->stream>>>(s->d_cases, s->d_membranes, step);
     if (s->n_groups && lanes)
-      k_spread_bl<<<s->n_groups, LANE_THREADS, SPREAD_LANES_SMEM, s->stream>>>(s->d_cases, s->d_groups);
+      k_spread_bl<<<s->n_groups, LANE_THREADS, SPREAD_LANES_SMEM, s->stream>>>(s->d_cases, s->d_groups, step);
     else if (s->n_groups)
-      k_spread_b<<<s->n_groups, SERVE_XFER_THREADS, SPREAD_SMEM, s->stream>>>(s->d_cases, s->d_groups);
-    for (int g = 0; g < 3; ++g) {
-      const int first = s->geom_first[g], n_items = s->geom_first[g + 1] - first;
-      if (n_items == 0) continue;
-      const dim3 block(SERVE_COLLIDE_TX, SERVE_COLLIDE_TY);
-      const int nxb = s->max_xblocks;
-      const dim3 grid((unsigned)nxb * (unsigned)((n_items + SERVE_COLLIDE_TY - 1) / SERVE_COLLIDE_TY));
-      const Item* items = s->d_rows + first;
-      const bool odd = step & 1;
-      switch (g * 2 + (odd ? 1 : 0)) {
-        case 0: k_collide_b<0, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb); break;
-        case 1: k_collide_b<1, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb); break;
-        case 2: k_collide_b<0, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb); break;
-        case 3: k_collide_b<1, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb); break;
-        case 4: k_collide_b<0, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb); break;
-        default: k_collide_b<1, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb); break;
-      }
-    }
+      k_spread_b<<<s->n_groups, SERVE_XFER_THREADS, SPREAD_SMEM, s->stream>>>(s->d_cases, s->d_groups, step);
+    launch_collide_b(s, step & 1, step);
     if (s->n_groups && lanes)
-      k_interpolate_bl<<<s->n_groups, LANE_THREADS, INTERP_SMEM, s->stream>>>(s->d_cases, s->d_groups);
+      k_interpolate_bl<<<s->n_groups, LANE_THREADS, INTERP_SMEM, s->stream>>>(s->d_cases, s->d_groups, step);
     else if (s->n_groups)
-      k_interpolate_b<<<s->n_groups, SERVE_XFER_THREADS, INTERP_SMEM, s->stream>>>(s->d_cases, s->d_groups);
-    k_book_end<<<(n + 127) / 128, 128, 0, s->stream>>>(s->d_cases, n);
+      k_interpolate_b<<<s->n_groups, SERVE_XFER_THREADS, INTERP_SMEM, s->stream>>>(s->d_cases, s->d_groups, step);
+    couple(step);
   }
+  k_chunk_end<<<(n + 127) / 128, 128, 0, s->stream>>>(s->d_cases, n, s->cfg.chunk_steps);
   cudaError_t ce = cudaStreamEndCapture(s->stream, &g);
   if (ce != cudaSuccess) return sfail(s, IBM_LBM_E_CUDA, std::string("capture: ") + cudaGetErrorString(ce));
   ce = cudaGraphInstantiate(&s->graph, g, 0);
@@ -552,7 +653,11 @@ static int impl_ibm_lbm_server_create(const ibm_lbm_server_config* cfg, const ib
   if (cudaFuncSetAttribute(k_spread_b, cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(k_interpolate_b, cudaFuncAttributeMaxDynamicSharedMemorySize, INTERP_SMEM) != cudaSuccess ||
       cudaFuncSetAttribute(k_spread_bl, cudaFuncAttributeMaxDynamicSharedMemorySize, SPREAD_LANES_SMEM) != cudaSuccess ||
-      cudaFuncSetAttribute(k_interpolate_bl, cudaFuncAttributeMaxDynamicSharedMemorySize, INTERP_SMEM) != cudaSuccess) {
+      cudaFuncSetAttribute(k_interpolate_bl, cudaFuncAttributeMaxDynamicSharedMemorySize, INTERP_SMEM) != cudaSuccess ||
+      cudaFuncSetAttribute(k_couple_cluster_b<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, CLUSTER_SMEM_MAX) !=
+          cudaSuccess ||
+      cudaFuncSetAttribute(k_couple_cluster_b<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, CLUSTER_SMEM_MAX) !=
+          cudaSuccess) {
     cudaGetLastError();
     ibm_lbm_server_destroy(s);
     return IBM_LBM_E_CUDA;
@@ -631,6 +736,7 @@ static int impl_ibm_lbm_server_advance(ibm_lbm_server_t* s, int32_t* n_running, 
     for (int i = 0; i < n; ++i) {
       ibm_lbm_server::Case* c = s->running[i];
       c->steps = s->h_cases[i].done;
+      c->primed = c->cluster_cap > 0;
       if (c->steps >= c->target) {
         if ((rc = retire(s, c))) return rc;
         if (c->unstable) status = IBM_LBM_E_UNSTABLE;
