@@ -852,6 +852,7 @@ static int impl_ibm_lbm_create(const ibm_lbm_config* cfg, const ibm_lbm_allocato
   L.yc = 0.5f * (float)(cfg->ny - 1); L.zc = 0.5f * (float)(cfg->nz - 1);
   L.R2 = (float)(cfg->tube_radius * cfg->tube_radius);
   L.g0x = (float)cfg->body_force[0]; L.g0y = (float)cfg->body_force[1]; L.g0z = (float)cfg->body_force[2];
+  L.by_nx = fast_div((unsigned)cfg->nx);
   L.ntx = (cfg->nx + 31) >> TILE_X_SHIFT;
   L.nty = (cfg->ny + 3) >> TILE_Y_SHIFT;
   L.ntz = (cfg->nz + 3) >> TILE_Z_SHIFT;

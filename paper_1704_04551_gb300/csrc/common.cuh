@@ -46,6 +46,22 @@ enum Storage : int { STORE_F32 = 0, STORE_F16 = 1, STORE_BF16 = 2 };
 // Tiles used to mark where markers touch the lattice: 32 (x) x 4 x 4 cells.
 constexpr int TILE_X_SHIFT = 5, TILE_Y_SHIFT = 2, TILE_Z_SHIFT = 2;
 
+// Exact n / d for 32-bit n (Granlund & Montgomery, "Division by invariant
+// integers using multiplication", 1994): four instructions.
+struct FastDiv {
+  unsigned m, s1, s2;
+};
+inline FastDiv fast_div(unsigned d) {
+  int l = 0;
+  while ((1ull << l) < d) ++l;
+  const unsigned m = (unsigned)(((1ull << 32) * ((1ull << l) - d)) / d + 1);
+  return {m, l < 1 ? (unsigned)l : 1u, l < 1 ? 0u : (unsigned)l - 1u};
+}
+__device__ __forceinline__ unsigned divide(unsigned n, const FastDiv& d) {
+  const unsigned t = __umulhi(d.m, n);
+  return (t + ((n - t) >> d.s1)) >> d.s2;
+}
+
 struct LatticeDev {
   int nx, ny, nz;
   int N;                 // nx*ny*nz (< 2^31)
@@ -67,6 +83,7 @@ struct LatticeDev {
   float4* g;             // spread force density (gx, gy, gz, 0) [N]
   uint8_t* flags;        // [ntx*nty*ntz]: tile touched by a marker stencil this step
   int* status;           // device status word (0 = OK)
+  FastDiv by_nx;         // cell of the fluid rows -> (row, x)
 };
 
 // One lattice row (fixed y, z; all x) that holds fluid. Solidity depends on

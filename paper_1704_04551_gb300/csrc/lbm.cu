@@ -24,10 +24,11 @@
 namespace ibm {
 
 
-// Fused collide-stream-force kernel: one thread per fluid cell, a 2-D grid
-// over (x, fluid row). Row data (offsets of the neighbouring rows, which of
-// them are solid) come from the precomputed row table, so a thread does no
-// integer division and no geometry arithmetic.
+// Fused collide-stream-force kernel: one thread per fluid cell, the cells of
+// the fluid rows numbered through (row, x), so that the warps of a lattice
+// whose rows are no multiple of 32 or 128 cells long stay full and read whole
+// lines. Row data (offsets of the neighbouring rows, which of them are solid)
+// come from the precomputed row table.
 constexpr int COLLIDE_THREADS = 128;
 // Resident blocks per SM the register budget is sized for (more blocks,
 // more loads in flight; fewer registers): measured best at 256^3 with 10
@@ -40,20 +41,17 @@ constexpr int collide_min_blocks() {
   return (S == STORE_F32 && ODD) ? 9 : 10;
 }
 
-// The grid is one-dimensional (a row count above 65535 blocks does not fit
-// the y dimension): block b covers x chunk b % nxb of row block b / nxb,
-// x chunks of a row consecutive.
 template <int S, int ODD, int GEOM, bool DENSE, bool IDX32>
 __global__ void __launch_bounds__(COLLIDE_THREADS, (collide_min_blocks<S, ODD>())) k_collide(LatticeDev L, const RowInfo* __restrict__ rows,
-                                                                int n_rows, int nxb) {
-  const int rb = blockIdx.x / nxb, xb = blockIdx.x - rb * nxb;
-  const int r = rb * blockDim.y + threadIdx.y;
-  const int x = xb * blockDim.x + threadIdx.x;
-  if (r >= n_rows || x >= L.nx) return;
+                                                                unsigned n_cells) {
+  const unsigned t = blockIdx.x * (unsigned)COLLIDE_THREADS + threadIdx.x;
+  if (t >= n_cells) return;
+  const unsigned r = divide(t, L.by_nx);
+  const int x = (int)(t - r * (unsigned)L.nx);
   const RowInfo R = rows[r];
   // In the neighbour-addressed (odd) step, rows without solid neighbours
-  // (all but a ring of rows along walls) skip the bounce-back tests; a warp
-  // lies in one row, so the branch is uniform. (The even step reads and
+  // (all but a ring of rows along walls) skip the bounce-back tests; few warps
+  // lie in two rows of different kinds. (The even step reads and
   // writes its own cell only: a second copy there only cost registers.)
   if constexpr (ODD == 1 && GEOM != GEOM_PERIODIC) {
     if (R.smask == 0) {
@@ -229,10 +227,8 @@ inline unsigned blocks_for(int n) { return (unsigned)((n + 255) / 256); }
 
 template <int S, int GEOM>
 void launch_collide_g(const LatticeDev& L, const RowInfo* rows, int n_rows, bool odd, bool dense, cudaStream_t st) {
-  const int tx = L.nx >= COLLIDE_THREADS ? COLLIDE_THREADS : ((L.nx + 31) / 32) * 32;
-  const int ty = COLLIDE_THREADS / tx;
-  const int nxb = (L.nx + tx - 1) / tx;
-  const dim3 block(tx, ty), grid((unsigned)nxb * (unsigned)((n_rows + ty - 1) / ty));
+  const unsigned n_cells = (unsigned)n_rows * (unsigned)L.nx;  // <= N < 2^31
+  const unsigned block = COLLIDE_THREADS, grid = (n_cells + block - 1) / block;
   // 32-bit element offsets in the odd step while 19 N < 2^32 (a build with
   // IBM_FORCE_IDX64 defined always takes the 64-bit variant, so that the
   // parity tests reach it on small lattices)
@@ -242,14 +238,14 @@ void launch_collide_g(const LatticeDev& L, const RowInfo* rows, int n_rows, bool
   const bool idx32 = (unsigned long long)Q * (unsigned long long)L.N < (1ull << 32);
 #endif
   if (odd && idx32) {
-    if (dense) k_collide<S, 1, GEOM, true, true><<<grid, block, 0, st>>>(L, rows, n_rows, nxb);
-    else k_collide<S, 1, GEOM, false, true><<<grid, block, 0, st>>>(L, rows, n_rows, nxb);
+    if (dense) k_collide<S, 1, GEOM, true, true><<<grid, block, 0, st>>>(L, rows, n_cells);
+    else k_collide<S, 1, GEOM, false, true><<<grid, block, 0, st>>>(L, rows, n_cells);
   } else if (odd) {
-    if (dense) k_collide<S, 1, GEOM, true, false><<<grid, block, 0, st>>>(L, rows, n_rows, nxb);
-    else k_collide<S, 1, GEOM, false, false><<<grid, block, 0, st>>>(L, rows, n_rows, nxb);
+    if (dense) k_collide<S, 1, GEOM, true, false><<<grid, block, 0, st>>>(L, rows, n_cells);
+    else k_collide<S, 1, GEOM, false, false><<<grid, block, 0, st>>>(L, rows, n_cells);
   } else {
-    if (dense) k_collide<S, 0, GEOM, true, false><<<grid, block, 0, st>>>(L, rows, n_rows, nxb);
-    else k_collide<S, 0, GEOM, false, false><<<grid, block, 0, st>>>(L, rows, n_rows, nxb);
+    if (dense) k_collide<S, 0, GEOM, true, false><<<grid, block, 0, st>>>(L, rows, n_cells);
+    else k_collide<S, 0, GEOM, false, false><<<grid, block, 0, st>>>(L, rows, n_cells);
   }
 }
 template <int S>

@@ -5,7 +5,7 @@
 // and bodies in device memory, created through the server's allocator and on
 // the server's stream). The server advances all of them together: one
 // launch per stage for all cases, with per-case work items
-//   rows   (case, fluid row)      -> collide-stream-force
+//   cells  (case, run of cells)   -> collide-stream-force
 //   groups (case, marker group)   -> spreading, interpolation
 //   bodies (case, body)           -> marker forces
 // and a device-side case table holding each case's arrays and step counts,
@@ -56,6 +56,7 @@ struct CaseDev {
   int clustered, primed;
   int cap;           // cells of a cluster block's box
   const RowInfo* rows;
+  unsigned n_cells;  // of the fluid rows
   MarkersDev m;
   const MarkerGroup* groups;
   int4* boxes;
@@ -142,7 +143,7 @@ __global__ void k_chunk_end(CaseDev* cases, int n, int steps) {
 }
 
 constexpr int SERVE_XFER_THREADS = XFER_THREADS;
-constexpr int SERVE_COLLIDE_TX = 32, SERVE_COLLIDE_TY = 4;
+constexpr int SERVE_COLLIDE = 128;  // threads of a collide block
 
 // Start of a step of the cases without clusters: clear the tile flags this
 // step's spreading marks and, for markers outside every body, the forces.
@@ -229,25 +230,25 @@ __global__ void __launch_bounds__(LANE_THREADS, 1) k_interpolate_bl(const CaseDe
   }
 }
 
-// One warp per (case, row) segment of 32 cells. Cases are admitted only at
-// chunk boundaries and every chunk has an even number of steps, so all
-// running cases share the AA parity of a step and it is a template argument;
-// rows are grouped by geometry, one launch per geometry present.
+// One block per (case, run of SERVE_COLLIDE cells of its fluid rows), as in the
+// single-lattice collide. Cases are admitted only at chunk boundaries and every
+// chunk has an even number of steps, so all running cases share the AA parity
+// of a step and it is a template argument; blocks are grouped by geometry, one
+// launch per geometry present.
 // 10 resident blocks per SM for the even step, 9 for the odd one, as for the
 // single-lattice collide (64-case stream: 17,610 -> 18,150 MLUPS against 6).
 template <int ODD, int GEOM>
-__global__ void __launch_bounds__(SERVE_COLLIDE_TX * SERVE_COLLIDE_TY, ODD ? 9 : 10)
-    k_collide_b(const CaseDev* cases, const Item* items, int n_items, int nxb, int s) {
-  const int ib = blockIdx.x / nxb, xb = blockIdx.x - ib * nxb;  // one-dimensional grid, x chunks fastest
-  const int item = ib * blockDim.y + threadIdx.y;
-  if (item >= n_items) return;
-  const Item it = items[item];
+__global__ void __launch_bounds__(SERVE_COLLIDE, ODD ? 9 : 10)
+    k_collide_b(const CaseDev* cases, const Item* items, int s) {
+  const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
-  const int x = xb * blockDim.x + threadIdx.x;
+  const unsigned t = (unsigned)it.i * (unsigned)SERVE_COLLIDE + threadIdx.x;
   const ChunkStep st = chunk_step(C, s);
-  if (!st.active || x >= C.L.nx) return;
+  if (!st.active || t >= C.n_cells) return;
   const LatticeDev L = case_lattice(C, ODD == 1 && C.clustered != 0);
-  const RowInfo R = C.rows[it.i];
+  const unsigned r = divide(t, L.by_nx);
+  const int x = (int)(t - r * (unsigned)L.nx);
+  const RowInfo R = C.rows[r];
   // served lattices are far below 2^32 / 19 cells (checked at submission)
   if (st.last) collide_cell<STORE_F32, ODD, GEOM, true, ODD == 1>(L, R, x);
   else collide_cell<STORE_F32, ODD, GEOM, false, ODD == 1>(L, R, x);
@@ -296,7 +297,7 @@ struct ibm_lbm_server {
   Item *d_rows = nullptr, *d_groups = nullptr, *d_rigid = nullptr, *d_membranes = nullptr;
   Item *d_cl_rigid = nullptr, *d_cl_membranes = nullptr;  // bodies coupled by clusters
   size_t cap_rows = 0, cap_groups = 0, cap_rigid = 0, cap_membranes = 0, cap_cl_rigid = 0, cap_cl_membranes = 0;
-  int n_rows = 0, n_groups = 0, n_rigid = 0, n_membranes = 0, max_xblocks = 0;
+  int n_rows = 0, n_groups = 0, n_rigid = 0, n_membranes = 0;
   int geom_first[4] = {0, 0, 0, 0};  // rows of geometry g: [geom_first[g], geom_first[g + 1])
   size_t membrane_smem = 0;
   std::vector<CaseDev> h_cases;
@@ -448,17 +449,15 @@ void launch_collide_b(ibm_lbm_server_t* s, bool odd, int step) {
   for (int g = 0; g < 3; ++g) {
     const int first = s->geom_first[g], n_items = s->geom_first[g + 1] - first;
     if (n_items == 0) continue;
-    const dim3 block(SERVE_COLLIDE_TX, SERVE_COLLIDE_TY);
-    const int nxb = s->max_xblocks;
-    const dim3 grid((unsigned)nxb * (unsigned)((n_items + SERVE_COLLIDE_TY - 1) / SERVE_COLLIDE_TY));
+    const unsigned block = SERVE_COLLIDE, grid = (unsigned)n_items;
     const Item* items = s->d_rows + first;
     switch (g * 2 + (odd ? 1 : 0)) {
-      case 0: k_collide_b<0, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
-      case 1: k_collide_b<1, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
-      case 2: k_collide_b<0, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
-      case 3: k_collide_b<1, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
-      case 4: k_collide_b<0, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
-      default: k_collide_b<1, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, n_items, nxb, step); break;
+      case 0: k_collide_b<0, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
+      case 1: k_collide_b<1, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
+      case 2: k_collide_b<0, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
+      case 3: k_collide_b<1, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
+      case 4: k_collide_b<0, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
+      default: k_collide_b<1, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
     }
   }
 }
@@ -468,7 +467,6 @@ int rebuild(ibm_lbm_server_t* s) {
   std::vector<Item> rows, groups, rigid, membranes, cl_rigid, cl_membranes;
   std::vector<Item> rows_g[3];
   s->h_cases.assign(n, CaseDev{});
-  s->max_xblocks = 0;
   s->membrane_smem = 0;
   for (int i = 0; i < n; ++i) {
     ibm_lbm_t* h = s->running[i]->h;
@@ -483,6 +481,7 @@ int rebuild(ibm_lbm_server_t* s) {
     C.cap = s->running[i]->cluster_cap;
     C.primed = s->running[i]->primed ? 1 : 0;
     C.rows = h->rows;
+    C.n_cells = (unsigned)h->n_rows * (unsigned)h->L.nx;
     C.m = h->m;
     C.groups = h->groups;
     C.boxes = h->boxes;
@@ -493,7 +492,7 @@ int rebuild(ibm_lbm_server_t* s) {
     C.ntiles = h->L.ntx * h->L.nty * h->L.ntz;
     C.zero_F = h->need_zero_F ? 1 : 0;
     const int geom = std::min(std::max(h->L.geometry, 0), 2);
-    for (int r = 0; r < h->n_rows; ++r) rows_g[geom].push_back({i, r});
+    for (int b = 0; b < (int)((C.n_cells + SERVE_COLLIDE - 1) / SERVE_COLLIDE); ++b) rows_g[geom].push_back({i, b});
     if (h->m.M > 0 && !C.clustered)
       for (int g = 0; g < h->n_groups; ++g) groups.push_back({i, g});
     for (int b = 0; b < h->n_bodies; ++b) {
@@ -503,7 +502,6 @@ int rebuild(ibm_lbm_server_t* s) {
     }
     if (h->n_membranes > 0 && !C.clustered)
       s->membrane_smem = std::max(s->membrane_smem, sizeof(float) * (size_t)h->mesh.work_floats);
-    s->max_xblocks = std::max(s->max_xblocks, (h->L.nx + SERVE_COLLIDE_TX - 1) / SERVE_COLLIDE_TX);
   }
   for (int g = 0; g < 3; ++g) {
     s->geom_first[g] = (int)rows.size();
