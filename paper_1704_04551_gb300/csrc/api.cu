@@ -1162,8 +1162,8 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.off_ve = section(vel.data(), vel.size() * 2);
     D.off_vt_start = section(vts.data(), vts.size() * 2);
     D.off_vt = section(vtl.data(), vtl.size() * 2);
-    {
-      // parts of consecutive vertices (cluster_body.cuh)
+    if (h->n_membranes <= CLUSTER_MEMBRANES_MAX) {
+      // parts of consecutive vertices for the clusters (cluster_body.cuh)
       int table[CLUSTER][8] = {};
       D.part_tris = 0;
       const int per = cluster_per(mesh->n_vertices);

@@ -22,6 +22,8 @@
 // and forces, which part 3 still reads. Part 3 also stores its vertex
 // order in global memory beside the box, for part 1 of the next step,
 // which gathers at the same positions.
+#include <type_traits>
+
 #include "common.cuh"
 #include "forces_body.cuh"
 #include "internal.h"
@@ -108,7 +110,13 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
   // (the first step after separate kernels) each thread gathers for its own
   // markers. The velocities go to shared memory; after a barrier each thread
   // advects its own markers and writes their positions over the box.
-  if (in_box) velocity_box_async<GEOM>(L, lo, dims, vbox);
+  // (a box larger than shared memory comes in slabs of z layers)
+  const int depth = in_box ? slab_depth(dims) : 0;
+  auto load_slab = [&](int z0) {
+    velocity_box_async<GEOM>(L, make_int4(lo.x, lo.y, lo.z + z0, 0),
+                             make_int4(dims.x, dims.y, min(depth, dims.z - z0), 1), vbox);
+  };
+  if (in_box) load_slab(0);
   // bounds of the new stencils, largest force component, residue counts
   if (threadIdx.x < 3) {
     s_lo[threadIdx.x] = INT_MAX;
@@ -132,28 +140,37 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
   }
   if (in_box) velocity_box_wait();
   __syncthreads();
-  auto gather = [&](int j) {
-    Stencil st;
-    load_stencil(m, G.first + j, st);
-    const int ox = st.bx - lo.x, oy = st.by - lo.y, oz = st.bz - lo.z;
-    float3 u;
-    if (in_box && ox >= 0 && oy >= 0 && oz >= 0 && ox + 4 <= dims.x && oy + 4 <= dims.y && oz + 4 <= dims.z)
-      u = box_gather(vbox, dims, st, ox, oy, oz);
-    else  // no box, or the stencil outside it
-      u = gather_global<GEOM>(L, st, !in_box);
-    uS[j] = make_float4(u.x, u.y, u.z, 0.f);
-  };
-  if (ordered) {
-    for (int w = threadIdx.x >> 5; w < omost; w += nwarps)
-      if (w < ocnt) gather(oS[ost + w]);
-  } else {
+  for (int z0 = 0;; z0 += depth - 3) {
+    const int dz = min(depth, dims.z - z0);
+    auto gather = [&](int j) {
+      Stencil st;
+      load_stencil(m, G.first + j, st);
+      const int ox = st.bx - lo.x, oy = st.by - lo.y, oz = st.bz - lo.z - z0;
+      float3 u;
+      if (in_box && ox >= 0 && oy >= 0 && oz >= 0 && ox + 4 <= dims.x && oy + 4 <= dims.y && oz + 4 <= dz)
+        u = box_gather(vbox, dims, st, ox, oy, oz);
+      else if (in_box && dims.w == 2)  // in another slab (the box holds every stencil)
+        return;
+      else  // no box, or the stencil outside it
+        u = gather_global<GEOM>(L, st, !in_box);
+      uS[j] = make_float4(u.x, u.y, u.z, 0.f);
+    };
+    if (ordered) {
+      for (int w = threadIdx.x >> 5; w < omost; w += nwarps)
+        if (w < ocnt) gather(oS[ost + w]);
+    } else {
 #pragma unroll
-    for (int q = 0; q < COUPLE_PER_THREAD; ++q) {
-      const int j = threadIdx.x + q * COUPLE_THREADS;
-      if (j < nv) gather(j);
+      for (int q = 0; q < COUPLE_PER_THREAD; ++q) {
+        const int j = threadIdx.x + q * COUPLE_THREADS;
+        if (j < nv) gather(j);
+      }
     }
+    __syncthreads();  // the slab is done: the next one, or the positions, go over it
+    if (!in_box || z0 + dz >= dims.z) break;
+    load_slab(z0 + depth - 3);
+    velocity_box_wait();
+    __syncthreads();
   }
-  __syncthreads();  // the velocity box is done: the positions go over it
   const MembraneSmem S = MembraneSmem::at(smem, nv, nt);
   const int oa[3] = {o.x, o.y, o.z};
   {
@@ -200,8 +217,9 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
   // by residue now, while the membrane part runs
   const long long ex = (long long)s_hi[0] - s_lo[0] + 4, ey = (long long)s_hi[1] - s_lo[1] + 4,
                   ez = (long long)s_hi[2] - s_lo[2] + 4;
-  const bool fits = ex > 0 && ey > 0 && ez > 0 && ex * ey * ez <= BOX_CELLS;
-  const int4 dims2 = make_int4(fits ? (int)ex : 0, fits ? (int)ey : 0, fits ? (int)ez : 0, fits ? 1 : 0);
+  const int kind = box_kind(ex, ey, ez);
+  const bool fits = kind != 0;
+  const int4 dims2 = make_int4(fits ? (int)ex : 0, fits ? (int)ey : 0, fits ? (int)ez : 0, kind);
   int l2[COUPLE_PER_THREAD];
 #pragma unroll
   for (int q = 0; q < COUPLE_PER_THREAD; ++q) {
@@ -268,7 +286,7 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
   // fixed-point box after the positions and forces (still read below)
   int* ibox = reinterpret_cast<int*>(S.sQ + 3 * nv);
   unsigned short* order = reinterpret_cast<unsigned short*>(ibox + 3 * BOX_CELLS);
-  const int vol = dims2.x * dims2.y * dims2.z;
+  const int depth2 = slab_depth(dims2), layer = dims2.x * dims2.y, vol = layer * depth2;
   const float Sc = fminf(33554432.0f, 8589934592.0f / (float)nv) / fmax;  // as in spread_group
   for (int i = threadIdx.x; i < 3 * vol; i += blockDim.x) ibox[i] = 0;
 #pragma unroll
@@ -286,20 +304,36 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
     }
     if (threadIdx.x == 0) wmeta[64] = R.most;
   }
-  {
-    const int n = R.cnt[lane], st = R.start[lane];
+  const int n = R.cnt[lane], st = R.start[lane];
+  auto scatter = [&](auto clipped, int z0, int dz) {
     for (int w = threadIdx.x >> 5; w < R.most; w += nwarps) {
       if (w >= n) continue;
       const int v = order[st + w];
       int c[3];
       float f[3];
       smem_cell(S, nv, v, o, c, f);
-      const int li0 = (c[0] - 1 - lo2.x) + dims2.x * ((c[1] - 1 - lo2.y) + dims2.y * (c[2] - 1 - lo2.z));
-      scatter_marker(ibox, vol, dims2, li0, f[0], f[1], f[2], sF(v) * Sc, sF(nv + v) * Sc, sF(2 * nv + v) * Sc);
+      const int oz = c[2] - 1 - lo2.z - z0;
+      if (clipped.value && (oz <= -4 || oz >= dz)) continue;
+      const int li0 = (c[0] - 1 - lo2.x) + dims2.x * ((c[1] - 1 - lo2.y) + dims2.y * oz);
+      scatter_marker<clipped.value>(ibox, vol, dims2, li0, f[0], f[1], f[2], sF(v) * Sc, sF(nv + v) * Sc,
+                                    sF(2 * nv + v) * Sc, -oz, dz - oz);
     }
+  };
+  if (kind == 1) {
+    scatter(std::false_type{}, 0, dims2.z);
+    __syncthreads();
+    flush_box<GEOM>(Ln, lo2, dims2, ibox, 1.0f / Sc);
+    return;
   }
-  __syncthreads();
-  flush_box<GEOM>(Ln, lo2, dims2, ibox, 1.0f / Sc);
+  for (int z0 = 0; z0 < dims2.z; z0 += depth2) {  // (the first slab is zero already)
+    const int dz = min(depth2, dims2.z - z0);
+    scatter(std::true_type{}, z0, dz);
+    __syncthreads();
+    flush_box<GEOM>(Ln, make_int4(lo2.x, lo2.y, lo2.z + z0, 0), make_int4(dims2.x, dims2.y, dz, 1), ibox, 1.0f / Sc, vol);
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * vol; i += blockDim.x) ibox[i] = 0;
+    __syncthreads();
+  }
 }
 
 template <int GEOM>

@@ -70,6 +70,25 @@ constexpr int INTERP_SMEM = BOX_CELLS * (int)sizeof(float4);
 // fixed-point sums [3][vol] (four lanes per marker: no marker records)
 constexpr int SPREAD_LANES_SMEM = 3 * BOX_CELLS * (int)sizeof(int);
 
+// Boxes. A group's stencil box of at most BOX_CELLS cells is held in shared
+// memory whole; a larger one of at most BOX_SLABBED cells whose z layers hold
+// at most BOX_CELLS / 4 cells in slabs of z layers, one after the other: the
+// gather's slabs overlap by three layers, so that each 4^3 stencil lies in
+// one; the scatter's do not, and a marker adds the layers that a slab holds.
+// (A tumbling red cell's box reaches ~6800 cells. Per-marker global atomics and
+// gathers, the path of every larger box, made one such body set the time of
+// the fused kernel: 207 instead of 47 us per 64^3 step.) box_kind: 1 whole,
+// 2 in slabs, 0 neither.
+constexpr int BOX_SLABBED = 8 * BOX_CELLS;
+__device__ __forceinline__ int box_kind(long long ex, long long ey, long long ez) {
+  if (ex <= 0 || ey <= 0 || ez <= 0 || ex > BOX_SLABBED || ey > BOX_SLABBED || ez > BOX_SLABBED) return 0;
+  const long long layer = ex * ey;
+  if (layer * ez <= BOX_CELLS) return 1;
+  return layer * 4 <= BOX_CELLS && layer * ez <= BOX_SLABBED ? 2 : 0;
+}
+// z layers a slab of the box holds (all of them for a box held whole)
+__device__ __forceinline__ int slab_depth(int4 dims) { return min(dims.z, BOX_CELLS / (dims.x * dims.y)); }
+
 // The four delta weights of one axis for a marker at fractional offset f.
 __device__ __forceinline__ void axis_weights(float f, float w[4]) {
   float s, c;
@@ -251,8 +270,8 @@ __device__ inline void group_box(const MarkersDev& m, const MarkerGroup& G, int4
   const long long ex = (long long)s_hi[0] - s_lo[0] + 4, ey = (long long)s_hi[1] - s_lo[1] + 4,
                   ez = (long long)s_hi[2] - s_lo[2] + 4;
   lo = make_int4(s_lo[0] - 1, s_lo[1] - 1, s_lo[2] - 1, 0);
-  const bool fits = ex > 0 && ey > 0 && ez > 0 && ex * ey * ez <= BOX_CELLS;
-  dims = make_int4(fits ? (int)ex : 0, fits ? (int)ey : 0, fits ? (int)ez : 0, fits ? 1 : 0);
+  const int kind = box_kind(ex, ey, ez);
+  dims = make_int4(kind ? (int)ex : 0, kind ? (int)ey : 0, kind ? (int)ez : 0, kind);
   fmax = __uint_as_float(s_fmax);
 }
 
@@ -369,8 +388,11 @@ __device__ __noinline__ void scatter_global(const LatticeDev& L, const Stencil& 
 // Adds one marker's force, already multiplied by the fixed-point scale, to
 // the box: li0 is the box index of its first stencil node, f its fractional
 // offsets (the weights), vol the box's cells per component.
+// With CLIPPED, only its z layers c in [c0, c1) (li0 counts from the slab's
+// first layer and may be negative).
+template <bool CLIPPED = false>
 __device__ __forceinline__ void scatter_marker(int* ibox, int vol, int4 dims, int li0, float fx, float fy, float fz,
-                                               float Fx, float Fy, float Fz) {
+                                               float Fx, float Fy, float Fz, int c0 = 0, int c1 = 4) {
   float wx[4], wy[4], wz[4];
   axis_weights(fx, wx);
   axis_weights(fy, wy);
@@ -383,7 +405,8 @@ __device__ __forceinline__ void scatter_marker(int* ibox, int vol, int4 dims, in
     az_[a] = Fz * wx[a];
   }
 #pragma unroll
-  for (int c = 0; c < 4; ++c)
+  for (int c = 0; c < 4; ++c) {
+    if (CLIPPED && (c < c0 || c >= c1)) continue;
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const float wyz = wy[b] * wz[c];
@@ -395,13 +418,15 @@ __device__ __forceinline__ void scatter_marker(int* ibox, int vol, int4 dims, in
         atomicAdd(p + 2 * vol + a, fixed_mul(az_[a], wyz));
       }
     }
+  }
 }
 
 // Adds the nonzero cells of a fixed-point box (1/inv units) to L.g, row by
 // row (one float4 atomic per cell).
 template <int GEOM>
-__device__ __forceinline__ void flush_box(const LatticeDev& L, int4 lo, int4 dims, const int* ibox, float inv) {
-  const int vol = dims.x * dims.y * dims.z;
+__device__ __forceinline__ void flush_box(const LatticeDev& L, int4 lo, int4 dims, const int* ibox, float inv,
+                                          int stride = 0) {
+  const int vol = stride ? stride : dims.x * dims.y * dims.z;  // cells per component
   const int nrows = dims.y * dims.z;
   const int nwarps = blockDim.x >> 5;
   const RowSweep sw = row_sweep(dims.x);
@@ -513,7 +538,7 @@ __device__ __forceinline__ void spread_group(const LatticeDev& L, const MarkersD
   int* ibox = reinterpret_cast<int*>(smem);                                   // [3][vol]
   float4* rec = reinterpret_cast<float4*>(smem + 3 * BOX_CELLS * sizeof(int));  // [2][XFER_GROUP_MAX]
   Residues& R = *reinterpret_cast<Residues*>(rec + 2 * XFER_GROUP_MAX);
-  const int vol = dims.x * dims.y * dims.z;
+  const int depth = slab_depth(dims), layer = dims.x * dims.y, vol = layer * depth;
   const size_t M = (size_t)m.M;
   // Fixed-point scale: a contribution is at most fmax / 8 (delta <= 1/8) and
   // a cell's sum at most count * fmax / 8; S keeps contributions below 2^22
@@ -543,17 +568,33 @@ __device__ __forceinline__ void spread_group(const LatticeDev& L, const MarkersD
     rec[XFER_GROUP_MAX + pos] = make_float4(F.x * S, F.y * S, F.z * S, 0.f);
   }
   __syncthreads();
-  {
-    const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-    const int n = R.cnt[lane], st = R.start[lane];
+  const int lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  const int n = R.cnt[lane], st = R.start[lane];
+  if (dims.w == 1) {
     for (int w = threadIdx.x >> 5; w < R.most; w += nwarps) {
       if (w >= n) continue;
       const float4 A = rec[st + w], B = rec[XFER_GROUP_MAX + st + w];
       scatter_marker(ibox, vol, dims, __float_as_int(A.x), A.y, A.z, A.w, B.x, B.y, B.z);
     }
+    __syncthreads();
+    flush_box<GEOM>(L, lo, dims, ibox, 1.0f / S);
+    return;
   }
-  __syncthreads();
-  flush_box<GEOM>(L, lo, dims, ibox, 1.0f / S);
+  for (int z0 = 0; z0 < dims.z; z0 += depth) {  // (the first slab is zero already)
+    const int dz = min(depth, dims.z - z0);
+    for (int w = threadIdx.x >> 5; w < R.most; w += nwarps) {
+      if (w >= n) continue;
+      const float4 A = rec[st + w], B = rec[XFER_GROUP_MAX + st + w];
+      const int li = __float_as_int(A.x), oz = li / layer - z0;
+      if (oz > -4 && oz < dz)
+        scatter_marker<true>(ibox, vol, dims, li - z0 * layer, A.y, A.z, A.w, B.x, B.y, B.z, -oz, dz - oz);
+    }
+    __syncthreads();
+    flush_box<GEOM>(L, make_int4(lo.x, lo.y, lo.z + z0, 0), make_int4(dims.x, dims.y, dz, 1), ibox, 1.0f / S, vol);
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * vol; i += blockDim.x) ibox[i] = 0;
+    __syncthreads();
+  }
 }
 
 // Velocity at one marker gathered from the lattice (groups whose box does
@@ -604,35 +645,48 @@ __device__ __forceinline__ void interpolate_group(const LatticeDev& L, const Mar
   const bool moves = !(G.flags & GROUP_FIXED);
   const bool in_box = dims.w != 0;
   float4* vbox = reinterpret_cast<float4*>(smem);  // [vol]
-  if (in_box) {
-    velocity_box_async<GEOM>(L, lo, dims, vbox);
-    velocity_box_wait();
-    __syncthreads();
-  }
-  for (int j = threadIdx.x; j < G.count; j += blockDim.x) {
-    const int k = G.first + j;
-    Stencil st;
-    load_stencil(m, k, st);
-    double Xo[3] = {0.0, 0.0, 0.0};
-    if (moves)
+  const int depth = in_box ? slab_depth(dims) : 0;
+  unsigned done = 0u;  // this thread's markers of earlier slabs (moved already)
+  for (int z0 = 0;; z0 += depth - 3) {
+    const int dz = min(depth, dims.z - z0);
+    const bool last = !in_box || z0 + dz >= dims.z;
+    if (in_box) {
+      velocity_box_async<GEOM>(L, make_int4(lo.x, lo.y, lo.z + z0, 0), make_int4(dims.x, dims.y, dz, 1), vbox);
+      velocity_box_wait();
+      __syncthreads();
+    }
+    int q = 0;
+    for (int j = threadIdx.x; j < G.count; j += blockDim.x, ++q) {
+      if ((done >> q) & 1u) continue;
+      const int k = G.first + j;
+      Stencil st;
+      load_stencil(m, k, st);
+      const int ox = st.bx - lo.x, oy = st.by - lo.y, oz = st.bz - lo.z - z0;
+      const bool inside = in_box && ox >= 0 && oy >= 0 && oz >= 0 && ox + 4 <= dims.x && oy + 4 <= dims.y && oz + 4 <= dz;
+      if (!inside && !last) continue;
+      done |= 1u << q;
+      double Xo[3] = {0.0, 0.0, 0.0};
+      if (moves)
 #pragma unroll
-      for (int a = 0; a < 3; ++a) Xo[a] = m.X[a * M + k];
-    const int ox = st.bx - lo.x, oy = st.by - lo.y, oz = st.bz - lo.z;
-    float3 u;
-    if (in_box && ox >= 0 && oy >= 0 && oz >= 0 && ox + 4 <= dims.x && oy + 4 <= dims.y && oz + 4 <= dims.z)
-      u = box_gather(vbox, dims, st, ox, oy, oz);
-    else  // no box (every visited cell is cleared), or the stencil outside it
-      u = gather_global<GEOM>(L, st, !in_box);
-    m.U[k] = make_float4(u.x, u.y, u.z, 0.f);
-    if (moves) {
-      const float ua[3] = {u.x, u.y, u.z};
+        for (int a = 0; a < 3; ++a) Xo[a] = m.X[a * M + k];
+      float3 u;
+      if (inside)
+        u = box_gather(vbox, dims, st, ox, oy, oz);
+      else  // no box (every visited cell is cleared), or the stencil outside it
+        u = gather_global<GEOM>(L, st, !in_box);
+      m.U[k] = make_float4(u.x, u.y, u.z, 0.f);
+      if (moves) {
+        const float ua[3] = {u.x, u.y, u.z};
 #pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        const double Xn = Xo[a] + (double)ua[a];
-        m.X[a * M + k] = Xn;
-        cache_coord(m, a * M + k, Xn);
+        for (int a = 0; a < 3; ++a) {
+          const double Xn = Xo[a] + (double)ua[a];
+          m.X[a * M + k] = Xn;
+          cache_coord(m, a * M + k, Xn);
+        }
       }
     }
+    if (last) return;
+    __syncthreads();  // the slab is done
   }
 }
 
@@ -667,7 +721,7 @@ __device__ __forceinline__ void spread_group_lanes(const LatticeDev& L, const Ma
   }
   const bool any_force = fmax > 0.f;
   const bool in_smem = dims.w != 0;
-  const int vol = dims.x * dims.y * dims.z;
+  const int depth = in_smem ? slab_depth(dims) : 0, vol = dims.x * dims.y * depth;
   const float S = any_force ? fminf(33554432.0f, 8589934592.0f / (float)G.count) / fmax : 0.f;  // as spread_group
   if (in_smem) {
     mark_box_tiles<GEOM>(L, lo, dims);
@@ -678,51 +732,61 @@ __device__ __forceinline__ void spread_group_lanes(const LatticeDev& L, const Ma
   const int a = threadIdx.x & 3;
   const int per_pass = blockDim.x >> 2;
   const int wfirst = (int)(threadIdx.x & ~31u) >> 2;  // first marker of this warp within a pass
-  // whole warps iterate together (shuffles in mark_tiles)
-  for (int j0 = 0; j0 + wfirst < G.count; j0 += per_pass) {
-    const int j = j0 + (int)(threadIdx.x >> 2);
-    const bool active = j < G.count;
-    const int k = G.first + (active ? j : 0);
-    RawStencil r;
-    load_raw(m, k, r);
-    const int bx = r.c[0] - 1, by = r.c[1] - 1, bz = r.c[2] - 1;
-    // the four lanes of a marker share its tiles: only the first stores them
-    if (!in_smem) mark_tiles<GEOM>(L, bx, by, bz, active);
-    if (!active || !any_force) continue;
-    const float wxa = axis_weight(r.f[0], a);
-    float wy[4], wz[4];
-    axis_weights(r.f[1], wy);
-    axis_weights(r.f[2], wz);
-    const float4 F = m.F[k];
-    if (in_smem) {
-      const float ax_ = F.x * S * wxa, ay_ = F.y * S * wxa, az_ = F.z * S * wxa;
-      int* p0 = ibox + (bx - lo.x + a) + dims.x * ((by - lo.y) + dims.y * (bz - lo.z));
+  for (int z0 = 0;; z0 += depth) {  // slabs of the box (one when it is held whole)
+    const int dz = min(depth, dims.z - z0);
+    // whole warps iterate together (shuffles in mark_tiles)
+    for (int j0 = 0; j0 + wfirst < G.count; j0 += per_pass) {
+      const int j = j0 + (int)(threadIdx.x >> 2);
+      const bool active = j < G.count;
+      const int k = G.first + (active ? j : 0);
+      RawStencil r;
+      load_raw(m, k, r);
+      const int bx = r.c[0] - 1, by = r.c[1] - 1, bz = r.c[2] - 1;
+      // the four lanes of a marker share its tiles: only the first stores them
+      if (!in_smem) mark_tiles<GEOM>(L, bx, by, bz, active);
+      const int oz = bz - lo.z - z0;
+      if (!active || !any_force || (in_smem && (oz <= -4 || oz >= dz))) continue;
+      const float wxa = axis_weight(r.f[0], a);
+      float wy[4], wz[4];
+      axis_weights(r.f[1], wy);
+      axis_weights(r.f[2], wz);
+      const float4 F = m.F[k];
+      if (in_smem) {
+        const float ax_ = F.x * S * wxa, ay_ = F.y * S * wxa, az_ = F.z * S * wxa;
+        int* p0 = ibox + (bx - lo.x + a) + dims.x * ((by - lo.y) + dims.y * oz);
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < 4; ++c) {
+          if (oz + c < 0 || oz + c >= dz) continue;  // (a layer of another slab)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const float wyz = wy[b] * wz[c];
-          int* p = p0 + dims.x * (b + dims.y * c);
-          atomicAdd(p, fixed_mul(ax_, wyz));
-          atomicAdd(p + vol, fixed_mul(ay_, wyz));
-          atomicAdd(p + 2 * vol, fixed_mul(az_, wyz));
+          for (int b = 0; b < 4; ++b) {
+            const float wyz = wy[b] * wz[c];
+            int* p = p0 + dims.x * (b + dims.y * c);
+            atomicAdd(p, fixed_mul(ax_, wyz));
+            atomicAdd(p + vol, fixed_mul(ay_, wyz));
+            atomicAdd(p + 2 * vol, fixed_mul(az_, wyz));
+          }
         }
-    } else {
-      const int x = wrapi(bx + a, L.nx);
+      } else {
+        const int x = wrapi(bx + a, L.nx);
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          int y = by + b, z = bz + c;
-          if (!fluid_row<GEOM>(L, y, z)) continue;
-          const float w = wxa * (wy[b] * wz[c]);
-          atomicAdd(L.g + (size_t)L.nx * (y + L.ny * z) + x, make_float4(F.x * w, F.y * w, F.z * w, 0.f));
-        }
+          for (int b = 0; b < 4; ++b) {
+            int y = by + b, z = bz + c;
+            if (!fluid_row<GEOM>(L, y, z)) continue;
+            const float w = wxa * (wy[b] * wz[c]);
+            atomicAdd(L.g + (size_t)L.nx * (y + L.ny * z) + x, make_float4(F.x * w, F.y * w, F.z * w, 0.f));
+          }
+      }
     }
+    if (!in_smem) return;
+    __syncthreads();
+    flush_box<GEOM>(L, make_int4(lo.x, lo.y, lo.z + z0, 0), make_int4(dims.x, dims.y, dz, 1), ibox, 1.0f / S, vol);
+    if (z0 + dz >= dims.z) return;
+    __syncthreads();
+    for (int i = threadIdx.x; i < 3 * vol; i += blockDim.x) ibox[i] = 0;
+    __syncthreads();
   }
-  if (!in_smem) return;
-  __syncthreads();
-  flush_box<GEOM>(L, lo, dims, ibox, 1.0f / S);
 }
 
 // Interpolation and advection of one marker group with four lanes per
@@ -743,79 +807,90 @@ __device__ __forceinline__ void interpolate_group_lanes(const LatticeDev& L, con
   const int per_pass = blockDim.x >> 2;
   const int slot = threadIdx.x >> 2;
   const int wfirst = (int)(threadIdx.x & ~31u) >> 2;
-  if (in_box) velocity_box_async<GEOM>(L, lo, dims, vbox);
-  RawStencil nxt;
-  if (wfirst < G.count) load_raw(m, G.first + (slot < G.count ? slot : 0), nxt);
-  if (in_box) {
-    velocity_box_wait();
-    __syncthreads();
-  }
-  // whole warps iterate together (shuffles); a warp stops at the first pass
-  // that lies entirely past the group's end
-  for (int j0 = 0; j0 + wfirst < G.count; j0 += per_pass) {
-    const int j = j0 + slot;
-    const bool active = j < G.count;
-    const int k = G.first + (active ? j : 0);
-    const size_t off = (size_t)a * M + k;
-    double Xo = 0.0;
-    if (active && moves && a < 3) Xo = m.X[off];
-    const RawStencil cur = nxt;
-    if (j0 + per_pass + wfirst < G.count) {
-      const int jn = j + per_pass;
-      load_raw(m, G.first + (jn < G.count ? jn : 0), nxt);
+  const int depth = in_box ? slab_depth(dims) : 0;
+  unsigned done = 0u;  // passes whose marker was in an earlier slab (moved already)
+  for (int z0 = 0;; z0 += depth - 3) {
+    const int dz = min(depth, dims.z - z0);
+    const bool last = !in_box || z0 + dz >= dims.z;
+    if (in_box) velocity_box_async<GEOM>(L, make_int4(lo.x, lo.y, lo.z + z0, 0), make_int4(dims.x, dims.y, dz, 1), vbox);
+    RawStencil nxt;
+    if (wfirst < G.count) load_raw(m, G.first + (slot < G.count ? slot : 0), nxt);
+    if (in_box) {
+      velocity_box_wait();
+      __syncthreads();
     }
-    const int bx = cur.c[0] - 1, by = cur.c[1] - 1, bz = cur.c[2] - 1;
-    const float wxa = axis_weight(cur.f[0], a);
-    float wy[4], wz[4];
-    axis_weights(cur.f[1], wy);
-    axis_weights(cur.f[2], wz);
-    const int ox = bx - lo.x, oy = by - lo.y, oz = bz - lo.z;
-    float ux = 0.f, uy = 0.f, uz = 0.f;
-    if (in_box && ox >= 0 && oy >= 0 && oz >= 0 && ox + 4 <= dims.x && oy + 4 <= dims.y && oz + 4 <= dims.z) {
-      const float4* p0 = vbox + (ox + a) + dims.x * (oy + dims.y * oz);
+    // whole warps iterate together (shuffles); a warp stops at the first pass
+    // that lies entirely past the group's end
+    int pass = 0;
+    for (int j0 = 0; j0 + wfirst < G.count; j0 += per_pass, ++pass) {
+      const int j = j0 + slot;
+      const int k = G.first + (j < G.count ? j : 0);
+      const RawStencil cur = nxt;
+      if (j0 + per_pass + wfirst < G.count) {
+        const int jn = j + per_pass;
+        load_raw(m, G.first + (jn < G.count ? jn : 0), nxt);
+      }
+      const int bx = cur.c[0] - 1, by = cur.c[1] - 1, bz = cur.c[2] - 1;
+      const int ox = bx - lo.x, oy = by - lo.y, oz = bz - lo.z - z0;
+      const bool inside = in_box && ox >= 0 && oy >= 0 && oz >= 0 && ox + 4 <= dims.x && oy + 4 <= dims.y && oz + 4 <= dz;
+      const bool active = j < G.count && !((done >> pass) & 1u) && (inside || last);
+      if (active) done |= 1u << pass;
+      const size_t off = (size_t)a * M + k;
+      double Xo = 0.0;
+      if (active && moves && a < 3) Xo = m.X[off];
+      const float wxa = axis_weight(cur.f[0], a);
+      float wy[4], wz[4];
+      axis_weights(cur.f[1], wy);
+      axis_weights(cur.f[2], wz);
+      float ux = 0.f, uy = 0.f, uz = 0.f;
+      if (inside) {
+        const float4* p0 = vbox + (ox + a) + dims.x * (oy + dims.y * oz);
 #pragma unroll
-      for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          const float4 v = p0[dims.x * (b + dims.y * c)];
-          const float wyz = wy[b] * wz[c];
-          ux = fmaf(wyz, v.x, ux);
-          uy = fmaf(wyz, v.y, uy);
-          uz = fmaf(wyz, v.z, uz);
-        }
-    } else {  // no box (every visited cell is cleared), or the stencil outside it
-      const int x = wrapi(bx + a, L.nx);
+          for (int b = 0; b < 4; ++b) {
+            const float4 v = p0[dims.x * (b + dims.y * c)];
+            const float wyz = wy[b] * wz[c];
+            ux = fmaf(wyz, v.x, ux);
+            uy = fmaf(wyz, v.y, uy);
+            uz = fmaf(wyz, v.z, uz);
+          }
+      } else if (active) {  // no box (every visited cell is cleared), or the stencil outside it
+        const int x = wrapi(bx + a, L.nx);
 #pragma unroll 1
-      for (int c = 0; c < 4; ++c)
+        for (int c = 0; c < 4; ++c)
 #pragma unroll
-        for (int b = 0; b < 4; ++b) {
-          int y = by + b, z = bz + c;
-          if (!fluid_row<GEOM>(L, y, z)) continue;
-          const size_t gi = (size_t)L.nx * (y + L.ny * z) + x;
-          const float4 v = L.uw[gi];
-          if (!in_box) L.g[gi] = make_float4(0.f, 0.f, 0.f, 0.f);
-          const float wyz = wy[b] * wz[c];
-          ux = fmaf(wyz, v.x, ux);
-          uy = fmaf(wyz, v.y, uy);
-          uz = fmaf(wyz, v.z, uz);
-        }
-    }
-    ux *= wxa;
-    uy *= wxa;
-    uz *= wxa;
+          for (int b = 0; b < 4; ++b) {
+            int y = by + b, z = bz + c;
+            if (!fluid_row<GEOM>(L, y, z)) continue;
+            const size_t gi = (size_t)L.nx * (y + L.ny * z) + x;
+            const float4 v = L.uw[gi];
+            if (!in_box) L.g[gi] = make_float4(0.f, 0.f, 0.f, 0.f);
+            const float wyz = wy[b] * wz[c];
+            ux = fmaf(wyz, v.x, ux);
+            uy = fmaf(wyz, v.y, uy);
+            uz = fmaf(wyz, v.z, uz);
+          }
+      }
+      ux *= wxa;
+      uy *= wxa;
+      uz *= wxa;
 #pragma unroll
-    for (int o = 1; o < 4; o <<= 1) {
-      ux += __shfl_xor_sync(0xffffffffu, ux, o);
-      uy += __shfl_xor_sync(0xffffffffu, uy, o);
-      uz += __shfl_xor_sync(0xffffffffu, uz, o);
+      for (int o = 1; o < 4; o <<= 1) {
+        ux += __shfl_xor_sync(0xffffffffu, ux, o);
+        uy += __shfl_xor_sync(0xffffffffu, uy, o);
+        uz += __shfl_xor_sync(0xffffffffu, uz, o);
+      }
+      if (!active) continue;
+      if (a == 0) m.U[k] = make_float4(ux, uy, uz, 0.f);
+      if (a < 3 && moves) {
+        const double Xn = Xo + (double)(a == 0 ? ux : (a == 1 ? uy : uz));
+        m.X[off] = Xn;
+        cache_coord(m, off, Xn);
+      }
     }
-    if (!active) continue;
-    if (a == 0) m.U[k] = make_float4(ux, uy, uz, 0.f);
-    if (a < 3 && moves) {
-      const double Xn = Xo + (double)(a == 0 ? ux : (a == 1 ? uy : uz));
-      m.X[off] = Xn;
-      cache_coord(m, off, Xn);
-    }
+    if (last) return;
+    __syncthreads();  // the slab is done
   }
 }
 
