@@ -167,6 +167,10 @@ enum Path { SEPARATE, FUSED, CLUSTERED };
 // (couple.cu) does less work in all, but its latency decides while the
 // bodies do not fill the chip.
 constexpr int CLUSTER_MEMBRANES_MAX = 38;
+// The solid-only dynamics of a launch, and up to how many membranes it takes
+// clusters.
+constexpr int64_t SOLID_CHUNK = 512;
+constexpr int SOLID_MEMBRANES_MAX = 128;
 
 Path path_of(const ibm_lbm_t* h) {
   if (h->m.M == 0 || h->morse_rc > 0.0) return SEPARATE;
@@ -1162,7 +1166,7 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.off_ve = section(vel.data(), vel.size() * 2);
     D.off_vt_start = section(vts.data(), vts.size() * 2);
     D.off_vt = section(vtl.data(), vtl.size() * 2);
-    if (h->n_membranes <= CLUSTER_MEMBRANES_MAX) {
+    if (h->n_membranes <= std::max(CLUSTER_MEMBRANES_MAX, SOLID_MEMBRANES_MAX)) {
       // parts of consecutive vertices for the clusters (cluster_body.cuh)
       int table[CLUSTER][8] = {};
       D.part_tris = 0;
@@ -1354,11 +1358,23 @@ static int impl_ibm_lbm_solid_steps(ibm_lbm_t* h, int64_t n_steps, double dt, do
       return fail(h, IBM_LBM_E_CUDA, "solid_steps: copy of f_ext failed");
     }
   }
-  for (int64_t s = 0; s < n_steps; ++s) {
-    enqueue_forces(h, st);
-    launch_solid_half(h->m, h->solid_v, fe, dt, gamma, mass, true, st);
-    enqueue_forces(h, st);
-    launch_solid_half(h->m, h->solid_v, fe, dt, gamma, mass, false, st);
+  // Few membranes and nothing else: a cluster per body, SOLID_CHUNK steps a
+  // launch (a few ms). Its work is ~1.5 times that of one block per body and
+  // its latency a tenth: better while the clusters fill the chip a few times.
+  const bool clusters = h->n_membranes > 0 && h->n_membranes == h->n_bodies && !h->need_zero_F &&
+                        !(h->morse_rc > 0.0) && h->mesh.part_tris > 0 && solid_cluster_fits(h->mesh);
+  if (clusters) {
+    for (int64_t s = 0; s < n_steps; s += SOLID_CHUNK)
+      launch_solid_cluster(h->m, h->d_bodies, h->membrane_list, h->n_membranes, h->mesh, h->solid_v, fe, dt, gamma,
+                           mass, (int)std::min<int64_t>(SOLID_CHUNK, n_steps - s), st);
+  } else {
+    for (int64_t s = 0; s < n_steps; ++s) {
+      // (from the second step on the forces are those the last one ended with)
+      if (s == 0) enqueue_forces(h, st);
+      launch_solid_half(h->m, h->solid_v, fe, dt, gamma, mass, true, st);
+      enqueue_forces(h, st);
+      launch_solid_half(h->m, h->solid_v, fe, dt, gamma, mass, false, st);
+    }
   }
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);

@@ -52,6 +52,140 @@ void launch_kind(const ClusterLaunch& Q, int n, size_t smem, cudaStream_t st) {
   }
 }
 
+// Solid-only dynamics of few membranes (solid.cu): a cluster per body takes
+// many steps in one launch. The general path launches the force kernel and a
+// Verlet half step twice per step, and one block's latency decides it (66 us a
+// step for a 1442-vertex cell: 2 x 42 us of forces, of which the first repeats
+// the last of the step before, 2 x 5 us of FP64). Here positions, velocities
+// and external forces stay in registers, each step's forces are computed once,
+// and the second half of a step and the first of the next are one update. Two
+// cluster barriers a step: the positions are double-buffered, so that a block
+// may write the next ones while another still reads these.
+constexpr int SOLID_THREADS = 512;
+constexpr int SOLID_ITEMS = 5;  // coordinates a thread carries: 3 * cluster_per(nv) <= 512 * 5
+
+struct SolidLaunch {
+  MarkersDev m;
+  BodyDev* bodies;
+  const int* list;
+  MeshDev mesh;
+  double* v;           // [3][M]
+  const double* fext;  // [3][M] or null
+  double dt, gamma, inv_mass;
+  int steps;
+};
+
+__host__ __device__ constexpr int solid_words(int nv, int nt_part) { return 3 * cluster_per(nv) + 12 * nv + 4 * nt_part; }
+
+__global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(SOLID_THREADS, 1)
+    k_solid_cluster(const __grid_constant__ SolidLaunch Q) {
+  using namespace cluster_detail;
+  extern __shared__ __align__(16) unsigned char smem[];
+  __shared__ ClusterShare S;
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x, lane = tid & 31;
+  const MarkersDev& m = Q.m;
+  const size_t M = (size_t)m.M;
+  BodyDev* B = Q.bodies + Q.list[blockIdx.x / CLUSTER];
+  const int nv = Q.mesh.nv, per = cluster_per(nv), nt_part = Q.mesh.part_tris;
+  const int c0 = min(rank * per, nv), n = min(per, nv - c0), first = B->first + c0;
+  const MeshPart P = mesh_part(Q.mesh, rank);
+  int* sQ = reinterpret_cast<int*>(smem);              // [3][per]
+  float* pos = reinterpret_cast<float*>(sQ + 3 * per);  // [2][6][nv]
+  float* sN = pos + 12 * nv;                           // [3][nt_part]
+  float* sA = sN + 3 * nt_part;                        // [nt_part]
+  const int o[3] = {m.cell[B->first], m.cell[M + B->first], m.cell[2 * M + B->first]};
+  const MembraneModuli Km{B->kBT_p, B->k_b, B->k_l, B->k_g, B->k_v};
+  float q_prev = B->qmax;
+  const double h = 0.5 * Q.dt, damp = 1.0 / (1.0 + 0.5 * Q.gamma * Q.dt);
+  // item i of this thread: coordinate a of own vertex j
+  double X[SOLID_ITEMS], v[SOLID_ITEMS], fe[SOLID_ITEMS];
+  float F[SOLID_ITEMS];
+#pragma unroll
+  for (int t = 0; t < SOLID_ITEMS; ++t) {
+    const int i = tid + t * SOLID_THREADS;
+    X[t] = v[t] = fe[t] = 0.0;
+    F[t] = 0.f;
+    if (i >= 3 * n) continue;
+    const int a = i / n;
+    const size_t k = a * M + first + (i - a * n);
+    X[t] = m.X[k];
+    v[t] = Q.v[k];
+    fe[t] = Q.fext ? Q.fext[k] * Q.inv_mass : 0.0;
+  }
+  for (int i = tid; i < 3 * per; i += SOLID_THREADS) sQ[i] = 0;
+  if (tid < 2) S.fix[tid] = 0;
+  if (tid < CLUSTER) S.qmax[tid] = 0u;
+  if (tid == 0) S.fmax_s = 0u;
+  cl.sync();  // every block has started and has read the origin
+  // s = -1: forces at the start; step s: Verlet update to new positions, their forces
+  for (int s = -1; s < Q.steps; ++s) {
+    float* sI = pos + ((s & 1) ? 6 * nv : 0);
+    float* sR = sI + 3 * nv;
+#pragma unroll
+    for (int t = 0; t < SOLID_ITEMS; ++t) {
+      const int i = tid + t * SOLID_THREADS;
+      if (i >= 3 * n) continue;
+      const int a = i / n, j = i - a * n;
+      if (s >= 0) {
+        const double acc = fma((double)F[t], Q.inv_mass, fe[t]);
+        if (s > 0) v[t] = fma(h, acc, v[t]) * damp;  // second half of step s - 1
+        v[t] = fma(h, fma(-Q.gamma, v[t], acc), v[t]);
+        X[t] = fma(Q.dt, v[t], X[t]);
+      }
+      int c;
+      float f;
+      split_coord(X[t], c, f);
+      const float fc = (float)(c - o[a]);
+#pragma unroll
+      for (int r = 0; r < CLUSTER; ++r) {
+        cl.map_shared_rank(sI, r)[a * nv + c0 + j] = fc;
+        cl.map_shared_rank(sR, r)[a * nv + c0 + j] = f;
+      }
+    }
+    cl.sync();  // positions complete; every block is done with the last sums
+    float unit;
+    float qmax = cluster_membrane<SOLID_THREADS>(S, MembraneArrays{sI, sR, sN, sA, sQ, nv, nt_part, per, c0, n}, P,
+                                                 Q.mesh, Km, q_prev, unit);
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, w));
+    if (lane == 0) atomicMax(&S.fmax_s, __float_as_uint(qmax));  // non-negative floats order as their bits
+    __syncthreads();  // the sums and the largest contribution are complete
+    const float qb = __uint_as_float(S.fmax_s);
+    q_prev = isfinite(qb) ? qb : 0.f;  // this block's scale: its own largest contribution
+#pragma unroll
+    for (int t = 0; t < SOLID_ITEMS; ++t) {
+      const int i = tid + t * SOLID_THREADS;
+      if (i >= 3 * n) continue;
+      const int a = i / n, j = i - a * n, q = a * per + j;
+      F[t] = unit > 0.f ? (float)sQ[q] * unit : __int_as_float(sQ[q]);
+      sQ[q] = 0;
+    }
+    __syncthreads();  // (all have read the maximum)
+    if (tid == 0) S.fmax_s = 0u;
+    if (tid < 2) S.fix[tid] = 0;
+  }
+  if (tid == 0) cl.map_shared_rank(&S.qmax[0], 0)[rank] = __float_as_uint(q_prev);
+#pragma unroll
+  for (int t = 0; t < SOLID_ITEMS; ++t) {
+    const int i = tid + t * SOLID_THREADS;
+    if (i >= 3 * n) continue;
+    const int a = i / n, j = i - a * n;
+    const size_t k = a * M + first + j;
+    if (Q.steps > 0) v[t] = fma(h, fma((double)F[t], Q.inv_mass, fe[t]), v[t]) * damp;
+    Q.v[k] = v[t];
+    m.X[k] = X[t];
+    cache_coord(m, k, X[t]);
+    reinterpret_cast<float*>(m.F + first + j)[a] = F[t];
+  }
+  cl.sync();
+  if (rank == 0 && tid == 0) {
+    float q = 0.f;
+    for (int r = 0; r < CLUSTER; ++r) q = fmaxf(q, __uint_as_float(S.qmax[r]));
+    B->qmax = q;
+  }
+}
+
 }  // namespace
 
 cudaError_t cluster_configure() {
@@ -59,8 +193,20 @@ cudaError_t cluster_configure() {
 #define CFG(k) if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, CLUSTER_SMEM_MAX)
   CFG((k_couple_cluster<GEOM_PERIODIC, 0>)); CFG((k_couple_cluster<GEOM_YWALLS, 0>)); CFG((k_couple_cluster<GEOM_TUBE, 0>));
   CFG((k_couple_cluster<GEOM_PERIODIC, 1>)); CFG((k_couple_cluster<GEOM_YWALLS, 1>)); CFG((k_couple_cluster<GEOM_TUBE, 1>));
+  CFG(k_solid_cluster);
 #undef CFG
   return e;
+}
+
+bool solid_cluster_fits(const MeshDev& mesh) {
+  return 3 * cluster_per(mesh.nv) <= SOLID_THREADS * SOLID_ITEMS &&
+         4 * (size_t)solid_words(mesh.nv, mesh.part_tris) <= (size_t)CLUSTER_SMEM_MAX;
+}
+
+void launch_solid_cluster(const MarkersDev& m, BodyDev* bodies, const int* list, int n, const MeshDev& mesh, double* v,
+                          const double* fext, double dt, double gamma, double mass, int steps, cudaStream_t st) {
+  const SolidLaunch Q{m, bodies, list, mesh, v, fext, dt, gamma, 1.0 / mass, steps};
+  k_solid_cluster<<<n * CLUSTER, SOLID_THREADS, 4 * (size_t)solid_words(mesh.nv, mesh.part_tris), st>>>(Q);
 }
 
 // Cells of a block's box: what one resident wave of the launch leaves, at

@@ -205,6 +205,118 @@ __device__ __forceinline__ void cluster_rows(const LatticeDev& L, const int4* lo
   }
 }
 
+// A block's views of its membrane: the whole body's positions (integer part
+// relative to a common origin, fraction), its part's normals and areas, its
+// own vertices' force sums.
+struct MembraneArrays {
+  const float *sI, *sR;  // [3][nv]
+  float *sN, *sA;        // [3][nt_part], [nt_part]
+  int* sQ;               // [3][per]
+  int nv, nt_part, per, c0, n;
+};
+struct MembraneModuli {
+  float kBT_p, k_b, k_l, k_g, k_v;
+};
+
+// Forces on this block's vertices c0 .. c0 + n - 1 of a membrane whose
+// positions all blocks of the cluster have written (and synchronised on),
+// with S.fix and sQ cleared. The sums are left in sQ: fixed point in units of
+// `unit`, or floats where unit = 0 (as membrane_core: no scale yet, or a
+// contribution above its headroom). Returns the thread's largest contribution;
+// q_prev: the largest one of the last evaluation. Contains one cluster barrier.
+template <int THREADS>
+__device__ __forceinline__ float cluster_membrane(ClusterShare& S, const MembraneArrays& W, const MeshPart& P,
+                                                  const MeshDev& mesh, const MembraneModuli& Km, float q_prev,
+                                                  float& unit) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), tid = threadIdx.x;
+  const float *sI = W.sI, *sR = W.sR;
+  float *sN = W.sN, *sA = W.sA;
+  int* sQ = W.sQ;
+  float* sF = reinterpret_cast<float*>(sQ);
+  const int nv = W.nv, nt_part = W.nt_part, per = W.per, c0 = W.c0, n = W.n;
+  const MembraneScale K = membrane_scale(mesh);
+  auto dv = [&](int p, int q) {
+    return make_float3((sI[p] - sI[q]) + (sR[p] - sR[q]), (sI[nv + p] - sI[nv + q]) + (sR[nv + p] - sR[nv + q]),
+                       (sI[2 * nv + p] - sI[2 * nv + q]) + (sR[2 * nv + p] - sR[2 * nv + q]));
+  };
+  auto normal = [&](int t) { return make_float3(sN[t], sN[nt_part + t], sN[2 * nt_part + t]); };
+  // A. normals and areas of the part's triangles; each triangle counts once
+  // for the body's area and volume (flag in .w)
+  float ap = 0.f, vp = 0.f;
+  for (int t = tid; t < P.nt; t += THREADS) {
+    const ushort4 Tr = P.tris[t];
+    const float3 N = cross(dv(Tr.y, Tr.x), dv(Tr.z, Tr.x));
+    const float At = 0.5f * sqrtf(dot(N, N));
+    sN[t] = N.x; sN[nt_part + t] = N.y; sN[2 * nt_part + t] = N.z;
+    sA[t] = At;
+    if (Tr.w) {
+      ap += At;
+      vp += dot(dv(Tr.x, 0), N) * (1.0f / 6.0f);
+    }
+  }
+  warp_fixed_sum(ap, vp, K, S.fix);
+  __syncthreads();
+  if (tid < 2 * CLUSTER) {
+    const int r = tid >> 1, q = tid & 1;
+    cl.map_shared_rank(&S.sum[0][0], r)[6 * rank + q] = (double)S.fix[q];
+  }
+  // the area and volume terms need the other blocks' sums; the edges do not
+  cl.barrier_arrive();
+  float qmax = 0.f;
+  auto edges = [&](auto&& add) {
+    for (int e = tid; e < P.ne; e += THREADS)
+      edge_forces(P.edges[e], P.edge_tris[e], P.edge_rest[e], Km.kBT_p, Km.k_b, dv, normal, add);
+  };
+  const float Sq = q_prev > 0.f ? mesh.qcap / (4.0f * q_prev) : 0.f;
+  bool over = !(q_prev > 0.f);
+  auto add_fixed = [&](int v, float3 f) {
+    const float c = fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z)));
+    qmax = fmaxf(qmax, c);
+    over |= !(c * Sq <= mesh.qcap);
+    const int i = v - c0;
+    if ((unsigned)i < (unsigned)n) {
+      atomicAdd(sQ + i, __float2int_rn(f.x * Sq));
+      atomicAdd(sQ + per + i, __float2int_rn(f.y * Sq));
+      atomicAdd(sQ + 2 * per + i, __float2int_rn(f.z * Sq));
+    }
+  };
+  const bool scaled = q_prev > 0.f;
+  if (scaled) edges(add_fixed);
+  cl.barrier_wait();  // partial areas and volumes of all blocks
+  double sa = 0.0, sv = 0.0;
+#pragma unroll
+  for (int r = 0; r < CLUSTER; ++r) {
+    sa += S.sum[r][0];
+    sv += S.sum[r][1];
+  }
+  const float cg_ = Km.k_g * ((float)(sa * K.qa - (double)mesh.A0) / mesh.A0);
+  const float cv_ = Km.k_v * ((float)(sv * K.qv - (double)mesh.V0) / mesh.V0);
+  auto triangles = [&](auto&& add) {
+    for (int t = tid; t < P.nt_own; t += THREADS)
+      triangle_forces(P.tris[t], normal(t), sA[t], P.area0[t], Km.k_l, cg_, cv_, dv, add);
+  };
+  if (scaled) triangles(add_fixed);
+  const bool redo = __syncthreads_or(over) != 0;
+  unit = redo ? 0.f : 1.0f / Sq;
+  if (redo) {
+    for (int i = tid; i < 3 * per; i += THREADS) sF[i] = 0.f;
+    __syncthreads();
+    auto add_float = [&](int v, float3 f) {
+      qmax = fmaxf(qmax, fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z))));
+      const int i = v - c0;
+      if ((unsigned)i < (unsigned)n) {
+        atomicAdd(sF + i, f.x);
+        atomicAdd(sF + per + i, f.y);
+        atomicAdd(sF + 2 * per + i, f.z);
+      }
+    };
+    edges(add_float);
+    triangles(add_float);
+  }
+  return qmax;
+}
+
 }  // namespace cluster_detail
 
 // The whole coupling of one body by its cluster (blockDim = CLUSTER_THREADS,
@@ -442,7 +554,6 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
       }
     }
   } else {
-    const MeshPart P = mesh_part(A.mesh, rank);
     __syncthreads();
     // own positions to every block of the cluster
     for (int i = tid; i < 3 * n; i += CLUSTER_THREADS) {
@@ -462,87 +573,10 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
     if (tid < 2) S.fix[tid] = 0;
     if (tid < CLUSTER) S.qmax[tid] = 0u;
     cl.sync();  // positions complete
-    const MembraneScale K = membrane_scale(A.mesh);
-    auto dv = [&](int p, int q) {
-      return make_float3((sI[p] - sI[q]) + (sR[p] - sR[q]), (sI[nv + p] - sI[nv + q]) + (sR[nv + p] - sR[nv + q]),
-                         (sI[2 * nv + p] - sI[2 * nv + q]) + (sR[2 * nv + p] - sR[2 * nv + q]));
-    };
-    auto normal = [&](int t) { return make_float3(sN[t], sN[nt_part + t], sN[2 * nt_part + t]); };
-    // A. normals and areas of the part's triangles; each triangle counts once
-    // for the body's area and volume (flag in .w)
-    float ap = 0.f, vp = 0.f;
-    for (int t = tid; t < P.nt; t += CLUSTER_THREADS) {
-      const ushort4 Tr = P.tris[t];
-      const float3 N = cross(dv(Tr.y, Tr.x), dv(Tr.z, Tr.x));
-      const float At = 0.5f * sqrtf(dot(N, N));
-      sN[t] = N.x; sN[nt_part + t] = N.y; sN[2 * nt_part + t] = N.z;
-      sA[t] = At;
-      if (Tr.w) {
-        ap += At;
-        vp += dot(dv(Tr.x, 0), N) * (1.0f / 6.0f);
-      }
-    }
-    warp_fixed_sum(ap, vp, K, S.fix);
-    __syncthreads();
-    if (tid < 2 * CLUSTER) {
-      const int r = tid >> 1, q = tid & 1;
-      cl.map_shared_rank(&S.sum[0][0], r)[6 * rank + q] = (double)S.fix[q];
-    }
-    // the area and volume terms need the other blocks' sums; the edges do not
-    cl.barrier_arrive();
-    const float kBT_p = B->kBT_p, k_b = B->k_b, k_l = B->k_l, q_prev = B->qmax;
-    float qmax = 0.f;
-    auto edges = [&](auto&& add) {
-      for (int e = tid; e < P.ne; e += CLUSTER_THREADS)
-        edge_forces(P.edges[e], P.edge_tris[e], P.edge_rest[e], kBT_p, k_b, dv, normal, add);
-    };
-    const float Sq = q_prev > 0.f ? A.mesh.qcap / (4.0f * q_prev) : 0.f;
-    bool over = !(q_prev > 0.f);
-    auto add_fixed = [&](int v, float3 f) {
-      const float c = fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z)));
-      qmax = fmaxf(qmax, c);
-      over |= !(c * Sq <= A.mesh.qcap);
-      const int i = v - c0;
-      if ((unsigned)i < (unsigned)n) {
-        atomicAdd(sQ + i, __float2int_rn(f.x * Sq));
-        atomicAdd(sQ + per + i, __float2int_rn(f.y * Sq));
-        atomicAdd(sQ + 2 * per + i, __float2int_rn(f.z * Sq));
-      }
-    };
-    if (!over) edges(add_fixed);
-    cl.barrier_wait();  // partial areas and volumes of all blocks
-    double sa = 0.0, sv = 0.0;
-#pragma unroll
-    for (int r = 0; r < CLUSTER; ++r) {
-      sa += S.sum[r][0];
-      sv += S.sum[r][1];
-    }
-    const float cgm = B->k_g * ((float)(sa * K.qa - (double)A.mesh.A0) / A.mesh.A0);
-    const float cvm = B->k_v * ((float)(sv * K.qv - (double)A.mesh.V0) / A.mesh.V0);
-    auto triangles = [&](auto&& add) {
-      for (int t = tid; t < P.nt_own; t += CLUSTER_THREADS)
-        triangle_forces(P.tris[t], normal(t), sA[t], P.area0[t], k_l, cgm, cvm, dv, add);
-    };
-    if (!over) triangles(add_fixed);
-    const bool redo = __syncthreads_or(over) != 0;
-    float unit = 0.f;
-    if (redo) {
-      for (int i = tid; i < 3 * per; i += CLUSTER_THREADS) sF[i] = 0.f;
-      __syncthreads();
-      auto add_float = [&](int v, float3 f) {
-        qmax = fmaxf(qmax, fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z))));
-        const int i = v - c0;
-        if ((unsigned)i < (unsigned)n) {
-          atomicAdd(sF + i, f.x);
-          atomicAdd(sF + per + i, f.y);
-          atomicAdd(sF + 2 * per + i, f.z);
-        }
-      };
-      edges(add_float);
-      triangles(add_float);
-    } else {
-      unit = 1.0f / Sq;
-    }
+    const MembraneModuli Km{B->kBT_p, B->k_b, B->k_l, B->k_g, B->k_v};
+    float unit;
+    float qmax = cluster_membrane<CLUSTER_THREADS>(S, MembraneArrays{sI, sR, sN, sA, sQ, nv, nt_part, per, c0, n},
+                                                   mesh_part(A.mesh, rank), A.mesh, Km, B->qmax, unit);
 #pragma unroll
     for (int s = 16; s > 0; s >>= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, s));
     if (lane == 0) atomicMax(cl.map_shared_rank(&S.qmax[0], 0) + rank, __float_as_uint(qmax));

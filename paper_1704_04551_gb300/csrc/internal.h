@@ -49,6 +49,10 @@ void launch_couple_cluster(const LatticeDev& L, float4* g_next, uint8_t* flags_n
                            BodyDev* bodies, const int* list, int n, bool membranes, int max_count,
                            const MeshDev& mesh, int4* boxes, int n_sm, bool interp, bool forces, bool spread,
                            cudaStream_t st);
+// many steps of the solid-only dynamics of few membranes in one launch
+bool solid_cluster_fits(const MeshDev& mesh);
+void launch_solid_cluster(const MarkersDev& m, BodyDev* bodies, const int* list, int n, const MeshDev& mesh, double* v,
+                          const double* fext, double dt, double gamma, double mass, int steps, cudaStream_t st);
 
 // solid.cu
 void launch_solid_half(const MarkersDev& m, double* v, const double* fext, double dt, double gamma, double mass,

@@ -98,3 +98,36 @@ def test_solid_steps_errors(cuda_lib):
     with pytest.raises(IbmLbmError) as e:
         sim.solid_steps(10, 1.0, 0.05, 1.0)
     assert e.value.code == E_STATE
+
+
+# (template frequency, bodies, calls): the smallest template, one that leaves
+# blocks of the clusters short, a large one, more bodies than take clusters
+# (the general path, which keeps the forces of the step before), a call
+# longer than one launch takes
+@pytest.mark.parametrize('freq,bodies,calls', [(1, 3, (1, 2, 5)), (3, 2, (20,)), (16, 2, (6, 1)), (4, 130, (1, 7)),
+                                               (2, 1, (520,))])
+def test_solid_steps_of_several_bodies_match_oracle(cuda_lib, freq, bodies, calls):
+    from paper_1704_04551_gb300.binding import Simulation
+    rest, tris = I.rbc_rest_shape(16.0, freq)
+    V = rest.shape[1]
+    rng = np.random.default_rng(17)
+    l0 = 16.0 / (2.0 * freq)
+    X = np.concatenate([rest * np.exp(rng.uniform(-0.04, 0.04, (3, 1))) + 20.0 * rng.random((3, 1)) for _ in range(bodies)],
+                       axis=1)
+    bs = [I._body(I.BODY_MEMBRANE, k * V, V, kBT_p=2e-3 * l0 * rng.uniform(0.8, 1.2), k_b=1e-3, k_l=5e-3, k_g=4e-3,
+                  k_v=3e-3) for k in range(bodies)]
+    F = 1e-4 * rng.standard_normal(X.shape)
+    sim, ora = Simulation(LAT), O.Oracle(LAT)
+    sim.set_markers(dict(rest_X=rest, tris=tris), bs, X)
+    ora.set_mesh(tris, rest)
+    ora.set_bodies(bs, X)
+    v = None
+    for n in calls:
+        sim.solid_steps(n, 1.0, 0.05, 1.0, F)
+        v = ora.solid_steps(n, 1.0, 0.05, 1.0, F, v=v)
+    Xg, _, Fg = sim.markers()
+    Xo, _, Fo = ora.markers()
+    disp = np.abs(Xo - X).max()
+    assert disp > 1e-4
+    assert np.abs(Xg - Xo).max() < 1e-4 * disp
+    assert np.abs(Fg - Fo).max() < 1e-3 * np.abs(Fo).max()
