@@ -560,11 +560,9 @@ MeshPartHost mesh_part_of(const HostMesh& m, int v0, int v1) {
         ghosts.push_back(t);
       }
   }
-  std::vector<std::array<int, 3>> tk;
-  for (int t : touching) tk.push_back({m.tris[t].x, m.tris[t].y, m.tris[t].z});
+  // (in the template's order, which spreads the shared-memory banks)
   P.nt_own = (int)touching.size();
-  std::vector<int> order;
-  for (int i : bank_order<3>(tk)) order.push_back(touching[i]);
+  std::vector<int> order = touching;
   order.insert(order.end(), ghosts.begin(), ghosts.end());
   for (size_t i = 0; i < order.size(); ++i) {
     const int t = order[i];
@@ -572,15 +570,10 @@ MeshPartHost mesh_part_of(const HostMesh& m, int v0, int v1) {
     P.tris.push_back(make_ushort4(m.tris[t].x, m.tris[t].y, m.tris[t].z, own(m.tris[t].x) ? 1 : 0));
     P.area0.push_back(m.area0[t]);
   }
-  std::vector<std::array<int, 6>> ek;
   for (int e : edges) {
     const int4 E = m.edges[e];
-    ek.push_back({E.x, E.y, E.z, E.w, local[m.edge_tris[e].x], local[m.edge_tris[e].y]});
-  }
-  for (int i : bank_order<6>(ek)) {
-    const int e = edges[i];
-    P.edges.push_back(make_ushort4(ek[i][0], ek[i][1], ek[i][2], ek[i][3]));
-    P.edge_tris.push_back(make_ushort2(ek[i][4], ek[i][5]));
+    P.edges.push_back(make_ushort4(E.x, E.y, E.z, E.w));
+    P.edge_tris.push_back(make_ushort2(local[m.edge_tris[e].x], local[m.edge_tris[e].y]));
     P.edge_rest.push_back(m.edge_rest[e]);
   }
   return P;
