@@ -6,7 +6,10 @@
 // of memory the library allocates. The operation is the spreading of Eq.
 // ibmForceSpread with the 4-point cosine delta of Eq. deltaPhiSimple, the
 // same as the SPREAD stage of a handle.
+#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "../../include/ibm_lbm.h"
 #include "common.cuh"
@@ -46,53 +49,84 @@ __device__ __forceinline__ bool grid_solid(const Grid& G, int y, int z) {
   return false;
 }
 
-__global__ void k_spread_noalloc(Grid G, const double* __restrict__ X, const double* __restrict__ F, int M,
-                                 float4* acc) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= M) return;
-  const double px = X[k], py = X[(size_t)M + k], pz = X[2 * (size_t)M + k];
-  // Positions come straight from device memory, unchecked by the host: a
-  // marker that is not finite or lies at |x| >= 2^30 (the bound the handle's
-  // set_markers enforces) is skipped, so that no index below overflows.
-  const double lim = 1073741824.0;
-  if (!(fabs(px) < lim && fabs(py) < lim && fabs(pz) < lim)) return;
-  const float fx = (float)F[k], fy = (float)F[(size_t)M + k], fz = (float)F[2 * (size_t)M + k];
-  const double bx = floor(px), by = floor(py), bz = floor(pz);
-  const float ox = (float)(px - bx), oy = (float)(py - by), oz = (float)(pz - bz);
-  float wx[4], wy[4], wz[4];
-  int xs[4];
+// One cooperative launch: clears the accumulator, spreads, writes g out, with
+// a grid barrier between the parts. (As a memset and two kernels, a call of
+// one body's markers on a 48x40x36 lattice took 22 us, most of it launches and
+// one thread's walk through its marker's 64 nodes; a 101x97x103 lattice with
+// 120,000 markers took 63 us, 49 of them the spreading.) Sixteen lanes share a
+// marker: lane q < 3 splits coordinate q and rounds force component q (FP64
+// conversions run at 2 lanes a cycle on an SM: once per marker), lanes 0..11
+// evaluate one of the twelve weights each; then four lanes add the four nodes
+// of an x row, 64 consecutive bytes, and the lane groups take four rows a pass
+// (one lane per row, each atomic a sector of its own, took 55 us on the second
+// lattice above).
+constexpr int SPREAD_THREADS = 256;
+constexpr int SPREAD_BLOCKS_PER_SM = 4;
+constexpr int SPREAD_LANES = 16;
+
+__global__ void __launch_bounds__(SPREAD_THREADS, SPREAD_BLOCKS_PER_SM)
+    k_spread_noalloc(Grid G, const double* __restrict__ X, const double* __restrict__ F, int M, float4* acc, double* g) {
+  const cooperative_groups::grid_group grid = cooperative_groups::this_grid();
+  const unsigned tid = blockIdx.x * (unsigned)SPREAD_THREADS + threadIdx.x;
+  const unsigned threads = gridDim.x * (unsigned)SPREAD_THREADS;
+  for (unsigned i = tid; i < (unsigned)G.N; i += threads) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+  grid.sync();
+  const int lane = threadIdx.x & (SPREAD_LANES - 1);
+  const unsigned group = tid / SPREAD_LANES, groups = threads / SPREAD_LANES;
+  // whole warps iterate together (shuffles)
+  const unsigned warp_group = group & ~1u;
+  for (unsigned k0 = 0; k0 + warp_group < (unsigned)M; k0 += groups) {
+    const unsigned k = k0 + group;
+    const bool active = k < (unsigned)M;
+    // Positions come straight from device memory, unchecked by the host: a
+    // marker that is not finite or lies at |x| >= 2^30 (the bound the handle's
+    // set_markers enforces) is skipped, so that no index below overflows.
+    int cell = 0;
+    float frac = 0.f, force = 0.f;
+    bool bad = !active;
+    if (active && lane < 3) {
+      const size_t off = (size_t)lane * (size_t)M + k;
+      const double x = X[off];
+      bad = ((__double2hiint(x) >> 20) & 0x7ff) >= 1023 + 30;  // exponent of 2^30 and above, infinities, NaN
+      if (!bad) split_coord(x, cell, frac);
+      force = (float)F[off];
+    }
+    const unsigned votes = __ballot_sync(0xffffffffu, bad);
+    const bool skip = ((votes >> (threadIdx.x & 16u)) & 7u) != 0u;
+    constexpr unsigned ALL = 0xffffffffu;
+    // weight lane & 3 of axis lane / 4
+    const float f = __shfl_sync(ALL, frac, min(lane >> 2, 2), SPREAD_LANES);
+    const float weight = 0.25f * (1.0f + cospif(0.5f * ((float)((lane & 3) - 1) - f)));
+    const int a = lane & 3, b = lane >> 2;
+    const float wx = __shfl_sync(ALL, weight, a, SPREAD_LANES), wy = __shfl_sync(ALL, weight, 4 + b, SPREAD_LANES);
+    float wz[4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    wx[a] = 0.25f * (1.0f + cospif(0.5f * ((float)(a - 1) - ox)));
-    wy[a] = 0.25f * (1.0f + cospif(0.5f * ((float)(a - 1) - oy)));
-    wz[a] = 0.25f * (1.0f + cospif(0.5f * ((float)(a - 1) - oz)));
-    xs[a] = wrapi((int)bx - 1 + a, G.nx);
-  }
-  for (int c = 0; c < 4; ++c) {
-    int z = (int)bz - 1 + c;
-    if (G.geometry != GEOM_TUBE) z = wrapi(z, G.nz);
-    for (int b = 0; b < 4; ++b) {
-      int y = (int)by - 1 + b;
-      if (G.geometry == GEOM_PERIODIC) y = wrapi(y, G.ny);
+    for (int c = 0; c < 4; ++c) wz[c] = __shfl_sync(ALL, weight, 8 + c, SPREAD_LANES);
+    const int bx = __shfl_sync(ALL, cell, 0, SPREAD_LANES) - 1 + a;
+    int y = __shfl_sync(ALL, cell, 1, SPREAD_LANES) - 1 + b;
+    const int bz = __shfl_sync(ALL, cell, 2, SPREAD_LANES) - 1;
+    const float fx = __shfl_sync(ALL, force, 0, SPREAD_LANES), fy = __shfl_sync(ALL, force, 1, SPREAD_LANES),
+                fz = __shfl_sync(ALL, force, 2, SPREAD_LANES);
+    if (skip) continue;
+    const int x = wrapi(bx, G.nx);
+    if (G.geometry == GEOM_PERIODIC) y = wrapi(y, G.ny);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      int z = bz + c;
+      if (G.geometry != GEOM_TUBE) z = wrapi(z, G.nz);
       if (grid_solid(G, y, z)) continue;
-      const float wyz = wy[b] * wz[c];
-      float4* row = acc + G.nx * (y + G.ny * z);
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        const float w = wx[a] * wyz;
-        atomicAdd(row + xs[a], make_float4(fx * w, fy * w, fz * w, 0.f));
-      }
+      const float w = wx * (wy * wz[c]);
+      atomicAdd(acc + G.nx * (y + G.ny * z) + x, make_float4(fx * w, fy * w, fz * w, 0.f));
     }
   }
-}
-
-__global__ void k_scatter_noalloc(const float4* acc, int N, double* g) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= N) return;
-  const float4 v = acc[i];
-  g[i] = v.x;
-  g[(size_t)N + i] = v.y;
-  g[2 * (size_t)N + i] = v.z;
+  grid.sync();
+  const size_t N = (size_t)G.N;
+  for (unsigned i = tid; i < (unsigned)G.N; i += threads) {
+    const float4 v = __ldcg(acc + i);
+    g[i] = v.x;
+    g[N + i] = v.y;
+    g[2 * N + i] = v.z;
+  }
 }
 
 }  // namespace
@@ -114,14 +148,22 @@ int spread_noalloc(const double* X, const double* F, int64_t n_markers, int32_t 
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Grid G{nx, ny, nz, (int)N, geometry, 0.5f * (float)(ny - 1), 0.5f * (float)(nz - 1),
          (float)(tube_radius * tube_radius)};
-  if (cudaMemsetAsync(acc, 0, sizeof(float4) * (size_t)N, st) != cudaSuccess) {
+  int M = (int)n_markers, dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
     cudaGetLastError();
     return IBM_LBM_E_CUDA;
   }
-  const int M = (int)n_markers;
-  if (M > 0) k_spread_noalloc<<<(M + 255) / 256, 256, 0, st>>>(G, X, F, M, acc);
-  k_scatter_noalloc<<<(unsigned)((N + 255) / 256), 256, 0, st>>>(acc, (int)N, g);
-  if (cudaGetLastError() != cudaSuccess) return IBM_LBM_E_CUDA;
+  // all blocks resident at once (grid barrier); fewer where there is little to do
+  const long long work = std::max((N + 1) / 2, (long long)M * SPREAD_LANES);
+  const unsigned blocks = (unsigned)std::min<long long>((work + SPREAD_THREADS - 1) / SPREAD_THREADS,
+                                                        (long long)sms * SPREAD_BLOCKS_PER_SM);
+  void* args[] = {&G, &X, &F, &M, &acc, &g};
+  if (cudaLaunchCooperativeKernel((const void*)k_spread_noalloc, dim3(blocks), dim3(SPREAD_THREADS), args, 0, st) !=
+      cudaSuccess) {
+    cudaGetLastError();
+    return IBM_LBM_E_CUDA;
+  }
   return IBM_LBM_OK;
 }
 }  // namespace
