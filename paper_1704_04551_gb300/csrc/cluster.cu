@@ -116,7 +116,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(SOLID_THREADS,
   for (int i = tid; i < 3 * per; i += SOLID_THREADS) sQ[i] = 0;
   if (tid < 2) S.fix[tid] = 0;
   if (tid < CLUSTER) S.qmax[tid] = 0u;
-  if (tid == 0) S.fmax_s = 0u;
+  if (tid == 0) S.fmax_s = S.redo_max = 0u;
   cl.sync();  // every block has started and has read the origin
   // s = -1: forces at the start; step s: Verlet update to new positions, their forces
   for (int s = -1; s < Q.steps; ++s) {

@@ -70,7 +70,7 @@ struct ClusterShare {
   double sum[CLUSTER][6];           // partial force and torque, or area and volume
   unsigned qmax[CLUSTER];           // largest membrane force contribution
   int lo_s[3], hi_s[3];             // own bounds
-  unsigned fmax_s;
+  unsigned fmax_s, redo_max;
   int zero;
   double total[6];                  // force and torque of all blocks
   double pose[12];                  // C, q (4), V; direct forcing
@@ -221,8 +221,7 @@ struct MembraneModuli {
 // Forces on this block's vertices c0 .. c0 + n - 1 of a membrane whose
 // positions all blocks of the cluster have written (and synchronised on),
 // with S.fix and sQ cleared. The sums are left in sQ: fixed point in units of
-// `unit`, or floats where unit = 0 (as membrane_core: no scale yet, or a
-// contribution above its headroom). Returns the thread's largest contribution;
+// `unit`, or floats where unit = 0 (a contribution that is not finite). Returns the thread's largest contribution;
 // q_prev: the largest one of the last evaluation. Contains one cluster barrier.
 template <int THREADS>
 __device__ __forceinline__ float cluster_membrane(ClusterShare& S, const MembraneArrays& W, const MeshPart& P,
@@ -298,21 +297,16 @@ __device__ __forceinline__ float cluster_membrane(ClusterShare& S, const Membran
   };
   if (scaled) triangles(add_fixed);
   const bool redo = __syncthreads_or(over) != 0;
-  unit = redo ? 0.f : 1.0f / Sq;
+  unit = 1.0f / Sq;
   if (redo) {
-    for (int i = tid; i < 3 * per; i += THREADS) sF[i] = 0.f;
-    __syncthreads();
-    auto add_float = [&](int v, float3 f) {
-      qmax = fmaxf(qmax, fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z))));
-      const int i = v - c0;
-      if ((unsigned)i < (unsigned)n) {
-        atomicAdd(sF + i, f.x);
-        atomicAdd(sF + per + i, f.y);
-        atomicAdd(sF + 2 * per + i, f.z);
-      }
+    bool is_float;
+    auto pass = [&](auto&& add) {
+      edges(add);
+      triangles(add);
     };
-    edges(add_float);
-    triangles(add_float);
+    unit = redo_scatter(pass, sQ, per, n, c0, per, mesh.qcap, qmax, &S.redo_max, is_float);
+    __syncthreads();
+    if (tid == 0) S.redo_max = 0u;
   }
   return qmax;
 }
@@ -359,7 +353,7 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
     S.hi_s[tid] = INT_MIN;
   }
   if (tid == 0) {
-    S.fmax_s = 0u;
+    S.fmax_s = S.redo_max = 0u;
     S.zero = 0;
   }
   if (tid < CLUSTER) {

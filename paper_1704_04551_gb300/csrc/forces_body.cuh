@@ -208,7 +208,7 @@ struct MembraneSmem {
 };
 
 // The per-vertex force sums membrane_core leaves in S.sQ [3][nv]: fixed-point
-// integers in units of `unit`, or float bits after the float redo.
+// integers in units of `unit`, or float bits where a contribution is not finite.
 struct ForceSums {
   const int* q;
   bool is_float;
@@ -220,6 +220,49 @@ struct ForceSums {
 
 __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& mesh, const MembraneSmem& S);
 
+// The scatter of a block's force contributions where the last step's largest
+// one gives no scale (none yet, or contributions above its headroom): their
+// maximum is taken first, then they are added in fixed point with the scale it allows, qcap. The sums depend on no
+// order, unlike float atomics, which reruns of a body's first step differed
+// by. Only contributions that are not finite are added as floats, to reach the
+// forces. pass(add) hands out the contributions; vertices [v0, v0 + n) are
+// summed in sQ [3][stride] (zero entries [n, stride) included in the clear).
+// Returns the unit of the sums.
+template <class Pass>
+__device__ __forceinline__ float redo_scatter(Pass&& pass, int* sQ, int stride, int n, int v0, int n_clear, float qcap,
+                                              float& qmax, unsigned* s_qmax, bool& is_float) {
+  float* sF = reinterpret_cast<float*>(sQ);
+  float S = 0.f;
+  for (int mode = 0; mode < 2; ++mode) {
+    if (mode == 1) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
+      if ((threadIdx.x & 31) == 0) atomicMax(s_qmax, __float_as_uint(qmax));
+      for (int i = threadIdx.x; i < 3 * n_clear; i += blockDim.x) sQ[i] = 0;  // (0.f as well)
+      __syncthreads();
+      const float q = __uint_as_float(*s_qmax);
+      is_float = !isfinite(q);
+      S = q > 0.f && !is_float ? qcap / q : 1.0f;
+    }
+    pass([&](int v, float3 f) {
+      const float c = fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z)));
+      qmax = isfinite(f.x + f.y + f.z) ? fmaxf(qmax, c) : __int_as_float(0x7f800000);  // (fmaxf drops a NaN)
+      const int i = v - v0;
+      if (mode == 0 || (unsigned)i >= (unsigned)n) return;
+      if (is_float) {
+        atomicAdd(sF + i, f.x);
+        atomicAdd(sF + stride + i, f.y);
+        atomicAdd(sF + 2 * stride + i, f.z);
+      } else {
+        atomicAdd(sQ + i, __float2int_rn(f.x * S));
+        atomicAdd(sQ + stride + i, __float2int_rn(f.y * S));
+        atomicAdd(sQ + 2 * stride + i, __float2int_rn(f.z * S));
+      }
+    });
+  }
+  return is_float ? 0.f : 1.0f / S;
+}
+
 // Membrane forces of one body by the whole thread block. smem: [9 nv + 4 nt]
 // words (positions as floor + fraction, force sums, normals, areas).
 //
@@ -229,7 +272,7 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
 // q the body's largest contribution component of the previous step, so that
 // contributions up to four times larger than last step's fit in qcap units
 // and no vertex sum can overflow. A block that meets a larger contribution,
-// or has no previous step, redoes the scatter with float atomics. The
+// or has no previous step, redoes the scatter (redo_scatter). The
 // quantum 1/Sq is ~3e-8 q, below the FP32 rounding of the sums.
 __device__ __forceinline__ void membrane_block(const MarkersDev& m, BodyDev* Bp, const MeshDev& mesh,
                                                unsigned char* smem) {
@@ -350,25 +393,17 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
       const float c = fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z)));
       qmax = fmaxf(qmax, c);
       // a contribution above the headroom (or not finite) sends the block to
-      // the float redo, which discards these sums: no branch here
+      // the redo, which discards these sums: no branch here
       over |= !(c * Sq <= mesh.qcap);
       atomicAdd(sQ + v, __float2int_rn(f.x * Sq));
       atomicAdd(sQ + nv + v, __float2int_rn(f.y * Sq));
       atomicAdd(sQ + 2 * nv + v, __float2int_rn(f.z * Sq));
     });
   }
-  const bool fallback = __syncthreads_or(over) != 0;
-  if (fallback) {
-    float* sF = reinterpret_cast<float*>(sQ);
-    for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) sF[i] = 0.f;
-    __syncthreads();
-    pass_b([&](int v, float3 f) {
-      qmax = fmaxf(qmax, fmaxf(fabsf(f.x), fmaxf(fabsf(f.y), fabsf(f.z))));
-      atomicAdd(sF + v, f.x);
-      atomicAdd(sF + nv + v, f.y);
-      atomicAdd(sF + 2 * nv + v, f.z);
-    });
-  }
+  const bool redo = __syncthreads_or(over) != 0;
+  float unit = 1.0f / Sq;
+  bool is_float = false;
+  if (redo) unit = redo_scatter(pass_b, sQ, nv, nv, 0, nv, mesh.qcap, qmax, &s_qmax, is_float);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) qmax = fmaxf(qmax, __shfl_xor_sync(0xffffffffu, qmax, o));
   if ((threadIdx.x & 31) == 0) atomicMax(&s_qmax, __float_as_uint(qmax));  // non-negative floats order as their bits
@@ -379,8 +414,8 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
   }
   ForceSums F;
   F.q = sQ;
-  F.is_float = fallback;
-  F.unit = fallback ? 0.f : 1.0f / Sq;
+  F.is_float = is_float;
+  F.unit = unit;
   return F;
 }
 
