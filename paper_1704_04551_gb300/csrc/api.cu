@@ -148,13 +148,6 @@ void drop_graphs(ibm_lbm_t* h) {
 
 int tiles(const LatticeDev& L) { return L.ntx * L.nty * L.ntz; }
 
-// Lattice view for a step (the AA parity is a kernel template argument, the
-// force density and its flags are single buffers).
-LatticeDev lat(const ibm_lbm_t* h, bool odd) {
-  (void)odd;
-  return h->L;
-}
-
 // How the markers and the lattice exchange velocities and forces. SEPARATE:
 // forces, spreading and interpolation as kernels of their own. FUSED (many
 // membranes) and CLUSTER (few bodies, rigid or membranes): one kernel between
@@ -198,7 +191,6 @@ void enqueue_cluster(ibm_lbm_t* h, int k, int next, bool interp, bool forces, bo
 // filaments), then the Morse excluded volume between bodies.
 void enqueue_forces(ibm_lbm_t* h, cudaStream_t st) {
   if (h->m.M == 0) return;
-  if (h->need_zero_F) cudaMemsetAsync(h->m.F, 0, sizeof(float4) * (size_t)h->m.M, st);
   if (h->cluster_boxes)
     enqueue_cluster(h, 0, 0, false, true, false);
   else
@@ -206,6 +198,19 @@ void enqueue_forces(ibm_lbm_t* h, cudaStream_t st) {
   launch_filaments(h->m, h->d_bodies, h->filament_list, h->n_filaments, st);
   if (h->morse_rc > 0.0 && h->morse_ready)
     launch_morse(h->morse, h->m, h->cfg.nx, h->cfg.ny, h->cfg.nz, h->cfg.geometry, st);
+}
+
+// Spreading of the bodies' forces and the tiles of the tracers' stencils (whose
+// forces a step has zeroed).
+void spread(ibm_lbm_t* h, const LatticeDev& L) {
+  launch_spread(L, h->m, h->groups, h->n_body_groups, h->boxes, h->stream);
+  if (!h->tracers_everywhere)
+    launch_tracers_mark(L, h->m, h->groups + h->n_body_groups, h->n_groups - h->n_body_groups, h->stream);
+}
+
+void interpolate(ibm_lbm_t* h, const LatticeDev& L) {
+  launch_interpolate(L, h->m, h->groups, h->n_body_groups, h->boxes, h->stream);
+  launch_tracers_move(L, h->m, h->groups + h->n_body_groups, h->n_groups - h->n_body_groups, h->stream);
 }
 
 // Forces and spreading of the first step into buffer k.
@@ -220,7 +225,7 @@ void couple_begin(ibm_lbm_t* h, Path p, int k) {
     return;
   }
   enqueue_forces(h, st);
-  launch_spread(L, h->m, h->groups, h->n_groups, h->boxes, st);
+  spread(h, L);
 }
 
 // Interpolation and advection of the step that used buffer k, forces and
@@ -240,11 +245,11 @@ void couple_mid(ibm_lbm_t* h, Path p, int k) {
 void couple_end(ibm_lbm_t* h, Path p, int k) {
   if (h->m.M == 0) return;
   if (p == CLUSTERED) enqueue_cluster(h, k, k, true, false, false);
-  else launch_interpolate(lattice_of(h, p, k), h->m, h->groups, h->n_groups, h->boxes, h->stream);
+  else interpolate(h, lattice_of(h, p, k));
 }
 
 void collide(ibm_lbm_t* h, Path p, int k, bool odd, bool dense) {
-  launch_collide(lattice_of(h, p, k), h->rows, h->n_rows, h->cfg.storage, odd, dense, h->stream);
+  launch_collide(lattice_of(h, p, k), h->rows, h->n_rows, h->cfg.storage, odd, dense || h->tracers_everywhere, h->stream);
 }
 
 // One coupled step by itself on the handle's stream (also used under
@@ -264,16 +269,16 @@ void enqueue_timed_step(ibm_lbm_t* h, bool odd, bool dense) {
   auto mark = [&](int k) {
     if (rec) cudaEventRecord(h->events[base + k], st);
   };
-  const LatticeDev L = lat(h, odd);
-  cudaMemsetAsync(L.flags, 0, (size_t)tiles(L), st);
+  const LatticeDev L = h->L;
   mark(0);
   enqueue_forces(h, st);
   mark(1);
-  if (h->m.M > 0) launch_spread(L, h->m, h->groups, h->n_groups, h->boxes, st);
+  cudaMemsetAsync(L.flags, 0, (size_t)tiles(L), st);
+  if (h->m.M > 0) spread(h, L);
   mark(2);
-  launch_collide(L, h->rows, h->n_rows, h->cfg.storage, odd, dense, st);
+  collide(h, SEPARATE, 0, odd, dense);
   mark(3);
-  if (h->m.M > 0) launch_interpolate(L, h->m, h->groups, h->n_groups, h->boxes, st);
+  if (h->m.M > 0) interpolate(h, L);
   mark(4);
   if (rec) {
     h->timed_odd.push_back(odd ? 1 : 0);
@@ -394,6 +399,8 @@ int enqueue_steps(ibm_lbm_t* h, int64_t n) {
   if (n < 0) return fail(h, IBM_LBM_E_ARG, "n_steps < 0");
   if (n == 0) return IBM_LBM_OK;
   h->boxes_valid = false;  // the last interpolation moves the markers
+  // no force acts on the tracers (set_marker_forces may have left some)
+  if (h->need_zero_F) CUDA_TRY(h, cudaMemsetAsync(h->m.F, 0, sizeof(float4) * (size_t)h->m.M, h->stream));
   int64_t left = n;
   if (path_of(h) != SEPARATE && !h->gbuf2 && (h->timing ? h->timing_fused && left > 2 : left > 1)) {
     if (!ensure_second_buffer(h)) CUDA_TRY(h, cudaGetLastError());  // (no memory: separate kernels)
@@ -1004,6 +1011,8 @@ static void clear_markers(ibm_lbm_t* h) {
   h->n_membranes = h->n_rigids = 0;
   h->groups = nullptr;
   h->n_groups = 0;
+  h->n_body_groups = 0;
+  h->tracers_everywhere = false;
   h->boxes = nullptr;
   h->couple_items = nullptr;
   h->n_couple = 0;
@@ -1209,9 +1218,12 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     for (int b = 0; b < n_bodies; ++b) cuts.push_back({bodies[b].first, b});
     std::sort(cuts.begin(), cuts.end());
     int64_t pos = 0;
+    std::vector<char> is_tracer;
     auto add_run = [&](int64_t a, int64_t b, int step, int flags) {
-      for (int64_t s0 = a; s0 < b; s0 += step)
+      for (int64_t s0 = a; s0 < b; s0 += step) {
         groups.push_back({(int)s0, (int)std::min<int64_t>(step, b - s0), flags});
+        is_tracer.push_back(step == TRACER_GROUP);
+      }
     };
     for (auto& c : cuts) {
       const ibm_lbm_body& B = bodies[c.second];
@@ -1251,8 +1263,14 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
                        [](const std::pair<uint64_t, size_t>& a, const std::pair<uint64_t, size_t>& b) {
                          return a.first < b.first;
                        });
-      std::vector<MarkerGroup> ordered(groups.size());
-      for (size_t g = 0; g < groups.size(); ++g) ordered[g] = groups[key[g].second];
+      // the bodies' groups first, then the tracers'
+      std::vector<MarkerGroup> ordered;
+      ordered.reserve(groups.size());
+      for (int tracers = 0; tracers < 2; ++tracers) {
+        for (size_t g = 0; g < groups.size(); ++g)
+          if (is_tracer[key[g].second] == tracers) ordered.push_back(groups[key[g].second]);
+        if (!tracers) h->n_body_groups = (int)ordered.size();
+      }
       groups.swap(ordered);
     }
     h->n_groups = (int)groups.size();
@@ -1306,6 +1324,10 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     }
   }
   h->need_zero_F = covered < n_markers;
+  // From a tracer per four tiles on the stencils (up to 8 tiles each) reach
+  // most of them: marking costs more than the velocities of the other cells (a
+  // 131x96x110 box with 150,000: 63 us against 16 bytes of 168 per cell).
+  h->tracers_everywhere = 4 * (n_markers - covered) >= (int64_t)tiles(h->L);
   if (h->morse_rc > 0.0) return prepare_morse(h);
   return IBM_LBM_OK;
 }
@@ -1336,6 +1358,7 @@ static int impl_ibm_lbm_solid_steps(ibm_lbm_t* h, int64_t n_steps, double dt, do
   if (M == 0 || n_steps == 0) return IBM_LBM_OK;
   cudaStream_t st = h->stream;
   CUDA_TRY(h, cudaStreamSynchronize(st));
+  if (h->need_zero_F) CUDA_TRY(h, cudaMemsetAsync(h->m.F, 0, sizeof(float4) * M, st));
   if (!h->solid_v) {
     h->solid_v = (double*)dalloc(h, h->marker_mem, sizeof(double) * 3 * M);
     if (!h->solid_v) return fail(h, IBM_LBM_E_NOMEM, "device allocation failed");
@@ -1419,18 +1442,19 @@ static int impl_ibm_lbm_run_stage(ibm_lbm_t* h, int32_t stage) {
   // per-marker path.
   switch (stage) {
     case IBM_LBM_STAGE_FORCES:
+      if (h->need_zero_F) CUDA_TRY(h, cudaMemsetAsync(h->m.F, 0, sizeof(float4) * (size_t)h->m.M, st));
       enqueue_forces(h, st);
       h->boxes_valid = false;
       break;
     case IBM_LBM_STAGE_SPREAD: {
-      const LatticeDev L = lat(h, h->odd_next);
+      const LatticeDev L = h->L;
       CUDA_TRY(h, cudaMemsetAsync(L.flags, 0, (size_t)tiles(L), st));
       launch_spread(L, h->m, h->groups, h->n_groups, h->boxes, st);
       h->boxes_valid = true;
       break;
     }
     case IBM_LBM_STAGE_COLLIDE:
-      launch_collide(lat(h, h->odd_next), h->rows, h->n_rows, h->cfg.storage, h->odd_next, true, st);
+      launch_collide(h->L, h->rows, h->n_rows, h->cfg.storage, h->odd_next, true, st);
       h->odd_next = !h->odd_next;
       break;
     case IBM_LBM_STAGE_INTERP:

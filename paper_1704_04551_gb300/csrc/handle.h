@@ -15,7 +15,6 @@ constexpr int CHUNK = 16;          // steps per captured chunk graph (even)
 constexpr int FUSED_LONG = 64;     // steps per long fused chunk graph (even)
 constexpr int MAX_MESH_VERTICES = 4096;
 constexpr int BODY_GROUP = 1024;   // markers per transfer block within a body
-constexpr int TRACER_GROUP = 256;  // markers per transfer block for passive tracers
 
 struct Alloc {
   void* p;
@@ -63,6 +62,8 @@ struct ibm_lbm {
   int n_sm = 0;
   MarkerGroup* groups = nullptr;  // transfer blocks
   int n_groups = 0;
+  int n_body_groups = 0;          // groups [n_body_groups, n_groups) are runs of tracers
+  bool tracers_everywhere = false;  // they reach most tiles: the collision writes every velocity instead
   int4* boxes = nullptr;          // per group: stencil box origin and size
   // Fused coupling (suspensions of membranes only): one block per body
   // interpolates, computes the forces and spreads; the collision of

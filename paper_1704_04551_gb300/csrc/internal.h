@@ -23,6 +23,9 @@ void launch_spread(const LatticeDev& L, const MarkersDev& m, const MarkerGroup* 
                    cudaStream_t st);
 void launch_interpolate(const LatticeDev& L, const MarkersDev& m, const MarkerGroup* groups, int n_groups,
                         const int4* boxes, cudaStream_t st);
+// tracer groups in a step: mark the tiles their stencils touch; interpolate and advect
+void launch_tracers_mark(const LatticeDev& L, const MarkersDev& m, const MarkerGroup* groups, int n, cudaStream_t st);
+void launch_tracers_move(const LatticeDev& L, const MarkersDev& m, const MarkerGroup* groups, int n, cudaStream_t st);
 cudaError_t transfer_configure();
 void launch_stencil_cache(const MarkersDev& m, cudaStream_t st);
 void launch_expand_xyz(const float4* in, double* out, int M, cudaStream_t st);

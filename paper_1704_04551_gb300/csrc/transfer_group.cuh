@@ -55,6 +55,7 @@ namespace xfer_detail {
 constexpr int XFER_THREADS = 352;   // 11 warps
 constexpr int BOX_CELLS = 6144;     // shared-memory box limit (cells)
 constexpr int XFER_GROUP_MAX = 1024;  // markers per group (records in shared memory)
+constexpr int TRACER_GROUP = 256;     // markers per group of passive tracers
 constexpr int XFER_PER_THREAD = (XFER_GROUP_MAX + XFER_THREADS - 1) / XFER_THREADS;
 constexpr int RESIDUE_BYTES = 512;   // the counting sort's counters (struct Residues)
 // Launches of fewer groups than this take the four-lanes-per-marker
@@ -135,10 +136,11 @@ __device__ __forceinline__ bool fluid_row(const LatticeDev& L, int& y, int& z) {
   return !solid_yz(L, y, z);
 }
 
-// Tiles (at most 2 per axis) covered by a stencil that starts at node b on
-// an axis of n nodes with tile shift sh; periodic axes wrap, others clip.
+// Tiles covered by a stencil that starts at node b on an axis of n nodes with
+// tile shift sh; periodic axes wrap, others clip. At most 3: a stencil that
+// wraps may cover the last tile whole, if that holds one or two nodes only.
 template <bool PERIODIC>
-__device__ __forceinline__ int axis_tiles(int b, int n, int sh, int t[2]) {
+__device__ __forceinline__ int axis_tiles(int b, int n, int sh, int t[3]) {
   int v = PERIODIC ? wrapi(b, n) : b;
   int cnt = 0;
 #pragma unroll
@@ -146,19 +148,19 @@ __device__ __forceinline__ int axis_tiles(int b, int n, int sh, int t[2]) {
     if (PERIODIC && v >= n) v -= n;
     if (!PERIODIC && (unsigned)v >= (unsigned)n) continue;
     const int q = v >> sh;
-    if (cnt == 0 || t[cnt - 1] != q) { if (cnt < 2) t[cnt++] = q; }
+    if (cnt == 0 || t[cnt - 1] != q) { if (cnt < 3) t[cnt++] = q; }
   }
   return cnt;
 }
 
-// Mark the (at most 8) tiles covered by a marker's stencil. Markers of a
+// Mark the (mostly at most 8) tiles covered by a marker's stencil. Markers of a
 // group are numbered along a space-filling curve, so a marker whose tile set
 // equals that of the previous lane's marker skips its stores. All 32 lanes
 // of the warp call this.
 template <int GEOM>
 __device__ __forceinline__ void mark_tiles(const LatticeDev& L, int bx, int by, int bz, bool active,
                                            uint8_t value = 1) {
-  int tx[2] = {-1, -1}, ty[2] = {-1, -1}, tz[2] = {-1, -1};
+  int tx[3] = {-1, -1, -1}, ty[3] = {-1, -1, -1}, tz[3] = {-1, -1, -1};
   const int nx_ = axis_tiles<true>(bx, L.nx, TILE_X_SHIFT, tx);
   const int ny_ = GEOM == GEOM_PERIODIC ? axis_tiles<true>(by, L.ny, TILE_Y_SHIFT, ty)
                                         : axis_tiles<false>(by, L.ny, TILE_Y_SHIFT, ty);
@@ -167,7 +169,7 @@ __device__ __forceinline__ void mark_tiles(const LatticeDev& L, int bx, int by, 
   const int lane = threadIdx.x & 31;
   bool same = __shfl_up_sync(0xffffffffu, (int)active, 1) != 0 && lane >= 1;
 #pragma unroll
-  for (int q = 0; q < 2; ++q) {
+  for (int q = 0; q < 3; ++q) {
     same &= __shfl_up_sync(0xffffffffu, tx[q], 1) == tx[q];
     same &= __shfl_up_sync(0xffffffffu, ty[q], 1) == ty[q];
     same &= __shfl_up_sync(0xffffffffu, tz[q], 1) == tz[q];
