@@ -179,12 +179,22 @@ LatticeDev lattice_of(const ibm_lbm_t* h, Path p, int k) {
   return L;
 }
 
+// Whether a collision and the coupling by clusters start ahead of one another
+// (await_predecessor): one kernel each (rigid bodies or membranes alone, a
+// lattice with fluid), nothing timed between them, and a small lattice: at 32^3
+// a step goes from 22.5 to 20.5 us, but blocks that wait in residence cost a
+// collision of many waves more than the gap between two kernels (256^3 tube:
+// 187 -> 206 ms per 200 steps).
+bool chained(const ibm_lbm_t* h) {
+  return !h->timing && h->n_rows > 0 && h->L.N <= CHAINED_CELLS_MAX && (h->n_rigids > 0) != (h->n_membranes > 0);
+}
+
 void enqueue_cluster(ibm_lbm_t* h, int k, int next, bool interp, bool forces, bool spread) {
   const LatticeDev L = lattice_of(h, CLUSTERED, k), Ln = lattice_of(h, CLUSTERED, next);
   launch_couple_cluster(L, Ln.g, Ln.flags, h->m, h->d_bodies, h->rigid_list, h->n_rigids, false, h->cluster_max,
-                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, h->stream);
+                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, interp && chained(h), h->stream);
   launch_couple_cluster(L, Ln.g, Ln.flags, h->m, h->d_bodies, h->membrane_list, h->n_membranes, true, h->mesh.nv,
-                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, h->stream);
+                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, interp && chained(h), h->stream);
 }
 
 // Marker forces: each body's own forces (membranes, rigid tethers,
@@ -249,7 +259,9 @@ void couple_end(ibm_lbm_t* h, Path p, int k) {
 }
 
 void collide(ibm_lbm_t* h, Path p, int k, bool odd, bool dense) {
-  launch_collide(lattice_of(h, p, k), h->rows, h->n_rows, h->cfg.storage, odd, dense || h->tracers_everywhere, h->stream);
+  const bool early = p == CLUSTERED && chained(h);  // a coupling comes right before
+  launch_collide(lattice_of(h, p, k), h->rows, h->n_rows, h->cfg.storage, odd, dense || h->tracers_everywhere, early,
+                 h->stream);
 }
 
 // One coupled step by itself on the handle's stream (also used under
@@ -343,7 +355,7 @@ int enqueue_fused(ibm_lbm_t* h, int64_t n, bool dense, bool timed) {
       }
       CUDA_TRY(h, cudaGraphLaunch(h->g_mid[which], st));
       mids -= len;
-      continue;
+        continue;
     }
     const size_t base = 5 * h->timed_steps;
     const bool rec = timed && base + 5 <= h->events.size();
@@ -1454,7 +1466,7 @@ static int impl_ibm_lbm_run_stage(ibm_lbm_t* h, int32_t stage) {
       break;
     }
     case IBM_LBM_STAGE_COLLIDE:
-      launch_collide(h->L, h->rows, h->n_rows, h->cfg.storage, h->odd_next, true, st);
+      launch_collide(h->L, h->rows, h->n_rows, h->cfg.storage, h->odd_next, true, false, st);
       h->odd_next = !h->odd_next;
       break;
     case IBM_LBM_STAGE_INTERP:

@@ -44,11 +44,12 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(CLUSTER_THREAD
 }
 
 template <int KIND>
-void launch_kind(const ClusterLaunch& Q, int n, size_t smem, cudaStream_t st) {
+void launch_kind(const ClusterLaunch& Q, int n, size_t smem, bool programmatic, cudaStream_t st) {
+  const dim3 grid(n * CLUSTER), block(CLUSTER_THREADS);
   switch (Q.L.geometry) {
-    case GEOM_PERIODIC: k_couple_cluster<GEOM_PERIODIC, KIND><<<n * CLUSTER, CLUSTER_THREADS, smem, st>>>(Q); break;
-    case GEOM_YWALLS: k_couple_cluster<GEOM_YWALLS, KIND><<<n * CLUSTER, CLUSTER_THREADS, smem, st>>>(Q); break;
-    default: k_couple_cluster<GEOM_TUBE, KIND><<<n * CLUSTER, CLUSTER_THREADS, smem, st>>>(Q); break;
+    case GEOM_PERIODIC: launch_after(k_couple_cluster<GEOM_PERIODIC, KIND>, grid, block, smem, st, programmatic, Q); break;
+    case GEOM_YWALLS: launch_after(k_couple_cluster<GEOM_YWALLS, KIND>, grid, block, smem, st, programmatic, Q); break;
+    default: launch_after(k_couple_cluster<GEOM_TUBE, KIND>, grid, block, smem, st, programmatic, Q); break;
   }
 }
 
@@ -222,14 +223,14 @@ int cluster_box_cells(size_t fixed_words, int n_clusters, int n_sm) {
 void launch_couple_cluster(const LatticeDev& L, float4* g_next, uint8_t* flags_next, const MarkersDev& m,
                            BodyDev* bodies, const int* list, int n, bool membranes, int max_count,
                            const MeshDev& mesh, int4* boxes, int n_sm, bool interp, bool forces, bool spread,
-                           cudaStream_t st) {
+                           bool programmatic, cudaStream_t st) {
   if (n == 0) return;
   const size_t fixed = cluster_fixed_words(max_count, membranes ? mesh.nv : 0, membranes ? mesh.part_tris : 0);
   const int cap = cluster_box_cells(fixed, n, n_sm);
   const ClusterLaunch Q{L, g_next, flags_next, m, bodies, list, mesh, boxes, cap, interp, forces, spread};
   const size_t smem = 4 * fixed + 12 * (size_t)cap;
-  if (membranes) launch_kind<1>(Q, n, smem, st);
-  else launch_kind<0>(Q, n, smem, st);
+  if (membranes) launch_kind<1>(Q, n, smem, programmatic, st);
+  else launch_kind<0>(Q, n, smem, programmatic, st);
 }
 
 }  // namespace ibm

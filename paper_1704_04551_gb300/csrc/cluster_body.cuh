@@ -62,6 +62,10 @@ __host__ __device__ constexpr int cluster_fixed_words(int count, int nv, int nt_
   return (9 * cluster_per(count) + 6 * nv + 4 * nt_part + 3) / 4 * 4;
 }
 
+struct RigidPrep {
+  double R0, R1, R2, wb, g, inv_I, inv_m, V, C;
+};
+
 // What the blocks of a cluster tell one another.
 struct ClusterShare {
   int4 lo[CLUSTER], dims[CLUSTER];  // their boxes (dims.w: the markers fit and were scattered there)
@@ -72,6 +76,8 @@ struct ClusterShare {
   int lo_s[3], hi_s[3];             // own bounds
   unsigned fmax_s, redo_max;
   int zero;
+  RigidPrep prep[3];                // per component (rigid_prepare)
+  double quat[4];
   double total[6];                  // force and torque of all blocks
   double pose[12];                  // C, q (4), V; direct forcing
   double part[CLUSTER_WORKERS / 32][6];
@@ -99,45 +105,74 @@ namespace cluster_detail {
 namespace cg = cooperative_groups;
 
 // Newton-Euler step of a rigid body (forces_body.cuh: rigid_update) by one
-// warp: lane a < 3 carries component a, so that the dependent FP64 chain is
-// a third as long. S.sum: the blocks' parts of the force and torque on the
-// body. Writes the new state to pose (C, q, V) or to the body.
-__device__ __forceinline__ void warp_rigid_update(BodyDev* B, ClusterShare& S, double* pose, bool store) {
+// warp: lane a < 3 carries component a, so that the dependent FP64 chain (the
+// pipe's latency, ~8 us when one thread did all of it between two cluster
+// barriers) is a third as long. What the old state alone decides is computed
+// ahead (rigid_prepare, while the other warps gather): column a of R, the
+// body-frame spin and its gyroscopic term.
+__device__ __forceinline__ void rigid_prepare(const BodyDev* B, ClusterShare& S) {
   const int lane = threadIdx.x & 31, a = lane < 3 ? lane : lane % 3, b = (a + 1) % 3, c = (a + 2) % 3;
   constexpr unsigned ALL = 0xffffffffu;
-  if (lane < 6) {
-    double t = 0.0;
-#pragma unroll
-    for (int r = 0; r < CLUSTER; ++r) t += S.sum[r][lane];
-    S.total[lane] = t;
-  }
-  __syncwarp();
-  const double* sum = S.total;
   const double w = B->quat[0], x = B->quat[1], y = B->quat[2], z = B->quat[3];
-  // column a of R: R[k][a]
-  double R0, R1, R2;
+  double R0, R1, R2;  // R[k][a]
   if (a == 0) { R0 = 1 - 2 * (y * y + z * z); R1 = 2 * (x * y + w * z); R2 = 2 * (x * z - w * y); }
   else if (a == 1) { R0 = 2 * (x * y - w * z); R1 = 1 - 2 * (x * x + z * z); R2 = 2 * (y * z + w * x); }
   else { R0 = 2 * (x * z + w * y); R1 = 2 * (y * z - w * x); R2 = 1 - 2 * (x * x + y * y); }
-  const double V = B->vel[a] + sum[a] * B->inv_mass;
-  const double C = B->center[a] + V;
-  double wb = R0 * B->omega[0] + R1 * B->omega[1] + R2 * B->omega[2];
-  const double tb = R0 * sum[3] + R1 * sum[4] + R2 * sum[5];
+  const double wb = R0 * B->omega[0] + R1 * B->omega[1] + R2 * B->omega[2];
   const double Iw = B->inertia[a] * wb;
   const double g = __shfl_sync(ALL, wb, b) * __shfl_sync(ALL, Iw, c) - __shfl_sync(ALL, wb, c) * __shfl_sync(ALL, Iw, b);
-  wb += (tb - g) * B->inv_inertia[a];
+  if (lane < 3) {
+    RigidPrep& P = S.prep[a];
+    P.R0 = R0; P.R1 = R1; P.R2 = R2;
+    P.wb = wb;
+    P.g = g;
+    P.inv_I = B->inv_inertia[a];
+    P.inv_m = B->inv_mass;
+    P.V = B->vel[a];
+    P.C = B->center[a];
+  }
+  if (lane < 4) S.quat[lane] = B->quat[lane];
+}
+
+// The step, from the blocks' parts S.sum of the force and torque on the body,
+// by the warp that called rigid_prepare. Writes the new state to pose (C, q, V)
+// or, with store, to the body.
+__device__ __forceinline__ void rigid_finish(BodyDev* B, ClusterShare& S, double* pose, bool store) {
+  const int lane = threadIdx.x & 31, a = lane < 3 ? lane : lane % 3;
+  constexpr unsigned ALL = 0xffffffffu;
+  __syncwarp();
+  if (lane < 6) {
+    const double t0 = S.sum[0][lane] + S.sum[1][lane], t1 = S.sum[2][lane] + S.sum[3][lane];
+    const double t2 = S.sum[4][lane] + S.sum[5][lane], t3 = S.sum[6][lane] + S.sum[7][lane];
+    S.total[lane] = (t0 + t1) + (t2 + t3);
+  }
+  __syncwarp();
+  const double* sum = S.total;
+  const RigidPrep P = S.prep[a];
+  const double V = P.V + sum[a] * P.inv_m;
+  const double C = P.C + V;
+  const double tb = P.R0 * sum[3] + P.R1 * sum[4] + P.R2 * sum[5];
+  const double wb = P.wb + (tb - P.g) * P.inv_I;
   // omega = R wb: row sums across the lanes that hold the columns
-  const double p0 = R0 * wb, p1 = R1 * wb, p2 = R2 * wb;
+  const double p0 = P.R0 * wb, p1 = P.R1 * wb, p2 = P.R2 * wb;
   const double ox = __shfl_sync(ALL, p0, 0) + __shfl_sync(ALL, p0, 1) + __shfl_sync(ALL, p0, 2);
   const double oy = __shfl_sync(ALL, p1, 0) + __shfl_sync(ALL, p1, 1) + __shfl_sync(ALL, p1, 2);
   const double oz = __shfl_sync(ALL, p2, 0) + __shfl_sync(ALL, p2, 1) + __shfl_sync(ALL, p2, 2);
-  double q0 = w + 0.5 * (-ox * x - oy * y - oz * z);
-  double q1 = x + 0.5 * (ox * w + oy * z - oz * y);
-  double q2 = y + 0.5 * (-ox * z + oy * w + oz * x);
-  double q3 = z + 0.5 * (ox * y - oy * x + oz * w);
-  const double rn = 1.0 / sqrt(q0 * q0 + q1 * q1 + q2 * q2 + q3 * q3);
-  q0 *= rn; q1 *= rn; q2 *= rn; q3 *= rn;
-  __syncwarp();  // every lane has read the old state
+  // lane k < 4: component k of the quaternion
+  const double w = S.quat[0], x = S.quat[1], y = S.quat[2], z = S.quat[3];
+  const int k = lane & 3;
+  const double d = k == 0 ? -ox * x - oy * y - oz * z
+                          : (k == 1 ? ox * w + oy * z - oz * y : (k == 2 ? -ox * z + oy * w + oz * x : ox * y - oy * x + oz * w));
+  double q = S.quat[k] + 0.5 * d;
+  double n2 = q * q;
+  n2 += __shfl_xor_sync(ALL, n2, 1);
+  n2 += __shfl_xor_sync(ALL, n2, 2);
+  // 1/sqrt(n2): two Newton steps from the FP32 value (relative error 1e-7,
+  // 1e-14, rounding)
+  double rn = (double)rsqrtf((float)n2);
+  rn = rn * (1.5 - 0.5 * n2 * rn * rn);
+  rn = rn * (1.5 - 0.5 * n2 * rn * rn);
+  q *= rn;
   if (lane < 3) {
     if (pose) { pose[a] = C; pose[7 + a] = V; }
     if (store) {
@@ -146,9 +181,9 @@ __device__ __forceinline__ void warp_rigid_update(BodyDev* B, ClusterShare& S, d
       B->omega[a] = a == 0 ? ox : (a == 1 ? oy : oz);
     }
   }
-  if (lane == 0) {
-    if (pose) { pose[3] = q0; pose[4] = q1; pose[5] = q2; pose[6] = q3; }
-    if (store) { B->quat[0] = q0; B->quat[1] = q1; B->quat[2] = q2; B->quat[3] = q3; }
+  if (lane < 4) {
+    if (pose) pose[3 + k] = q;
+    if (store) B->quat[k] = q;
   }
 }
 
@@ -380,6 +415,13 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
 
   // ---- 1. interpolation of step n, advection; rigid forces --------------------
   const bool boxed = S.old_dims[rank].w != 0;
+  // (what follows is the markers', bodies' and boxes' own state: the coupling
+  // before the finished collision wrote it)
+  if (!worker) {
+    if (KIND == 0 && A.forces && (direct || rank == 0)) rigid_prepare(B, S);
+    await_predecessor();
+    dependents_may_launch();
+  }
   if (!worker && A.interp) {
     // the last warp clears the force density and flags that the finished
     // collision read
@@ -400,6 +442,8 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
       load_raw(m, k, rs_next);
     };
     if ((warp << 3) < n) load_marker(quad);
+    await_predecessor();
+    dependents_may_launch();
     for (int j0 = 0; j0 + (warp << 3) < n; j0 += QUADS) {
       const int j = j0 + quad;
       const bool active = j < n, on = active && a < 3;
@@ -525,7 +569,7 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
       m.F[first + j] = make_float4(sF[j], sF[per + j], sF[2 * per + j], 0.f);
     if (direct) {
       cl.sync();
-      if (warp == NWORK) warp_rigid_update(B, S, S.pose, false);
+      if (warp == NWORK) rigid_finish(B, S, S.pose, false);
       __syncthreads();
       rotation_row(S.pose + 3, ra, row);
       Ca = S.pose[ra];
@@ -590,7 +634,7 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
   // the body's new state, from all blocks' sums (the last warp of block 0)
   auto update_body = [&]() {
     if constexpr (KIND == 0) {
-      warp_rigid_update(B, S, nullptr, true);
+      rigid_finish(B, S, nullptr, true);
     } else if (lane == 0) {
       float q = 0.f;
 #pragma unroll

@@ -46,6 +46,33 @@ enum Storage : int { STORE_F32 = 0, STORE_F16 = 1, STORE_BF16 = 2 };
 // Tiles used to mark where markers touch the lattice: 32 (x) x 4 x 4 cells.
 constexpr int TILE_X_SHIFT = 5, TILE_Y_SHIFT = 2, TILE_Z_SHIFT = 2;
 
+// Programmatic dependent launch: a kernel launched by launch_after(..., true)
+// may start while its predecessor in the stream still runs, once all the
+// predecessor's blocks have called dependents_may_launch (or ended). Before
+// await_predecessor returns it may read only what was complete before the
+// predecessor started. The collision and the coupling kernels of a step
+// await theirs before they let their successor go, so a kernel may read,
+// ahead of the wait, whatever the kernel before its predecessor wrote: the
+// coupling its markers. (In an ordinary launch both calls are no-ops.)
+__device__ __forceinline__ void await_predecessor() { cudaGridDependencySynchronize(); }
+__device__ __forceinline__ void dependents_may_launch() { cudaTriggerProgrammaticLaunchCompletion(); }
+
+template <class... P, class... A>
+inline void launch_after(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, bool programmatic,
+                         A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = programmatic ? 1 : 0;
+  cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Exact n / d for 32-bit n (Granlund & Montgomery, "Division by invariant
 // integers using multiplication", 1994): four instructions.
 struct FastDiv {

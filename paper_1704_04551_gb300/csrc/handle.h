@@ -14,6 +14,7 @@ namespace ibm {
 constexpr int CHUNK = 16;          // steps per captured chunk graph (even)
 constexpr int FUSED_LONG = 64;     // steps per long fused chunk graph (even)
 constexpr int MAX_MESH_VERTICES = 4096;
+constexpr int CHAINED_CELLS_MAX = 1 << 18;  // collision and coupling start ahead of one another (api.cu, chained)
 constexpr int BODY_GROUP = 1024;   // markers per transfer block within a body
 
 struct Alloc {

@@ -8,8 +8,8 @@
 namespace ibm {
 
 // lbm.cu
-void launch_collide(const LatticeDev& L, const RowInfo* rows, int n_rows, int storage, bool odd, bool dense,
-                    cudaStream_t st);
+void launch_collide(const LatticeDev& L, const RowInfo* rows, int n_rows, int storage, bool odd, bool dense, bool early,
+                    cudaStream_t st);  // early: right after a coupling kernel (await_predecessor)
 void launch_init_equilibrium(const LatticeDev& L, int storage, cudaStream_t st);
 void launch_export(const LatticeDev& L, int storage, bool odd_next, double* out, cudaStream_t st);
 void launch_import(const LatticeDev& L, int storage, const double* in, cudaStream_t st);
@@ -51,7 +51,7 @@ int cluster_box_cells(size_t fixed_words, int n_clusters, int n_sm);
 void launch_couple_cluster(const LatticeDev& L, float4* g_next, uint8_t* flags_next, const MarkersDev& m,
                            BodyDev* bodies, const int* list, int n, bool membranes, int max_count,
                            const MeshDev& mesh, int4* boxes, int n_sm, bool interp, bool forces, bool spread,
-                           cudaStream_t st);
+                           bool programmatic, cudaStream_t st);
 // many steps of the solid-only dynamics of few membranes in one launch
 bool solid_cluster_fits(const MeshDev& mesh);
 void launch_solid_cluster(const MarkersDev& m, BodyDev* bodies, const int* list, int n, const MeshDev& mesh, double* v,

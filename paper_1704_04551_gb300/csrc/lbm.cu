@@ -41,7 +41,11 @@ constexpr int collide_min_blocks() {
   return (S == STORE_F32 && ODD) ? 9 : 10;
 }
 
-template <int S, int ODD, int GEOM, bool DENSE, bool IDX32>
+// CHAINED: launched ahead of the end of the coupling before it (lattices of at
+// most CHAINED_CELLS_MAX cells). A variant of its own: the test of an argument
+// cost the large launches 1-5 %, and the wait after the populations' loads,
+// which the coupling leaves alone, 6 % (FP16 at 256^3: 186 -> 198 us).
+template <int S, int ODD, int GEOM, bool DENSE, bool IDX32, bool CHAINED>
 __global__ void __launch_bounds__(COLLIDE_THREADS, (collide_min_blocks<S, ODD>())) k_collide(LatticeDev L, const RowInfo* __restrict__ rows,
                                                                 unsigned n_cells) {
   const unsigned t = blockIdx.x * (unsigned)COLLIDE_THREADS + threadIdx.x;
@@ -49,6 +53,10 @@ __global__ void __launch_bounds__(COLLIDE_THREADS, (collide_min_blocks<S, ODD>()
   const unsigned r = divide(t, L.by_nx);
   const int x = (int)(t - r * (unsigned)L.nx);
   const RowInfo R = rows[r];
+  if constexpr (CHAINED) {
+    await_predecessor();
+    dependents_may_launch();
+  }
   // In the neighbour-addressed (odd) step, rows without solid neighbours
   // (all but a ring of rows along walls) skip the bounce-back tests; few warps
   // lie in two rows of different kinds. (The even step reads and
@@ -226,7 +234,7 @@ namespace {
 inline unsigned blocks_for(int n) { return (unsigned)((n + 255) / 256); }
 
 template <int S, int GEOM>
-void launch_collide_g(const LatticeDev& L, const RowInfo* rows, int n_rows, bool odd, bool dense, cudaStream_t st) {
+void launch_collide_g(const LatticeDev& L, const RowInfo* rows, int n_rows, bool odd, bool dense, bool early, cudaStream_t st) {
   const unsigned n_cells = (unsigned)n_rows * (unsigned)L.nx;  // <= N < 2^31
   const unsigned block = COLLIDE_THREADS, grid = (n_cells + block - 1) / block;
   // 32-bit element offsets in the odd step while 19 N < 2^32 (a build with
@@ -237,23 +245,29 @@ void launch_collide_g(const LatticeDev& L, const RowInfo* rows, int n_rows, bool
 #else
   const bool idx32 = (unsigned long long)Q * (unsigned long long)L.N < (1ull << 32);
 #endif
-  if (odd && idx32) {
-    if (dense) k_collide<S, 1, GEOM, true, true><<<grid, block, 0, st>>>(L, rows, n_cells);
-    else k_collide<S, 1, GEOM, false, true><<<grid, block, 0, st>>>(L, rows, n_cells);
+  auto launch = [&](auto kernel) { launch_after(kernel, grid, block, 0, st, early, L, rows, n_cells); };
+  if (early) {  // (a small lattice: 32-bit offsets)
+    if (odd && dense) launch(k_collide<S, 1, GEOM, true, true, true>);
+    else if (odd) launch(k_collide<S, 1, GEOM, false, true, true>);
+    else if (dense) launch(k_collide<S, 0, GEOM, true, false, true>);
+    else launch(k_collide<S, 0, GEOM, false, false, true>);
+  } else if (odd && idx32) {
+    if (dense) launch(k_collide<S, 1, GEOM, true, true, false>);
+    else launch(k_collide<S, 1, GEOM, false, true, false>);
   } else if (odd) {
-    if (dense) k_collide<S, 1, GEOM, true, false><<<grid, block, 0, st>>>(L, rows, n_cells);
-    else k_collide<S, 1, GEOM, false, false><<<grid, block, 0, st>>>(L, rows, n_cells);
+    if (dense) launch(k_collide<S, 1, GEOM, true, false, false>);
+    else launch(k_collide<S, 1, GEOM, false, false, false>);
   } else {
-    if (dense) k_collide<S, 0, GEOM, true, false><<<grid, block, 0, st>>>(L, rows, n_cells);
-    else k_collide<S, 0, GEOM, false, false><<<grid, block, 0, st>>>(L, rows, n_cells);
+    if (dense) launch(k_collide<S, 0, GEOM, true, false, false>);
+    else launch(k_collide<S, 0, GEOM, false, false, false>);
   }
 }
 template <int S>
-void launch_collide_s(const LatticeDev& L, const RowInfo* rows, int n_rows, bool odd, bool dense, cudaStream_t st) {
+void launch_collide_s(const LatticeDev& L, const RowInfo* rows, int n_rows, bool odd, bool dense, bool early, cudaStream_t st) {
   switch (L.geometry) {
-    case GEOM_PERIODIC: launch_collide_g<S, GEOM_PERIODIC>(L, rows, n_rows, odd, dense, st); break;
-    case GEOM_YWALLS: launch_collide_g<S, GEOM_YWALLS>(L, rows, n_rows, odd, dense, st); break;
-    default: launch_collide_g<S, GEOM_TUBE>(L, rows, n_rows, odd, dense, st); break;
+    case GEOM_PERIODIC: launch_collide_g<S, GEOM_PERIODIC>(L, rows, n_rows, odd, dense, early, st); break;
+    case GEOM_YWALLS: launch_collide_g<S, GEOM_YWALLS>(L, rows, n_rows, odd, dense, early, st); break;
+    default: launch_collide_g<S, GEOM_TUBE>(L, rows, n_rows, odd, dense, early, st); break;
   }
 }
 template <int S, int GEOM>
@@ -283,13 +297,13 @@ void launch_export_s(const LatticeDev& L, bool odd_next, double* out, cudaStream
 }
 }  // namespace
 
-void launch_collide(const LatticeDev& L, const RowInfo* rows, int n_rows, int storage, bool odd, bool dense,
+void launch_collide(const LatticeDev& L, const RowInfo* rows, int n_rows, int storage, bool odd, bool dense, bool early,
                     cudaStream_t st) {
   if (n_rows == 0) return;
   switch (storage) {
-    case STORE_F32: launch_collide_s<STORE_F32>(L, rows, n_rows, odd, dense, st); break;
-    case STORE_F16: launch_collide_s<STORE_F16>(L, rows, n_rows, odd, dense, st); break;
-    default: launch_collide_s<STORE_BF16>(L, rows, n_rows, odd, dense, st); break;
+    case STORE_F32: launch_collide_s<STORE_F32>(L, rows, n_rows, odd, dense, early, st); break;
+    case STORE_F16: launch_collide_s<STORE_F16>(L, rows, n_rows, odd, dense, early, st); break;
+    default: launch_collide_s<STORE_BF16>(L, rows, n_rows, odd, dense, early, st); break;
   }
 }
 

@@ -106,7 +106,10 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(CLUSTER_THREAD
     A.forces = A.spread = true;
   } else {
     const ChunkStep st = chunk_step(C, s);
-    if (!st.active) return;
+    if (!st.active) {
+      await_predecessor();  // a kernel's end stands for its predecessors'
+      return;
+    }
     second = (s & 1) != 0;  // chunks are even: parity and buffers go with s
     A.interp = true;
     A.forces = A.spread = !st.last;
@@ -237,18 +240,25 @@ __global__ void __launch_bounds__(LANE_THREADS, 1) k_interpolate_bl(const CaseDe
 // launch per geometry present.
 // 10 resident blocks per SM for the even step, 9 for the odd one, as for the
 // single-lattice collide (64-case stream: 17,610 -> 18,150 MLUPS against 6).
-template <int ODD, int GEOM>
+template <int ODD, int GEOM, bool CHAINED>
 __global__ void __launch_bounds__(SERVE_COLLIDE, ODD ? 9 : 10)
     k_collide_b(const CaseDev* cases, const Item* items, int s) {
   const Item it = items[blockIdx.x];
   const CaseDev& C = cases[it.c];
   const unsigned t = (unsigned)it.i * (unsigned)SERVE_COLLIDE + threadIdx.x;
   const ChunkStep st = chunk_step(C, s);
-  if (!st.active || t >= C.n_cells) return;
+  if (!st.active || t >= C.n_cells) {
+    if constexpr (CHAINED) await_predecessor();  // a kernel's end stands for its predecessors'
+    return;
+  }
   const LatticeDev L = case_lattice(C, ODD == 1 && C.clustered != 0);
   const unsigned r = divide(t, L.by_nx);
   const int x = (int)(t - r * (unsigned)L.nx);
   const RowInfo R = C.rows[r];
+  if constexpr (CHAINED) {  // launched ahead of the coupling's end
+    await_predecessor();
+    dependents_may_launch();
+  }
   // served lattices are far below 2^32 / 19 cells (checked at submission)
   if (st.last) collide_cell<STORE_F32, ODD, GEOM, true, ODD == 1>(L, R, x);
   else collide_cell<STORE_F32, ODD, GEOM, false, ODD == 1>(L, R, x);
@@ -445,19 +455,27 @@ int admit(ibm_lbm_server_t* s) {
 
 // The collision of step `step` of the chunk for all cases, one launch per
 // geometry present.
-void launch_collide_b(ibm_lbm_server_t* s, bool odd, int step) {
+// early: right after a coupling kernel (await_predecessor).
+void launch_collide_b(ibm_lbm_server_t* s, bool odd, int step, bool early) {
   for (int g = 0; g < 3; ++g) {
     const int first = s->geom_first[g], n_items = s->geom_first[g + 1] - first;
     if (n_items == 0) continue;
     const unsigned block = SERVE_COLLIDE, grid = (unsigned)n_items;
     const Item* items = s->d_rows + first;
-    switch (g * 2 + (odd ? 1 : 0)) {
-      case 0: k_collide_b<0, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
-      case 1: k_collide_b<1, GEOM_PERIODIC><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
-      case 2: k_collide_b<0, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
-      case 3: k_collide_b<1, GEOM_YWALLS><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
-      case 4: k_collide_b<0, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
-      default: k_collide_b<1, GEOM_TUBE><<<grid, block, 0, s->stream>>>(s->d_cases, items, step); break;
+    auto launch = [&](auto kernel) { launch_after(kernel, grid, block, 0, s->stream, early, s->d_cases, items, step); };
+    switch (g * 4 + (odd ? 2 : 0) + (early ? 1 : 0)) {
+      case 0: launch(k_collide_b<0, GEOM_PERIODIC, false>); break;
+      case 1: launch(k_collide_b<0, GEOM_PERIODIC, true>); break;
+      case 2: launch(k_collide_b<1, GEOM_PERIODIC, false>); break;
+      case 3: launch(k_collide_b<1, GEOM_PERIODIC, true>); break;
+      case 4: launch(k_collide_b<0, GEOM_YWALLS, false>); break;
+      case 5: launch(k_collide_b<0, GEOM_YWALLS, true>); break;
+      case 6: launch(k_collide_b<1, GEOM_YWALLS, false>); break;
+      case 7: launch(k_collide_b<1, GEOM_YWALLS, true>); break;
+      case 8: launch(k_collide_b<0, GEOM_TUBE, false>); break;
+      case 9: launch(k_collide_b<0, GEOM_TUBE, true>); break;
+      case 10: launch(k_collide_b<1, GEOM_TUBE, false>); break;
+      default: launch(k_collide_b<1, GEOM_TUBE, true>); break;
     }
   }
 }
@@ -548,14 +566,23 @@ int rebuild(ibm_lbm_server_t* s) {
   const bool lanes = s->n_groups < LANE_MAX_GROUPS;
   SCUDA(s, cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal));
   const int n_cr = (int)cl_rigid.size(), n_cm = (int)cl_membranes.size();
-  auto couple = [&](int step) {
-    if (n_cr)
-      k_couple_cluster_b<0><<<n_cr * CLUSTER, CLUSTER_THREADS, CLUSTER_SHARE, s->stream>>>(s->d_cases, s->d_cl_rigid, step);
-    if (n_cm)
-      k_couple_cluster_b<1>
-          <<<n_cm * CLUSTER, CLUSTER_THREADS, CLUSTER_SHARE, s->stream>>>(s->d_cases, s->d_cl_membranes, step);
-  };
   const bool separate = n_cr + n_cm == 0 || s->n_groups + s->n_rigid + s->n_membranes > 0;
+  // one collision and one coupling kernel a step of few cells: they start ahead
+  // of one another (as api.cu, chained)
+  int geometries = 0;
+  for (int gm = 0; gm < 3; ++gm) geometries += s->geom_first[gm + 1] > s->geom_first[gm];
+  size_t cells = 0;
+  for (const CaseDev& C : s->h_cases) cells += C.n_cells;
+  const bool chained = !separate && geometries == 1 && cells <= (size_t)CHAINED_CELLS_MAX && (n_cr > 0) != (n_cm > 0);
+  auto couple = [&](int step) {
+    const bool ahead = chained && step >= 0;
+    if (n_cr)
+      launch_after(k_couple_cluster_b<0>, n_cr * CLUSTER, CLUSTER_THREADS, CLUSTER_SHARE, s->stream, ahead, s->d_cases,
+                   s->d_cl_rigid, step);
+    if (n_cm)
+      launch_after(k_couple_cluster_b<1>, n_cm * CLUSTER, CLUSTER_THREADS, CLUSTER_SHARE, s->stream, ahead, s->d_cases,
+                   s->d_cl_membranes, step);
+  };
   if (n_cr + n_cm) k_chunk_begin<<<n, 256, 0, s->stream>>>(s->d_cases);
   couple(-1);
   for (int step = 0; step < s->cfg.chunk_steps; ++step) {
@@ -567,7 +594,7 @@ int rebuild(ibm_lbm_server_t* s) {
       k_spread_bl<<<s->n_groups, LANE_THREADS, SPREAD_LANES_SMEM, s->stream>>>(s->d_cases, s->d_groups, step);
     else if (s->n_groups)
       k_spread_b<<<s->n_groups, SERVE_XFER_THREADS, SPREAD_SMEM, s->stream>>>(s->d_cases, s->d_groups, step);
-    launch_collide_b(s, step & 1, step);
+    launch_collide_b(s, step & 1, step, chained);
     if (s->n_groups && lanes)
       k_interpolate_bl<<<s->n_groups, LANE_THREADS, INTERP_SMEM, s->stream>>>(s->d_cases, s->d_groups, step);
     else if (s->n_groups)
