@@ -217,7 +217,7 @@ int cluster_box_cells(size_t fixed_words, int n_clusters, int n_sm) {
   const int per_sm = std::max(1, (n_clusters * CLUSTER + n_sm - 1) / n_sm);
   const size_t share = std::min<size_t>(CLUSTER_SMEM_MAX, (size_t)(CLUSTER_SMEM_SM / std::min(per_sm, CLUSTER_PER_SM)) - 5 * 1024);
   if (4 * fixed_words + 12 * 1024 > share) return 0;
-  return (int)std::min<size_t>(CLUSTER_BOX_MAX, (share / 4 - fixed_words) / 3);
+  return (int)std::min<size_t>(CLUSTER_BOX_MAX, (share / 4 - fixed_words) / 3) & ~3;  // (cleared 16 bytes at a time)
 }
 
 void launch_couple_cluster(const LatticeDev& L, float4* g_next, uint8_t* flags_next, const MarkersDev& m,

@@ -48,6 +48,8 @@ constexpr int CLUSTER_WORKERS = 224;     // threads that work on markers (7 warp
 constexpr int CLUSTER_THREADS = CLUSTER_WORKERS + 32;
 constexpr int CLUSTER_MAX_COUNT = 4096;  // markers per body
 constexpr int CLUSTER_BOX_MAX = 12288;   // cells of a block's box
+constexpr int CLUSTER_UNION_MAX = 1 << 18;  // cells of a body's box (its blocks' boxes together)
+constexpr int CLUSTER_CLEAR_AHEAD = 1024;   // cells a block's last warp clears while the others gather
 constexpr int CLUSTER_PER_SM = 2;        // resident blocks the registers are sized for
 constexpr int CLUSTER_SMEM_SM = 227 * 1024, CLUSTER_SMEM_MAX = 220 * 1024;
 // dynamic shared memory of a block at CLUSTER_PER_SM blocks
@@ -75,7 +77,6 @@ struct ClusterShare {
   unsigned qmax[CLUSTER];           // largest membrane force contribution
   int lo_s[3], hi_s[3];             // own bounds
   unsigned fmax_s, redo_max;
-  int zero;
   RigidPrep prep[3];                // per component (rigid_prepare)
   double quat[4];
   double total[6];                  // force and torque of all blocks
@@ -195,7 +196,9 @@ __device__ __forceinline__ void rotation_row(const double* q, int a, double r[3]
   else { r[0] = 2 * (x * z - w * y); r[1] = 2 * (y * z + w * x); r[2] = 1 - 2 * (x * x + y * y); }
 }
 
-// Smallest box around the boxes lo[r], dims[r] of the blocks (dims.w != 0).
+// Smallest box around the boxes lo[r], dims[r] of the blocks (dims.w != 0), at
+// most CLUSTER_UNION_MAX cells: above that (markers of one body far apart), or
+// with no box at all, dims.w = 0.
 __device__ __forceinline__ void union_box(const int4* lo, const int4* dims, int4& ulo, int4& udims) {
   int l[3] = {INT_MAX, INT_MAX, INT_MAX}, h[3] = {INT_MIN, INT_MIN, INT_MIN};
 #pragma unroll
@@ -205,27 +208,33 @@ __device__ __forceinline__ void union_box(const int4* lo, const int4* dims, int4
     l[0] = min(l[0], a.x); l[1] = min(l[1], a.y); l[2] = min(l[2], a.z);
     h[0] = max(h[0], a.x + d.x); h[1] = max(h[1], a.y + d.y); h[2] = max(h[2], a.z + d.z);
   }
-  const bool any = h[0] > l[0];
+  const long long ex = (long long)h[0] - l[0], ey = (long long)h[1] - l[1], ez = (long long)h[2] - l[2];
+  constexpr long long most = CLUSTER_UNION_MAX;
+  const bool ok = ex > 0 && ex <= most && ey <= most && ez <= most && ex * ey <= most && ex * ey * ez <= most;
   ulo = make_int4(l[0], l[1], l[2], 0);
-  udims = any ? make_int4(h[0] - l[0], h[1] - l[1], h[2] - l[2], 1) : make_int4(0, 0, 0, 0);
+  udims = ok ? make_int4((int)ex, (int)ey, (int)ez, 1) : make_int4(0, 0, 0, 0);
 }
 
-// Visits the cells of the rows of a box that are block `rank`'s, row by row:
-// f(cell index in the lattice, unwrapped x, y, z, mask of the blocks whose
-// boxes meet the row). Rows no block's box meets, and solid ones, are skipped.
+// Cells of the rows of a body's box that are block `rank`'s (every eighth).
+__device__ __forceinline__ int cluster_share(int4 udims, int rank) {
+  const int nrows = udims.y * udims.z;
+  return nrows > rank ? (nrows - rank + CLUSTER - 1) / CLUSTER * udims.x : 0;
+}
+
+// Visits those cells, thread t of n: f(cell index in the lattice, unwrapped x,
+// y, z, mask of the blocks whose boxes meet the row). Rows no block's box meets,
+// and solid ones, are skipped. The cells are numbered through, so that rows a
+// little longer than a warp leave no lanes idle.
 template <int GEOM, class F>
-__device__ __forceinline__ void cluster_rows(const LatticeDev& L, const int4* lo, const int4* dims, int rank, int warp,
-                                             int nwarps, F&& f) {
-  int4 ulo, ud;
-  union_box(lo, dims, ulo, ud);
-  if (ud.w == 0) return;
-  const int nrows = ud.y * ud.z;
-  const RowSweep sw = row_sweep(ud.x);
-  const float inv_dy = 1.0f / (float)ud.y;
+__device__ __forceinline__ void cluster_cells(const LatticeDev& L, const int4* lo, const int4* dims, int4 ulo, int4 ud,
+                                              int rank, int t, int n, F&& f) {
+  const int total = cluster_share(ud, rank);
+  const float inv_dx = 1.0f / (float)ud.x, inv_dy = 1.0f / (float)ud.y;
   const int xw0 = wrapi(ulo.x, L.nx);
-  for (int r = rank + CLUSTER * (warp * sw.rpw + sw.sub); sw.on && r < nrows; r += CLUSTER * nwarps * sw.rpw) {
-    int iy, iz;
-    row_yz(r, ud.y, inv_dy, iy, iz);
+  for (int c = t; c < total; c += n) {
+    int i, ax, iy, iz;
+    row_yz(c, ud.x, inv_dx, ax, i);  // c = ax + ud.x i (exact: c < 2^20)
+    row_yz(rank + CLUSTER * i, ud.y, inv_dy, iy, iz);
     int y = ulo.y + iy, z = ulo.z + iz;
     unsigned mask = 0u;
 #pragma unroll
@@ -235,8 +244,7 @@ __device__ __forceinline__ void cluster_rows(const LatticeDev& L, const int4* lo
     if (mask == 0u) continue;
     const int uy = y, uz = z;
     if (!fluid_row<GEOM>(L, y, z)) continue;
-    const size_t row = (size_t)L.nx * (y + L.ny * z);
-    for (int ax = sw.ax; ax < ud.x; ax += 32) f(row + box_x(xw0, ax, L.nx), ulo.x + ax, uy, uz, mask);
+    f((size_t)L.nx * (y + L.ny * z) + box_x(xw0, ax, L.nx), ulo.x + ax, uy, uz, mask);
   }
 }
 
@@ -389,7 +397,6 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
   }
   if (tid == 0) {
     S.fmax_s = S.redo_max = 0u;
-    S.zero = 0;
   }
   if (tid < CLUSTER) {
     S.old_lo[tid] = A.boxes[2 * tid];
@@ -422,13 +429,18 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
     await_predecessor();
     dependents_may_launch();
   }
-  if (!worker && A.interp) {
-    // the last warp clears the force density and flags that the finished
-    // collision read
-    cluster_rows<GEOM>(L, S.old_lo, S.old_dims, rank, 0, 1,
-                       [&](size_t gi, int, int, int, unsigned) { L.g[gi] = make_float4(0.f, 0.f, 0.f, 0.f); });
-    if (boxed) mark_box_tiles<GEOM>(L, S.old_lo[rank], S.old_dims[rank], lane, 32, 0);
-  }
+  // The force density and flags that the finished collision read are cleared by
+  // the last warp while the others gather (a small body), or by all while the
+  // blocks wait for one another.
+  int4 old_lo, old_dims;
+  union_box(S.old_lo, S.old_dims, old_lo, old_dims);
+  const bool clears = A.interp && old_dims.w != 0, ahead = cluster_share(old_dims, 0) <= CLUSTER_CLEAR_AHEAD;
+  auto clear_consumed = [&](int t, int n_threads) {
+    cluster_cells<GEOM>(L, S.old_lo, S.old_dims, old_lo, old_dims, rank, t, n_threads,
+                        [&](size_t gi, int, int, int, unsigned) { L.g[gi] = make_float4(0.f, 0.f, 0.f, 0.f); });
+    if (boxed) mark_box_tiles<GEOM>(L, S.old_lo[rank], S.old_dims[rank], t, n_threads, 0);
+  };
+  if (!worker && clears && ahead) clear_consumed(lane, 32);
   if (worker) {
     // (the next pass's marker is loaded while this one is gathered)
     double Xnext = 0.0, arm_next[3] = {0, 0, 0};
@@ -533,6 +545,7 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
   }
   cl.barrier_wait();  // every block has started and has read the origin
   if (!A.forces) {
+    if (clears && !ahead) clear_consumed(tid, CLUSTER_THREADS);
     if (KIND == 1) {
       __syncthreads();
       for (int i = tid; i < 3 * n; i += CLUSTER_THREADS) {
@@ -666,9 +679,9 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
   const long long ex = (long long)S.hi_s[0] - S.lo_s[0] + 4, ey = (long long)S.hi_s[1] - S.lo_s[1] + 4,
                   ez = (long long)S.hi_s[2] - S.lo_s[2] + 4;
   // each extent below cap before the products: no overflow
-  const bool fits = n > 0 && ex <= A.cap && ey <= A.cap && ez <= A.cap && ex * ey <= A.cap && ex * ey * ez <= A.cap;
+  const bool own_fits = n > 0 && ex <= A.cap && ey <= A.cap && ez <= A.cap && ex * ey <= A.cap && ex * ey * ez <= A.cap;
   const int4 lo2 = make_int4(S.lo_s[0] - 1, S.lo_s[1] - 1, S.lo_s[2] - 1, 0);
-  const int4 dims2 = make_int4(fits ? (int)ex : 0, fits ? (int)ey : 0, fits ? (int)ez : 0, fits ? 1 : 0);
+  const int4 dims2 = make_int4(own_fits ? (int)ex : 0, own_fits ? (int)ey : 0, own_fits ? (int)ez : 0, own_fits ? 1 : 0);
   const int vol = dims2.x * dims2.y * dims2.z;
   if (tid < CLUSTER) {
     ClusterShare* R = cl.map_shared_rank(&S, tid);
@@ -676,18 +689,23 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
     R->dims[rank] = dims2;
     R->fmax[rank] = S.fmax_s;
   }
-  for (int i = tid; i < 3 * vol; i += CLUSTER_THREADS) ibox[i] = 0;
+  for (int i = tid; i < (3 * vol + 3) / 4; i += CLUSTER_THREADS)  // (cap is a multiple of 4)
+    reinterpret_cast<int4*>(ibox)[i] = make_int4(0, 0, 0, 0);
   LatticeDev Ln = L;
   Ln.g = A.g_next;
   Ln.flags = A.flags_next;
   __syncthreads();
   cl.barrier_arrive();
-  if (fits) mark_box_tiles<GEOM>(Ln, lo2, dims2);
+  if (clears && !ahead) clear_consumed(tid, CLUSTER_THREADS);
   cl.barrier_wait();  // boxes, forces and sums of all blocks
+  int4 ulo, udims;
+  union_box(S.lo, S.dims, ulo, udims);
+  const bool fits = own_fits && udims.w != 0;  // (markers of one body far apart: no box)
   if (tid == 0) {  // (every block has read the old ones)
     A.boxes[2 * rank] = lo2;
-    A.boxes[2 * rank + 1] = dims2;
+    A.boxes[2 * rank + 1] = make_int4(dims2.x, dims2.y, dims2.z, fits ? 1 : 0);
   }
+  if (fits) mark_box_tiles<GEOM>(Ln, lo2, dims2);
   unsigned fbits = 0u;
 #pragma unroll
   for (int r = 0; r < CLUSTER; ++r) fbits = max(fbits, S.fmax[r]);
@@ -744,18 +762,21 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
     if (rank == 0) update_body();
   }
   cl.barrier_wait();  // the boxes are complete
-  if (any_force) {
+  if (any_force && udims.w != 0) {
     const float inv = 1.0f / Sc;
-    cluster_rows<GEOM>(L, S.lo, S.dims, rank, warp, CLUSTER_THREADS / 32, [&](size_t gi, int ux, int uy, int uz, unsigned mask) {
+    cluster_cells<GEOM>(L, S.lo, S.dims, ulo, udims, rank, tid, CLUSTER_THREADS, [&](size_t gi, int ux, int uy, int uz, unsigned mask) {
       int q[3] = {0, 0, 0}, lo4[3] = {0, 0, 0};
 #pragma unroll
       for (int r = 0; r < CLUSTER; ++r) {
         const int4 lo = S.lo[r], d = S.dims[r];
         const int ox = ux - lo.x, v = d.x * d.y * d.z;
-        const bool in = ((mask >> r) & 1u) != 0u && (unsigned)ox < (unsigned)d.x;
-        const int* p = in ? cl.map_shared_rank(ibox, r) + (ox + d.x * ((uy - lo.y) + d.y * (uz - lo.z))) : &S.zero;
-        const int st = in ? v : 0;
-        const int t[3] = {p[0], p[st], p[2 * st]};
+        int t[3] = {0, 0, 0};
+        if (((mask >> r) & 1u) != 0u && (unsigned)ox < (unsigned)d.x) {
+          const int* p = cl.map_shared_rank(ibox, r) + (ox + d.x * ((uy - lo.y) + d.y * (uz - lo.z)));
+          t[0] = p[0];
+          t[1] = p[v];
+          t[2] = p[2 * v];
+        }
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
           if (wide) {  // eight sums below 2^30: their high parts and low 4 bits apart

@@ -4,7 +4,8 @@ as the stage interface, which spreads and interpolates with the separate
 kernels. Sizes at the edges of the split: fewer markers than blocks, one more
 than a multiple, the largest count a body may have, bodies across periodic
 boundaries and against a wall, a body whose boxes do not fit shared memory
-(global atomics), several bodies that share cells, odd starts and single
+(global atomics), one whose parts are too far apart for a common box, one large
+enough that all warps clear its box, several bodies that share cells, odd starts and single
 steps.
 
 Tolerances as in test_gpu_parity.py: both paths do the same arithmetic on
@@ -48,6 +49,8 @@ CASES = {
     'across_boundaries': (PER, [(300, (0.5, 27.5, 1.0), (5, 4, 3), False)]),
     'against_a_wall': (WALL, [(812, (16, 2.0, 15), (6, 3, 3), True)]),
     'direct_and_tether_sharing_cells': (TUBE, [(812, (12, 14, 15), (6, 4, 4), True), (400, (18, 15, 14), (4, 4, 4), False)]),
+    'eighths_far_apart': (WIDE, [(8, (48, 45, 44), (70, 60, 60), False)]),
+    'large_body': (WIDE, [(812, (40, 45, 44), (19, 9, 8), False)]),
     'boxes_too_large': (WIDE, [(640, (48, 45, 44), (40, 38, 37), False)]),
 }
 
