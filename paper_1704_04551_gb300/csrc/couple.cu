@@ -148,7 +148,7 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
       const int ox = st.bx - lo.x, oy = st.by - lo.y, oz = st.bz - lo.z - z0;
       float3 u;
       if (in_box && ox >= 0 && oy >= 0 && oz >= 0 && ox + 4 <= dims.x && oy + 4 <= dims.y && oz + 4 <= dz)
-        u = box_gather(vbox, dims, st, ox, oy, oz);
+        u = box_gather<false>(vbox, dims, st, ox, oy, oz);
       else if (in_box && dims.w == 2)  // in another slab (the box holds every stencil)
         return;
       else  // no box, or the stencil outside it

@@ -399,13 +399,14 @@ __device__ __forceinline__ void scatter_marker(int* ibox, int vol, int4 dims, in
   axis_weights(fx, wx);
   axis_weights(fy, wy);
   axis_weights(fz, wz);
-  float ax_[4], ay_[4], az_[4];
+  F32x2 axy[4];
+  float az_[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) {
-    ax_[a] = Fx * wx[a];
-    ay_[a] = Fy * wx[a];
+    axy[a] = pack2(Fx * wx[a], Fy * wx[a]);
     az_[a] = Fz * wx[a];
   }
+  const F32x2 bias = pack2(12582912.0f, 12582912.0f);  // as fixed_mul
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     if (CLIPPED && (c < c0 || c >= c1)) continue;
@@ -415,8 +416,10 @@ __device__ __forceinline__ void scatter_marker(int* ibox, int vol, int4 dims, in
       int* p = ibox + li0 + dims.x * (b + dims.y * c);
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        atomicAdd(p + a, fixed_mul(ax_[a], wyz));
-        atomicAdd(p + vol + a, fixed_mul(ay_[a], wyz));
+        float qx, qy;
+        unpack2(fma2(axy[a], pack2(wyz, wyz), bias), qx, qy);
+        atomicAdd(p + a, __float_as_int(qx) - 0x4B400000);
+        atomicAdd(p + vol + a, __float_as_int(qy) - 0x4B400000);
         atomicAdd(p + 2 * vol + a, fixed_mul(az_[a], wyz));
       }
     }
@@ -483,25 +486,51 @@ __device__ __forceinline__ void velocity_box_async(const LatticeDev& L, int4 lo,
 }
 __device__ __forceinline__ void velocity_box_wait() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
 
+// PACKED: the x and y sums in packed FP32 pairs (the same bits; 512^3 channel:
+// interpolation 1.574 -> 1.505 ms); not in the fused kernel, whose 64 registers
+// the pairs overflow (256^3 step 0.819 -> 0.842 ms).
 // Velocity at a marker whose 4^3 stencil lies in the box (first node at
 // box offsets ox, oy, oz), gathered from the shared-memory box.
+template <bool PACKED = true>
 __device__ __forceinline__ float3 box_gather(const float4* vbox, int4 dims, const Stencil& st, int ox, int oy, int oz) {
   const int li0 = ox + dims.x * (oy + dims.y * oz);
-  float ux = 0.f, uy = 0.f, uz = 0.f;
+  if constexpr (!PACKED) {
+    float ux = 0.f, uy = 0.f, uz = 0.f;
+#pragma unroll
+    for (int c = 0; c < 4; ++c)
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const float4* p = vbox + li0 + dims.x * (b + dims.y * c);
+        const float4 v0 = p[0], v1 = p[1], v2 = p[2], v3 = p[3];
+        const float rx = fmaf(st.wx[3], v3.x, fmaf(st.wx[2], v2.x, fmaf(st.wx[1], v1.x, st.wx[0] * v0.x)));
+        const float ry = fmaf(st.wx[3], v3.y, fmaf(st.wx[2], v2.y, fmaf(st.wx[1], v1.y, st.wx[0] * v0.y)));
+        const float rz = fmaf(st.wx[3], v3.z, fmaf(st.wx[2], v2.z, fmaf(st.wx[1], v1.z, st.wx[0] * v0.z)));
+        const float wyz = st.wy[b] * st.wz[c];
+        ux = fmaf(wyz, rx, ux);
+        uy = fmaf(wyz, ry, uy);
+        uz = fmaf(wyz, rz, uz);
+      }
+    return make_float3(ux, uy, uz);
+  }
+  F32x2 w[4], uxy = pack2(0.f, 0.f);
+#pragma unroll
+  for (int a = 0; a < 4; ++a) w[a] = pack2(st.wx[a], st.wx[a]);
+  float uz = 0.f;
 #pragma unroll
   for (int c = 0; c < 4; ++c)
 #pragma unroll
     for (int b = 0; b < 4; ++b) {
       const float4* p = vbox + li0 + dims.x * (b + dims.y * c);
       const float4 v0 = p[0], v1 = p[1], v2 = p[2], v3 = p[3];
-      const float rx = fmaf(st.wx[3], v3.x, fmaf(st.wx[2], v2.x, fmaf(st.wx[1], v1.x, st.wx[0] * v0.x)));
-      const float ry = fmaf(st.wx[3], v3.y, fmaf(st.wx[2], v2.y, fmaf(st.wx[1], v1.y, st.wx[0] * v0.y)));
+      const F32x2 rxy = fma2(w[3], pack2(v3.x, v3.y),
+                             fma2(w[2], pack2(v2.x, v2.y), fma2(w[1], pack2(v1.x, v1.y), mul2(w[0], pack2(v0.x, v0.y)))));
       const float rz = fmaf(st.wx[3], v3.z, fmaf(st.wx[2], v2.z, fmaf(st.wx[1], v1.z, st.wx[0] * v0.z)));
       const float wyz = st.wy[b] * st.wz[c];
-      ux = fmaf(wyz, rx, ux);
-      uy = fmaf(wyz, ry, uy);
+      uxy = fma2(pack2(wyz, wyz), rxy, uxy);
       uz = fmaf(wyz, rz, uz);
     }
+  float ux, uy;
+  unpack2(uxy, ux, uy);
   return make_float3(ux, uy, uz);
 }
 
