@@ -171,6 +171,13 @@ __device__ __forceinline__ F32x2 mul2(F32x2 a, F32x2 b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
   return r;
 }
+__device__ __forceinline__ F32x2 add2(F32x2 a, F32x2 b) {
+  F32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F32x2 both(float a) { return pack2(a, a); }
+__device__ __forceinline__ F32x2 sub2(F32x2 a, F32x2 b) { return fma2(b, both(-1.0f), a); }
 
 // ---- population storage ---------------------------------------------------
 template <int S> struct Store;

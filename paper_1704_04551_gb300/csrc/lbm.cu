@@ -70,6 +70,18 @@ __global__ void __launch_bounds__(COLLIDE_THREADS, (collide_min_blocks<S, ODD>()
   collide_cell<S, ODD, GEOM, DENSE, IDX32>(L, R, x);
 }
 
+// The even step in half-precision storage on lattices with even rows, two cells
+// per thread (collide_pair_even).
+constexpr int PAIR_MIN_BLOCKS = 7;
+template <int S, int GEOM, bool DENSE>
+__global__ void __launch_bounds__(COLLIDE_THREADS, PAIR_MIN_BLOCKS) k_collide_pair(LatticeDev L, const RowInfo* __restrict__ rows,
+                                                                      unsigned n_cells) {
+  const unsigned t = 2u * (blockIdx.x * (unsigned)COLLIDE_THREADS + threadIdx.x);
+  if (t >= n_cells) return;
+  const unsigned r = divide(t, L.by_nx);
+  collide_pair_even<S, GEOM, DENSE>(L, rows[r], (int)(t - r * (unsigned)L.nx));
+}
+
 // Equilibrium initialisation from the moments in uw (ux, uy, uz, rho - 1).
 template <int S, int GEOM>
 __global__ void k_init_equilibrium(LatticeDev L) {
@@ -258,6 +270,14 @@ void launch_collide_g(const LatticeDev& L, const RowInfo* rows, int n_rows, bool
     if (dense) launch(k_collide<S, 1, GEOM, true, false, false>);
     else launch(k_collide<S, 1, GEOM, false, false, false>);
   } else {
+    if constexpr (S != STORE_F32) {
+      if (L.nx % 2 == 0) {
+        const unsigned pairs = (n_cells / 2 + block - 1) / block;
+        if (dense) launch_after(k_collide_pair<S, GEOM, true>, pairs, block, 0, st, false, L, rows, n_cells);
+        else launch_after(k_collide_pair<S, GEOM, false>, pairs, block, 0, st, false, L, rows, n_cells);
+        return;
+      }
+    }
     if (dense) launch(k_collide<S, 0, GEOM, true, false, false>);
     else launch(k_collide<S, 0, GEOM, false, false, false>);
   }

@@ -242,4 +242,121 @@ __device__ __forceinline__ void collide_cell(const LatticeDev& L, const RowInfo&
 }
 
 
+// Two neighbouring fluid cells (x even, x + 1) of the local (even) step in
+// half-precision storage: 4-byte loads and stores, and the arithmetic of
+// relax_cell's half-precision branch in packed FP32 pairs. The single-cell
+// kernel keeps ~48 KB of loads in flight on an SM, less than the memory's
+// latency times its rate; a thread of this one has twice the bytes and half
+// the instructions per cell. Needs an even nx (cell pairs aligned to 4 bytes).
+template <int S, int GEOM, bool DENSE>
+__device__ __forceinline__ void collide_pair_even(const LatticeDev& L, const RowInfo& R, int x) {
+  static_assert(S != STORE_F32, "half-precision storage");
+  using P = Pop<S>;
+  using T = typename P::T;
+  T* A = reinterpret_cast<T*>(L.pop);
+  const int idx = R.base + x;
+  const size_t N = (size_t)L.N;
+  F32x2 d[Q];
+#pragma unroll
+  for (int j = 0; j < Q; ++j) {
+    const unsigned w = *reinterpret_cast<const unsigned*>(A + j * N + idx);
+    if constexpr (S == STORE_F16) {
+      const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w));
+      d[j] = pack2(f.x, f.y);
+    } else {
+      d[j] = pack2(__uint_as_float(w << 16), __uint_as_float(w & 0xffff0000u));
+    }
+  }
+  F32x2 drho = both(0.f), jx = both(0.f), jy = both(0.f), jz = both(0.f);
+#pragma unroll
+  for (int i = 0; i < Q; ++i) {
+    const float k = 1.0f / dev_scale(i);
+    drho = fma2(d[i], both(k), drho);
+    if (cx(i)) jx = fma2(d[i], both(cx(i) * k), jx);
+    if (cy(i)) jy = fma2(d[i], both(cy(i) * k), jy);
+    if (cz(i)) jz = fma2(d[i], both(cz(i) * k), jz);
+  }
+  F32x2 Gx = both(L.g0x), Gy = both(L.g0y), Gz = both(L.g0z);
+  const bool touched = L.flags[R.trow + (x >> TILE_X_SHIFT)] != 0;  // (a tile holds both cells)
+  if (touched) {
+    const float4 a = L.g[idx], b = L.g[idx + 1];
+    Gx = add2(Gx, pack2(a.x, b.x));
+    Gy = add2(Gy, pack2(a.y, b.y));
+    Gz = add2(Gz, pack2(a.z, b.z));
+  }
+  const F32x2 rho = add2(both(1.0f), drho);
+  float r0, r1;
+  unpack2(rho, r0, r1);
+  const F32x2 irho = pack2(1.0f / r0, 1.0f / r1);
+  const F32x2 ux = mul2(fma2(both(0.5f), Gx, jx), irho);
+  const F32x2 uy = mul2(fma2(both(0.5f), Gy, jy), irho);
+  const F32x2 uz = mul2(fma2(both(0.5f), Gz, jz), irho);
+  if (DENSE || touched) {
+    float x0, x1, y0, y1, z0, z1, e0, e1;
+    unpack2(ux, x0, x1);
+    unpack2(uy, y0, y1);
+    unpack2(uz, z0, z1);
+    unpack2(drho, e0, e1);
+    L.uw[idx] = make_float4(x0, y0, z0, e0);
+    L.uw[idx + 1] = make_float4(x1, y1, z1, e1);
+  }
+  const float om = L.omega, pre = L.guo_pre;
+  constexpr float KW = 8.0f / 9.0f;
+  const F32x2 usq15 = mul2(both(1.5f), fma2(uz, uz, fma2(uy, uy, mul2(ux, ux))));
+  const F32x2 uG = fma2(uz, Gz, fma2(uy, Gy, mul2(ux, Gx)));
+  const F32x2 om1 = both(1.0f - om);
+  const F32x2 T0 = sub2(mul2(both(om), sub2(drho, mul2(rho, usq15))), mul2(both(3.0f * pre), uG));
+  const F32x2 Aq = mul2(both((KW * 3.0f) * om), rho), Bq = mul2(both((KW * 4.5f) * om), rho);
+  const F32x2 P3 = both((KW * 3.0f) * pre), P9 = both((KW * 9.0f) * pre);
+  const F32x2 T0w = mul2(both(KW), T0);
+  // component of a direction along +-(c_x, c_y, c_z)
+  auto along = [](int i, F32x2 a, F32x2 b, F32x2 c) {
+    F32x2 s = both(0.f);
+    bool have = false;
+    auto take = [&](int k, F32x2 v) {
+      if (k == 0) return;
+      s = have ? (k > 0 ? add2(s, v) : sub2(s, v)) : (k > 0 ? v : mul2(both(-1.0f), v));
+      have = true;
+    };
+    take(cx(i), a);
+    take(cy(i), b);
+    take(cz(i), c);
+    return s;
+  };
+  auto store = [&](int slot, F32x2 v) {
+    float a, b;
+    unpack2(v, a, b);
+    unsigned w;
+    if constexpr (S == STORE_F16) {
+      const __half2 p = __floats2half2_rn(a, b);
+      w = *reinterpret_cast<const unsigned*>(&p);
+    } else {
+      const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
+      w = *reinterpret_cast<const unsigned*>(&p);
+    }
+    *reinterpret_cast<unsigned*>(A + slot * N + idx) = w;
+  };
+  store(0, fma2(om1, d[0], mul2(both(4.0f / 3.0f), T0)));
+#pragma unroll
+  for (int i = 1; i < Q; i += 2) {
+    const F32x2 cu = along(i, ux, uy, uz), cG = along(i, Gx, Gy, Gz);
+    const F32x2 even = fma2(fma2(Bq, cu, mul2(P9, cG)), cu, T0w);
+    const F32x2 odd = fma2(Aq, cu, mul2(P3, cG));
+    F32x2 p = fma2(om1, d[i], add2(even, odd)), m = fma2(om1, d[i + 1], sub2(even, odd));
+    if (GEOM == GEOM_YWALLS && cx(i) != 0 && cy(i) != 0) {
+      // half-way bounce-back at the moving walls, as in collide_cell
+      auto wall = [&](int k, F32x2 v) {
+        const int yn = R.y + cy(k);
+        if ((unsigned)yn < (unsigned)L.ny) return v;
+        const float uw = yn < 0 ? L.wall_u0 : L.wall_u1;
+        return fma2(both(-dev_scale(opp(k)) * 6.0f * wgt(k) * (float)cx(k) * uw), rho, v);
+      };
+      p = wall(i, p);
+      m = wall(i + 1, m);
+    }
+    store(opp(i), p);
+    store(opp(i + 1), m);
+  }
+}
+
 }  // namespace ibm
