@@ -70,16 +70,30 @@ __global__ void __launch_bounds__(COLLIDE_THREADS, (collide_min_blocks<S, ODD>()
   collide_cell<S, ODD, GEOM, DENSE, IDX32>(L, R, x);
 }
 
-// The even step in half-precision storage on lattices with even rows, two cells
-// per thread (collide_pair_even).
+// Half-precision storage on lattices with even rows: two cells per thread
+// (collide_pair); in the odd step rows with solid neighbours cell by cell.
+// 256^3 tube, FP16: even step 186 -> 158 us, odd 208 -> 187 us; 7 resident
+// blocks (72 registers) measured best (even: 6: 166, 8: 160 us). From
+// PAIR_CELLS_MIN fluid cells on: below, the single-cell kernel is one wave, and
+// half the threads only wait longer (60x47x33, odd: 9.0 against 10.6 us).
+constexpr unsigned PAIR_CELLS_MIN = 1u << 18;
 constexpr int PAIR_MIN_BLOCKS = 7;
-template <int S, int GEOM, bool DENSE>
+template <int S, int ODD, int GEOM, bool DENSE, bool IDX32>
 __global__ void __launch_bounds__(COLLIDE_THREADS, PAIR_MIN_BLOCKS) k_collide_pair(LatticeDev L, const RowInfo* __restrict__ rows,
                                                                       unsigned n_cells) {
   const unsigned t = 2u * (blockIdx.x * (unsigned)COLLIDE_THREADS + threadIdx.x);
   if (t >= n_cells) return;
   const unsigned r = divide(t, L.by_nx);
-  collide_pair_even<S, GEOM, DENSE>(L, rows[r], (int)(t - r * (unsigned)L.nx));
+  const int x = (int)(t - r * (unsigned)L.nx);
+  const RowInfo R = rows[r];
+  if constexpr (ODD == 1 && GEOM != GEOM_PERIODIC) {
+    if (R.smask != 0) {
+#pragma unroll 1
+      for (int q = 0; q < 2; ++q) collide_cell<S, ODD, GEOM, DENSE, IDX32>(L, R, x + q);
+      return;
+    }
+  }
+  collide_pair<S, ODD, GEOM, DENSE, IDX32>(L, R, x);
 }
 
 // Equilibrium initialisation from the moments in uw (ux, uy, uz, rho - 1).
@@ -263,21 +277,32 @@ void launch_collide_g(const LatticeDev& L, const RowInfo* rows, int n_rows, bool
     else if (odd) launch(k_collide<S, 1, GEOM, false, true, true>);
     else if (dense) launch(k_collide<S, 0, GEOM, true, false, true>);
     else launch(k_collide<S, 0, GEOM, false, false, true>);
-  } else if (odd && idx32) {
+    return;
+  }
+  if constexpr (S != STORE_F32) {
+    if (L.nx % 2 == 0 && n_cells >= PAIR_CELLS_MIN) {
+      const unsigned pairs = (n_cells / 2 + block - 1) / block;
+      auto launch2 = [&](auto kernel) { launch_after(kernel, pairs, block, 0, st, false, L, rows, n_cells); };
+      if (odd && idx32) {
+        if (dense) launch2(k_collide_pair<S, 1, GEOM, true, true>);
+        else launch2(k_collide_pair<S, 1, GEOM, false, true>);
+      } else if (odd) {
+        if (dense) launch2(k_collide_pair<S, 1, GEOM, true, false>);
+        else launch2(k_collide_pair<S, 1, GEOM, false, false>);
+      } else {
+        if (dense) launch2(k_collide_pair<S, 0, GEOM, true, false>);
+        else launch2(k_collide_pair<S, 0, GEOM, false, false>);
+      }
+      return;
+    }
+  }
+  if (odd && idx32) {
     if (dense) launch(k_collide<S, 1, GEOM, true, true, false>);
     else launch(k_collide<S, 1, GEOM, false, true, false>);
   } else if (odd) {
     if (dense) launch(k_collide<S, 1, GEOM, true, false, false>);
     else launch(k_collide<S, 1, GEOM, false, false, false>);
   } else {
-    if constexpr (S != STORE_F32) {
-      if (L.nx % 2 == 0) {
-        const unsigned pairs = (n_cells / 2 + block - 1) / block;
-        if (dense) launch_after(k_collide_pair<S, GEOM, true>, pairs, block, 0, st, false, L, rows, n_cells);
-        else launch_after(k_collide_pair<S, GEOM, false>, pairs, block, 0, st, false, L, rows, n_cells);
-        return;
-      }
-    }
     if (dense) launch(k_collide<S, 0, GEOM, true, false, false>);
     else launch(k_collide<S, 0, GEOM, false, false, false>);
   }

@@ -242,24 +242,44 @@ __device__ __forceinline__ void collide_cell(const LatticeDev& L, const RowInfo&
 }
 
 
-// Two neighbouring fluid cells (x even, x + 1) of the local (even) step in
-// half-precision storage: 4-byte loads and stores, and the arithmetic of
+// Two neighbouring fluid cells (x even, x + 1) in half-precision storage: 4-byte
+// loads and stores (in the neighbour-addressed odd step, which takes rows
+// without solid neighbours only, where a direction has no x component), and the
+// arithmetic of
 // relax_cell's half-precision branch in packed FP32 pairs. The single-cell
 // kernel keeps ~48 KB of loads in flight on an SM, less than the memory's
 // latency times its rate; a thread of this one has twice the bytes and half
 // the instructions per cell. Needs an even nx (cell pairs aligned to 4 bytes).
-template <int S, int GEOM, bool DENSE>
-__device__ __forceinline__ void collide_pair_even(const LatticeDev& L, const RowInfo& R, int x) {
+template <int S, int ODD, int GEOM, bool DENSE, bool IDX32 = false>
+__device__ __forceinline__ void collide_pair(const LatticeDev& L, const RowInfo& R, int x) {
   static_assert(S != STORE_F32, "half-precision storage");
   using P = Pop<S>;
   using T = typename P::T;
   T* A = reinterpret_cast<T*>(L.pop);
   const int idx = R.base + x;
   const size_t N = (size_t)L.N;
+  auto elem = [&](int j, int e) -> T* {
+    if constexpr (IDX32) return A + (unsigned)((unsigned)j * (unsigned)N + (unsigned)e);
+    else return A + (size_t)j * N + e;
+  };
+  // odd step: element offset of the pair's row along s c_i, and of its two
+  // cells there (periodic x)
+  int oyp = R.oyp, oym = R.oym, ozp = R.ozp, ozm = R.ozm;
+  int left = x == 0 ? L.nx - 1 : -1, right = x + 2 == L.nx ? 2 - L.nx : 2;  // to x - 1, x + 2
+  auto row_off = [&](int i, int s) {
+    const int dy = s * cy(i), dz = s * cz(i);
+    return (dy > 0 ? oyp : (dy < 0 ? oym : 0)) + (dz > 0 ? ozp : (dz < 0 ? ozm : 0));
+  };
   F32x2 d[Q];
 #pragma unroll
   for (int j = 0; j < Q; ++j) {
-    const unsigned w = *reinterpret_cast<const unsigned*>(A + j * N + idx);
+    if (ODD && cx(j) != 0) {  // f_j(x) is at x - c_j
+      const int e = idx + row_off(j, -1);
+      d[j] = cx(j) > 0 ? pack2(P::ld_raw(elem(opp(j), e + left)), P::ld_raw(elem(opp(j), e)))
+                       : pack2(P::ld_raw(elem(opp(j), e + 1)), P::ld_raw(elem(opp(j), e + right)));
+      continue;
+    }
+    const unsigned w = *reinterpret_cast<const unsigned*>(ODD ? elem(opp(j), idx + row_off(j, -1)) : elem(j, idx));
     if constexpr (S == STORE_F16) {
       const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&w));
       d[j] = pack2(f.x, f.y);
@@ -323,9 +343,18 @@ __device__ __forceinline__ void collide_pair_even(const LatticeDev& L, const Row
     take(cz(i), c);
     return s;
   };
-  auto store = [&](int slot, F32x2 v) {
+  // (write addresses recomputed, not kept across the collision)
+  int widx = idx;
+  asm volatile("" : "+r"(widx), "+r"(left), "+r"(right), "+r"(oyp), "+r"(oym), "+r"(ozp), "+r"(ozm));
+  auto store = [&](int i, F32x2 v) {  // f*_i of both cells
     float a, b;
     unpack2(v, a, b);
+    if (ODD && cx(i) != 0) {
+      const int e = widx + row_off(i, +1);
+      P::st_raw(elem(i, cx(i) > 0 ? e + 1 : e + left), a);
+      P::st_raw(elem(i, cx(i) > 0 ? e + right : e), b);
+      return;
+    }
     unsigned w;
     if constexpr (S == STORE_F16) {
       const __half2 p = __floats2half2_rn(a, b);
@@ -334,7 +363,7 @@ __device__ __forceinline__ void collide_pair_even(const LatticeDev& L, const Row
       const __nv_bfloat162 p = __floats2bfloat162_rn(a, b);
       w = *reinterpret_cast<const unsigned*>(&p);
     }
-    *reinterpret_cast<unsigned*>(A + slot * N + idx) = w;
+    *reinterpret_cast<unsigned*>(ODD ? elem(i, widx + row_off(i, +1)) : elem(opp(i), widx)) = w;
   };
   store(0, fma2(om1, d[0], mul2(both(4.0f / 3.0f), T0)));
 #pragma unroll
@@ -343,7 +372,7 @@ __device__ __forceinline__ void collide_pair_even(const LatticeDev& L, const Row
     const F32x2 even = fma2(fma2(Bq, cu, mul2(P9, cG)), cu, T0w);
     const F32x2 odd = fma2(Aq, cu, mul2(P3, cG));
     F32x2 p = fma2(om1, d[i], add2(even, odd)), m = fma2(om1, d[i + 1], sub2(even, odd));
-    if (GEOM == GEOM_YWALLS && cx(i) != 0 && cy(i) != 0) {
+    if (!ODD && GEOM == GEOM_YWALLS && cx(i) != 0 && cy(i) != 0) {
       // half-way bounce-back at the moving walls, as in collide_cell
       auto wall = [&](int k, F32x2 v) {
         const int yn = R.y + cy(k);
@@ -354,8 +383,8 @@ __device__ __forceinline__ void collide_pair_even(const LatticeDev& L, const Row
       p = wall(i, p);
       m = wall(i + 1, m);
     }
-    store(opp(i), p);
-    store(opp(i + 1), m);
+    store(i, p);
+    store(i + 1, m);
   }
 }
 
