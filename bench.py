@@ -405,22 +405,28 @@ def kernels_per_step(w):
     return n
 
 
+def clustered_path(w):
+    """Whether ibm_lbm_step couples workload w by clusters of blocks: rigid
+    bodies of any number and membranes up to 38, nothing else."""
+    kinds = [b['kind'] for b in w['bodies']]
+    if not kinds or (w.get('morse') or {}).get('rc', 0) > 0 or any(k == 2 for k in kinds):
+        return False
+    return (sum(b['count'] for b in w['bodies']) == w['X'].shape[1] and kinds.count(0) <= 38
+            and max(b['count'] for b in w['bodies']) <= 4096)
+
+
 def production_launches(w, steps, fused):
-    """Kernels ibm_lbm_step launches for `steps` steps from an even AA step:
-    fused chunks of 64 (while more than 64 steps remain) or 16 steps (first
-    step's forces and spreading, then collide + fused kernel per step, the
-    last interpolation alone), the remaining steps one by one through the
-    separate kernels, and the conservation check. Without the fused path
-    every step takes the separate kernels."""
-    per_step = kernels_per_step(w)
+    """Kernels ibm_lbm_step launches for `steps` steps: on the fused paths the
+    first step's forces and spreading (two kernels, or one per kind of body by
+    clusters), then per step the collision and the coupling into the next, the
+    last step's interpolation, and the conservation check. Without them every
+    step takes the separate kernels."""
+    if clustered_path(w):
+        kinds = {b['kind'] == 0 for b in w['bodies']}
+        return steps + (steps + 1) * len(kinds) + 1
     if not fused:
-        return per_step * steps + 1
-    n, left = 0, steps
-    while left > 16:
-        c = 64 if left > 64 else 16
-        n += 2 + c + (c - 1) + 1
-        left -= c
-    return n + per_step * left + 1
+        return kernels_per_step(w) * steps + 1
+    return 2 + steps + (steps - 1) + 1 + 1
 
 
 def fused_path(w, storage):
@@ -811,7 +817,8 @@ def run_serve(args):
                      note='serving is end to end by construction: submission copies from host, results are read back to host inside the timed loop'),
             clocks=dict(sm_mhz=clk['sm_mhz'], sm_max_mhz=clk['sm_max_mhz'], reasons=clk['reasons'],
                         samples=clk['samples']),
-            gpu_launches=burst['chunks'] * args.serve_chunk * 7 + 4 * n)
+            # per chunk: its begin, first coupling and end, two kernels a step
+            gpu_launches=burst['chunks'] * (2 * args.serve_chunk + 3) + 4 * n)
         print(json.dumps(line), flush=True)
     if dist is not None:
         dist.destroy_process_group()
