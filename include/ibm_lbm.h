@@ -247,13 +247,13 @@ int ibm_lbm_get_force_density(ibm_lbm_t* h, double* g);
  * odd (neighbour-addressed) AA steps; then resets the sums. */
 int ibm_lbm_set_timing(ibm_lbm_t* h, int64_t max_steps);
 int ibm_lbm_get_timing(ibm_lbm_t* h, double out[6]);
-/* Timing of the production path of membrane suspensions. With on != 0 and
- * timing on, a handle that takes the fused coupling kernel (see
- * ibm_lbm_step) runs its timed steps on that path, with direct launches:
- * each step that launches the fused kernel is timed, out[2] receiving its
- * collision and out[3] the fused kernel (interpolation and advection of the
+/* Timing of the production path of suspensions. With on != 0 and timing on,
+ * a handle that takes a fused coupling (membranes, or rigid bodies, and no
+ * other markers) runs its timed steps on that path, with direct launches:
+ * each step that launches the coupling is timed, out[2] receiving its
+ * collision and out[3] the coupling (interpolation and advection of the
  * step, marker forces and spreading of the next, Sec. 2.3) with the clear
- * of the touched-tile flags before it; out[0] and out[1] stay zero and
+ * of the touched-tile flags where it is separate; out[0] and out[1] stay zero and
  * out[4] counts these steps. The other steps of the call (the first step's
  * forces and spreading, a step that restores the even AA parity, the last
  * step) run untimed. A handle that does not take the fused path is timed
@@ -267,7 +267,7 @@ int ibm_lbm_set_timing_fused(ibm_lbm_t* h, int on);
  * the GB300 build. Cases are submitted at any time and wait in FIFO order
  * until the device-memory budget and a slot allow their admission; every
  * ibm_lbm_server_advance then runs one chunk of steps for all admitted cases
- * together (one batched launch per stage, replayed as a CUDA graph), retires
+ * together (batched launches, a chunk replayed as a CUDA graph), retires
  * the cases that reached their step count (their results are copied to host
  * memory and their device memory is released) and admits waiting ones. A
  * case's result is the same as running it alone with ibm_lbm_step. Cases use

@@ -1,6 +1,7 @@
 // C ABI of the coupled IBM-LBM step (include/ibm_lbm.h): handle lifetime,
 // device memory, host<->device conversion, validation, and the step loop
-// (captured into CUDA graphs: one graph per 16 steps, plus single steps).
+// (CUDA graphs of 64 and 16 steps of collision and coupling, or of 16 steps
+// and single steps of the separate kernels; see Path below).
 #include <cuda_runtime.h>
 
 #include <unistd.h>
@@ -1180,7 +1181,8 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.off_ve = section(vel.data(), vel.size() * 2);
     D.off_vt_start = section(vts.data(), vts.size() * 2);
     D.off_vt = section(vtl.data(), vtl.size() * 2);
-    if (h->n_membranes <= std::max(CLUSTER_MEMBRANES_MAX, SOLID_MEMBRANES_MAX)) {
+    const size_t whole = buf.size();
+    if (!h->lean && h->n_membranes <= std::max(CLUSTER_MEMBRANES_MAX, SOLID_MEMBRANES_MAX)) {
       // parts of consecutive vertices for the clusters (cluster_body.cuh)
       int table[CLUSTER][8] = {};
       D.part_tris = 0;
@@ -1198,9 +1200,15 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
       }
       D.off_parts = section(table, sizeof(table));
     }
-    D.packed_bytes = (int)buf.size();
     unsigned char* dpk = nullptr;
-    if ((rc = upload<unsigned char>(h, h->marker_mem, &dpk, buf.data(), buf.size()))) return rc;
+    rc = upload<unsigned char>(h, h->marker_mem, &dpk, buf.data(), buf.size());
+    if (rc == IBM_LBM_E_NOMEM && buf.size() > whole) {  // without the parts: the paths that need none
+      buf.resize(whole);
+      D.off_parts = D.part_tris = 0;
+      rc = upload<unsigned char>(h, h->marker_mem, &dpk, buf.data(), buf.size());
+    }
+    if (rc) return rc;
+    D.packed_bytes = (int)buf.size();
     D.packed = dpk;
     D.nv = mesh->n_vertices;
     D.nt = mesh->n_triangles;
@@ -1315,8 +1323,9 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     // stage interface allows that) takes the per-marker path
     CUDA_TRY(h, cudaMemset(h->boxes, 0, sizeof(int4) * 2 * std::max<size_t>(1, groups.size())));
   }
-  // clusters: bodies of a size one cluster takes, nothing else
-  {
+  // clusters: bodies of a size one cluster takes, nothing else, and memory for
+  // the boxes (without it the separate kernels)
+  if (!h->lean) {
     bool few = n_bodies > 0 && covered == n_markers && h->n_filaments == 0 && h->n_membranes <= CLUSTER_MEMBRANES_MAX;
     for (int b = 0; b < n_bodies && few; ++b) {
       few = bodies[b].count <= CLUSTER_MAX_COUNT;
@@ -1325,13 +1334,13 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     few = few && (h->n_rigids == 0 ||
                   cluster_box_cells(cluster_fixed_words(h->cluster_max, 0, 0), h->n_rigids, h->n_sm) > 0);
     few = few && (h->n_membranes == 0 ||
-                  cluster_box_cells(cluster_fixed_words(h->mesh.nv, h->mesh.nv, h->mesh.part_tris), h->n_membranes,
-                                    h->n_sm) > 0);
+                  (h->mesh.part_tris > 0 &&
+                   cluster_box_cells(cluster_fixed_words(h->mesh.nv, h->mesh.nv, h->mesh.part_tris), h->n_membranes,
+                                     h->n_sm) > 0));
     if (few) {
       const size_t bytes = sizeof(int4) * 2 * CLUSTER * (size_t)n_bodies;
       int4* boxes = (int4*)dalloc(h, h->marker_mem, bytes);
-      if (!boxes) return fail(h, IBM_LBM_E_NOMEM, "device allocation failed");
-      CUDA_TRY(h, cudaMemset(boxes, 0, bytes));
+      if (boxes) CUDA_TRY(h, cudaMemset(boxes, 0, bytes));
       h->cluster_boxes = boxes;
     }
   }

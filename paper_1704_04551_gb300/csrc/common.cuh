@@ -106,7 +106,8 @@ struct LatticeDev {
   // is set, and the interpolation, which sweeps the same boxes of cells
   // afterwards, writes g back to zero there (in its latency-bound box load,
   // not in the bandwidth-bound collision). flags is cleared at the start of
-  // each step.
+  // each step (couplings by clusters have two of each: a coupling clears what
+  // its collision read and sets the other).
   float4* g;             // spread force density (gx, gy, gz, 0) [N]
   uint8_t* flags;        // [ntx*nty*ntz]: tile touched by a marker stencil this step
   int* status;           // device status word (0 = OK)

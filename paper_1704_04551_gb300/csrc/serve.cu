@@ -279,6 +279,7 @@ struct ibm_lbm_server {
     int unstable = 0;
     int cluster_cap = 0;  // > 0: its bodies are coupled by clusters (cells of a block's box)
     bool primed = false;  // then: the next step's forces are spread already
+    bool lean = false;    // the budget alone has no room for what clusters need
     // inputs
     ibm_lbm_config lat{};
     std::vector<double> rho0, u0, X;
@@ -392,7 +393,8 @@ int ensure(ibm_lbm_server_t* s, Item** buf, size_t* cap, size_t n) {
 // handle allocates: populations, wall velocities, two force-density and
 // tile-flag buffers, the row table, per-marker arrays (X, U, F, stencil
 // cache; reference positions of rigid markers), marker groups and boxes,
-// bodies and lists, packed mesh topology, plus allocation rounding.
+// bodies and lists, packed mesh topology, plus allocation rounding. What only
+// couplings by clusters need (template parts, boxes) is left to admit().
 size_t case_estimate(const ibm_lbm_config& L, int64_t M, int n_bodies, bool rigid, int nv, int nt) {
   const size_t N = (size_t)L.nx * L.ny * L.nz;
   const size_t tiles = (size_t)((L.nx + 31) / 32) * ((L.ny + 3) / 4) * ((L.nz + 3) / 4);
@@ -422,6 +424,7 @@ int admit(ibm_lbm_server_t* s) {
     if (rc == IBM_LBM_OK)
       rc = ibm_lbm_set_lattice(h, c->rho0.empty() ? nullptr : c->rho0.data(), c->u0.empty() ? nullptr : c->u0.data());
     if (rc == IBM_LBM_OK) {
+      h->lean = c->lean;
       ibm_lbm_mesh mesh{c->nv, c->nt, c->tris.data(), c->rest.data()};
       const int64_t M = (int64_t)(c->X.size() / 3);
       rc = ibm_lbm_set_markers(h, c->has_mesh ? &mesh : nullptr, (int32_t)c->bodies.size(), c->bodies.data(), M,
@@ -432,6 +435,17 @@ int admit(ibm_lbm_server_t* s) {
       if (h) ibm_lbm_destroy(h);
       if (rc == IBM_LBM_E_NOMEM) break;  // retry after retirements
       return sfail(s, rc, "server: admission failed: " + why);
+    }
+    // What clusters need beside the estimate (template parts, boxes; small
+    // next to a lattice) stays inside the budget too: a case waits for it, or,
+    // where the whole budget has no room, runs without clusters.
+    const size_t need = ibm_lbm_device_bytes(h) + (h->cluster_boxes ? sizeof(float4) * (size_t)h->L.N : 0);
+    if (!c->lean && need > c->estimate && s->used + need > s->cfg.device_mem_budget) {
+      ibm_lbm_destroy(h);
+      c->lean = need > s->cfg.device_mem_budget;
+      if (c->lean) continue;
+      c->estimate = need;
+      break;
     }
     // Clusters where they apply and the second force-density buffer is to be
     // had (part of the estimate). The boxes' size is that of two blocks per SM

@@ -38,8 +38,9 @@
 //   16-byte shared load serves a node) once, with asynchronous copies, and
 //   gathers from shared memory; the same sweep clears the force density the
 //   collision has consumed.
-// Larger boxes (scattered tracers, very large bodies) fall back to
-// per-marker global float4 atomics / gathers. The box of each group is
+// Larger boxes are taken in slabs of z layers (see Boxes below), very large
+// ones by per-marker global float4 atomics / gathers; passive tracers move in
+// a kernel of their own without a box. The box of each group is
 // computed by the spread kernel and reused by the interpolation of the same
 // step (markers do not move in between; a marker found outside the box
 // takes the per-marker path).
