@@ -1323,8 +1323,7 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     // stage interface allows that) takes the per-marker path
     CUDA_TRY(h, cudaMemset(h->boxes, 0, sizeof(int4) * 2 * std::max<size_t>(1, groups.size())));
   }
-  // clusters: bodies of a size one cluster takes, nothing else, and memory for
-  // the boxes (without it the separate kernels)
+  // clusters: bodies of a size one cluster takes, nothing else
   if (!h->lean) {
     bool few = n_bodies > 0 && covered == n_markers && h->n_filaments == 0 && h->n_membranes <= CLUSTER_MEMBRANES_MAX;
     for (int b = 0; b < n_bodies && few; ++b) {
@@ -1340,7 +1339,8 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     if (few) {
       const size_t bytes = sizeof(int4) * 2 * CLUSTER * (size_t)n_bodies;
       int4* boxes = (int4*)dalloc(h, h->marker_mem, bytes);
-      if (boxes) CUDA_TRY(h, cudaMemset(boxes, 0, bytes));
+      if (!boxes) return fail(h, IBM_LBM_E_NOMEM, "device allocation failed");
+      CUDA_TRY(h, cudaMemset(boxes, 0, bytes));
       h->cluster_boxes = boxes;
     }
   }
