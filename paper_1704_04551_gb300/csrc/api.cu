@@ -4,6 +4,7 @@
 // and single steps of the separate kernels; see Path below).
 #include <cuda_runtime.h>
 
+#include <sys/mman.h>
 #include <unistd.h>
 
 #include <algorithm>
@@ -84,16 +85,34 @@ void* dalloc(ibm_lbm_t* h, std::vector<Alloc>& pool, size_t bytes) {
   return p;
 }
 
+// Whether every page of a host buffer is in memory (false if the system does
+// not say).
+bool pages_mapped(const void* p, size_t bytes, size_t page) {
+  const size_t first = (size_t)p / page * page, last = (size_t)p + bytes;
+  unsigned char in[256];
+  for (size_t a = first; a < last; a += sizeof(in) * page) {
+    const size_t n = std::min(sizeof(in), (last - a + page - 1) / page);
+    if (mincore(reinterpret_cast<void*>(a), n * page, in) != 0) return false;
+    for (size_t i = 0; i < n; ++i)
+      if (!(in[i] & 1)) return false;
+  }
+  return true;
+}
+
 // Take the page faults of a host buffer before a copy, which would fault its
 // pages one by one from the device's side: one byte per page is written (an
 // output that is about to be overwritten) or read (an input), by several
 // threads for a large buffer. A copy of 8 MB into fresh pages took 6 ms, and
 // 0.25 ms into mapped ones; a page touched here costs ~0.25 us, or a cache
 // miss if it was mapped. Below 64 KiB a copy is a few tens of us either way.
+// Up to 16 MiB a buffer whose pages are all there is left alone: its copy takes
+// less than the threads below (get_fields of a 77x94x67 lattice into arrays in
+// use before: 0.14 of 1.88 ms of a two-step run).
 void touch_pages(const void* p, size_t bytes, bool write) {
   if (!p || bytes < ((size_t)64 << 10)) return;
   const long pg = sysconf(_SC_PAGESIZE);
   const size_t page = pg > 0 ? (size_t)pg : 4096;
+  if (bytes < ((size_t)16 << 20) && pages_mapped(p, bytes, page)) return;
   // a thread for every 2 MiB (starting one costs as much as touching ~100 pages)
   const unsigned nt = std::min({8u, std::max(1u, std::thread::hardware_concurrency()), (unsigned)(bytes >> 21)});
   const size_t chunk = nt > 1 ? (bytes / nt + page - 1) / page * page : 0;
