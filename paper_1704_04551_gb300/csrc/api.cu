@@ -285,16 +285,21 @@ void collide(ibm_lbm_t* h, Path p, int k, bool odd, bool dense) {
 }
 
 // One coupled step by itself on the handle's stream (also used under
-// capture); it needs the first buffers only.
-void enqueue_step(ibm_lbm_t* h, bool odd, bool dense) {
+// capture); it needs the first buffers only. With `waiting`, a force density
+// that a SPREAD stage left in the first buffer goes into this step wherever it
+// lies (every tile is read) and is gone after it: the couplings clear what
+// they spread themselves.
+void enqueue_step(ibm_lbm_t* h, bool odd, bool dense, bool waiting = false) {
   const Path p = path_of(h);
   couple_begin(h, p, 0);
+  if (waiting) cudaMemsetAsync(h->fbuf, 1, (size_t)tiles(h->L), h->stream);
   collide(h, p, 0, odd, dense);
+  if (waiting) cudaMemsetAsync(h->gbuf, 0, sizeof(float4) * (size_t)h->L.N, h->stream);
   couple_end(h, p, 0);
 }
 
 // One step with an event before each stage and after the last.
-void enqueue_timed_step(ibm_lbm_t* h, bool odd, bool dense) {
+void enqueue_timed_step(ibm_lbm_t* h, bool odd, bool dense, bool waiting) {
   cudaStream_t st = h->stream;
   const size_t base = 5 * h->timed_steps;
   const bool rec = base + 5 <= h->events.size();
@@ -307,9 +312,11 @@ void enqueue_timed_step(ibm_lbm_t* h, bool odd, bool dense) {
   mark(1);
   cudaMemsetAsync(L.flags, 0, (size_t)tiles(L), st);
   if (h->m.M > 0) spread(h, L);
+  if (waiting) cudaMemsetAsync(L.flags, 1, (size_t)tiles(L), st);
   mark(2);
   collide(h, SEPARATE, 0, odd, dense);
   mark(3);
+  if (waiting) cudaMemsetAsync(L.g, 0, sizeof(float4) * (size_t)L.N, st);
   if (h->m.M > 0) interpolate(h, L);
   mark(4);
   if (rec) {
@@ -438,6 +445,15 @@ int enqueue_steps(ibm_lbm_t* h, int64_t n) {
     if (!ensure_second_buffer(h)) CUDA_TRY(h, cudaGetLastError());  // (no memory: separate kernels)
   }
   const bool fused = fused_applies(h);
+  if (h->density_waiting && path_of(h) == SEPARATE) {
+    const bool odd = h->odd_next, dense = left == 1;
+    if (h->timing && !fused) enqueue_timed_step(h, odd, dense, true);
+    else enqueue_step(h, odd, dense, true);
+    h->density_waiting = false;
+    --left;
+    h->steps += 1;
+    h->odd_next = !odd;
+  }
   if (h->timing) {
     // with timing_fused, a handle on a fused path times only its coupled
     // steps, the last one of the call apart; every other handle is timed
@@ -451,7 +467,7 @@ int enqueue_steps(ibm_lbm_t* h, int64_t n) {
         continue;
       }
       if (fused) enqueue_step(h, h->odd_next, left == 1);
-      else enqueue_timed_step(h, h->odd_next, left == 1);
+      else enqueue_timed_step(h, h->odd_next, left == 1, false);
       --left;
       h->steps += 1;
       h->odd_next = !h->odd_next;
@@ -979,6 +995,7 @@ static int impl_ibm_lbm_set_lattice(ibm_lbm_t* h, const double* rho, const doubl
   CUDA_TRY(h, cudaMemsetAsync(h->fbuf, 0, (size_t)tiles(L), h->stream));
   CUDA_TRY(h, cudaMemsetAsync(L.status, 0, sizeof(int), h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  h->density_waiting = false;
   h->steps = 0;
   h->odd_next = false;
   return IBM_LBM_OK;
@@ -1002,6 +1019,7 @@ static int impl_ibm_lbm_set_populations(ibm_lbm_t* h, const double* f) {
   CUDA_TRY(h, cudaMemsetAsync(h->gbuf, 0, sizeof(float4) * (size_t)h->L.N, h->stream));
   CUDA_TRY(h, cudaMemsetAsync(h->fbuf, 0, (size_t)tiles(h->L), h->stream));
   CUDA_TRY(h, cudaStreamSynchronize(h->stream));
+  h->density_waiting = false;
   h->odd_next = false;
   return IBM_LBM_OK;
 }
@@ -1491,6 +1509,7 @@ static int impl_ibm_lbm_run_stage(ibm_lbm_t* h, int32_t stage) {
       CUDA_TRY(h, cudaMemsetAsync(L.flags, 0, (size_t)tiles(L), st));
       launch_spread(L, h->m, h->groups, h->n_groups, h->boxes, st);
       h->boxes_valid = true;
+      h->density_waiting = true;
       break;
     }
     case IBM_LBM_STAGE_COLLIDE:
@@ -1502,6 +1521,7 @@ static int impl_ibm_lbm_run_stage(ibm_lbm_t* h, int32_t stage) {
         CUDA_TRY(h, cudaMemsetAsync(h->boxes, 0, sizeof(int4) * 2 * (size_t)h->n_groups, st));
       launch_interpolate(h->L, h->m, h->groups, h->n_groups, h->boxes, st);
       h->boxes_valid = false;
+      h->density_waiting = false;
       h->steps += 1;
       break;
     default:

@@ -81,6 +81,7 @@ struct ibm_lbm {
   int cluster_max = 0;            // largest marker count of a body
   bool lean = false;              // markers set without what only clusters need
   uint8_t* fbuf2 = nullptr;       // second tile flags (beside gbuf2)
+  bool density_waiting = false;   // a SPREAD stage's force density is in gbuf, for the next step
   bool boxes_valid = false;       // boxes match the markers' current positions (stage interface)
   bool need_zero_F = false;
   // state
