@@ -445,7 +445,7 @@ int enqueue_steps(ibm_lbm_t* h, int64_t n) {
     if (!ensure_second_buffer(h)) CUDA_TRY(h, cudaGetLastError());  // (no memory: separate kernels)
   }
   const bool fused = fused_applies(h);
-  if (h->density_waiting && path_of(h) == SEPARATE) {
+  if (h->density_waiting) {
     const bool odd = h->odd_next, dense = left == 1;
     if (h->timing && !fused) enqueue_timed_step(h, odd, dense, true);
     else enqueue_step(h, odd, dense, true);

@@ -79,3 +79,32 @@ def test_spread_collide_then_step_leaves_no_density(cuda_lib):
     sim.stage(cuda_lib.STAGE_COLLIDE)
     sim.step(2)
     assert np.abs(sim.force_density()).max() == 0.0
+
+
+def _tethered():
+    lat = LATTICES['tube']
+    X, body = I.rigid_ellipsoid([18.0, 6.5, 6.0], (3.0, 2.0, 2.0), [1.0, 0.0, 0.0, 0.0], 0, freq=3, kappa=0.05)
+    return dict(lattice=lat, mesh=None, bodies=[dict(body, vel=[1e-3, 5e-4, 0.0])], X=X)
+
+
+def _membranes(n):
+    """n red cells of a coarse template (42 vertices): clusters, or from 39 on the fused kernel."""
+    lat = dict(nx=40, ny=28, nz=26, tau=0.8, geometry=0, body_force=[2e-6, -1e-6, 5e-7])
+    rest, tris = I.rbc_rest_shape(8.0, 2)
+    V = rest.shape[1]
+    rng = np.random.default_rng(6)
+    C = rng.random((n, 3)) * [40, 28, 26]
+    X = np.concatenate([1.04 * rest + c[:, None] + 0.01 * rng.standard_normal(rest.shape) for c in C], axis=1)
+    bodies = [I._body(I.BODY_MEMBRANE, k * V, V, kBT_p=1e-3, k_b=5e-4, k_l=3e-3, k_g=2e-3, k_v=2e-3)
+              for k in range(n)]
+    return dict(lattice=lat, mesh=dict(rest_X=rest, tris=tris), bodies=bodies, X=X)
+
+
+BODIES = dict(rigid=_tethered, cluster_membranes=lambda: _membranes(3), fused_membranes=lambda: _membranes(40))
+
+
+@pytest.mark.parametrize('before,after', [(0, (2, 20)), (1, (1, 2)), (1, (20,)), (3, (3,))])
+@pytest.mark.parametrize('kind', list(BODIES))
+def test_spread_then_step_with_bodies(cuda_lib, kind, before, after):
+    """Both parities: a coupled step's buffer goes with the parity, the stage's does not."""
+    _run(cuda_lib, BODIES[kind](), before, after)
