@@ -224,10 +224,13 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
 // one gives no scale (none yet, or contributions above its headroom): their
 // maximum is taken first, then they are added in fixed point with the scale it allows, qcap. The sums depend on no
 // order, unlike float atomics, which reruns of a body's first step differed
-// by. Only contributions that are not finite are added as floats, to reach the
-// forces. pass(add) hands out the contributions; vertices [v0, v0 + n) are
+// by. Contributions that are not finite are added as floats, to reach the
+// forces, and so are those of a body whose largest one is below REDO_TINY: the
+// scale qcap / q and its inverse stay normal numbers down to there (qcap < 2^31).
+// pass(add) hands out the contributions; vertices [v0, v0 + n) are
 // summed in sQ [3][stride] (zero entries [n, stride) included in the clear).
 // Returns the unit of the sums.
+constexpr float REDO_TINY = 1e-25f;
 template <class Pass>
 __device__ __forceinline__ float redo_scatter(Pass&& pass, int* sQ, int stride, int n, int v0, int n_clear, float qcap,
                                               float& qmax, unsigned* s_qmax, bool& is_float) {
@@ -241,7 +244,7 @@ __device__ __forceinline__ float redo_scatter(Pass&& pass, int* sQ, int stride, 
       for (int i = threadIdx.x; i < 3 * n_clear; i += blockDim.x) sQ[i] = 0;  // (0.f as well)
       __syncthreads();
       const float q = __uint_as_float(*s_qmax);
-      is_float = !isfinite(q);
+      is_float = !isfinite(q) || (q > 0.f && q < REDO_TINY);
       S = q > 0.f && !is_float ? qcap / q : 1.0f;
     }
     pass([&](int v, float3 f) {
