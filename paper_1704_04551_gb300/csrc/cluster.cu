@@ -115,7 +115,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(SOLID_THREADS,
     fe[t] = Q.fext ? Q.fext[k] * Q.inv_mass : 0.0;
   }
   for (int i = tid; i < 3 * per; i += SOLID_THREADS) sQ[i] = 0;
-  if (tid < 2) S.fix[tid] = 0;
+  if (tid == 0) S.part_sum = BodySums{};
   if (tid < CLUSTER) S.qmax[tid] = 0u;
   if (tid == 0) S.fmax_s = S.redo_max = 0u;
   cl.sync();  // every block has started and has read the origin
@@ -164,7 +164,7 @@ __global__ void __cluster_dims__(CLUSTER, 1, 1) __launch_bounds__(SOLID_THREADS,
     }
     __syncthreads();  // (all have read the maximum)
     if (tid == 0) S.fmax_s = 0u;
-    if (tid < 2) S.fix[tid] = 0;
+    if (tid == 0) S.part_sum = BodySums{};
   }
   if (tid == 0) cl.map_shared_rank(&S.qmax[0], 0)[rank] = __float_as_uint(q_prev);
 #pragma unroll

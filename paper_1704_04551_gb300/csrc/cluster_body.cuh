@@ -82,7 +82,7 @@ struct ClusterShare {
   double total[6];                  // force and torque of all blocks
   double pose[12];                  // C, q (4), V; direct forcing
   double part[CLUSTER_WORKERS / 32][6];
-  long long fix[2];                 // area and volume, fixed point
+  BodySums part_sum;                // this block's area and volume
 };
 
 // Arguments of one body's coupling: the lattice as the finished collision
@@ -263,7 +263,7 @@ struct MembraneModuli {
 
 // Forces on this block's vertices c0 .. c0 + n - 1 of a membrane whose
 // positions all blocks of the cluster have written (and synchronised on),
-// with S.fix and sQ cleared. The sums are left in sQ: fixed point in units of
+// with S.part_sum and sQ cleared. The sums are left in sQ: fixed point in units of
 // `unit`, or floats where unit = 0 (a contribution that is not finite). Returns the thread's largest contribution;
 // q_prev: the largest one of the last evaluation. Contains one cluster barrier.
 template <int THREADS>
@@ -297,11 +297,11 @@ __device__ __forceinline__ float cluster_membrane(ClusterShare& S, const Membran
       vp += dot(dv(Tr.x, 0), N) * (1.0f / 6.0f);
     }
   }
-  warp_fixed_sum(ap, vp, K, S.fix);
+  warp_fixed_sum(ap, vp, K, &S.part_sum);
   __syncthreads();
   if (tid < 2 * CLUSTER) {
     const int r = tid >> 1, q = tid & 1;
-    cl.map_shared_rank(&S.sum[0][0], r)[6 * rank + q] = (double)S.fix[q];
+    cl.map_shared_rank(&S.sum[0][0], r)[6 * rank + q] = S.part_sum.units(q, q == 0 ? K.qa : K.qv);
   }
   // the area and volume terms need the other blocks' sums; the edges do not
   cl.barrier_arrive();
@@ -621,7 +621,7 @@ __device__ __forceinline__ void cluster_couple(const ClusterArgs& A, ClusterShar
       m.frac[q * M + first + j] = fr;
     }
     for (int i = tid; i < 3 * per; i += CLUSTER_THREADS) sQ[i] = 0;
-    if (tid < 2) S.fix[tid] = 0;
+    if (tid == 0) S.part_sum = BodySums{};
     if (tid < CLUSTER) S.qmax[tid] = 0u;
     cl.sync();  // positions complete
     const MembraneModuli Km{B->kBT_p, B->k_b, B->k_l, B->k_g, B->k_v};

@@ -76,12 +76,15 @@ __device__ __forceinline__ Topo topo_at(const unsigned char* base, const MeshDev
 }
 
 // The body's area and volume are sums of FP32 values of which only a small
-// difference from the rest value matters. They are added exactly, in fixed
-// point: a value v is hi + lo with hi = round(v s) (s a power of two, the
-// whole sum about 2^20 of its units) and lo the rest in units 2^22 finer, each
-// summed over a warp by one integer reduction. A tree of FP64 adds keeps an
-// SM's FP64 pipe (2 lanes a cycle) busy for ~1 us per body, and its last
-// serial sum of the warps for as long again.
+// difference from the rest value matters. They are added in fixed point: a
+// value v is hi + lo with hi = round(v s) (s a power of two, the whole sum
+// about 2^20 of its units) and lo the rest in units 2^22 finer (rounded to
+// them: 2^-42 of the rest area or volume), each summed over a warp by one
+// integer reduction. A tree of FP64 adds keeps an SM's FP64 pipe (2 lanes a
+// cycle) busy for ~1 us per body, and its last serial sum of the warps for as
+// long again. A warp with a value past 2^26 units (64 times the rest sum: a
+// body swollen or torn far beyond its rest shape), or one that is not finite,
+// would leave the integers' range: it is added in FP64 beside them.
 struct MembraneScale {
   float sa, sv;    // units of hi per area, volume
   double qa, qv;   // area, volume per unit of lo
@@ -94,17 +97,45 @@ __device__ __forceinline__ MembraneScale membrane_scale(const MeshDev& mesh) {
   K.qv = (double)(0x1p-22f / mesh.fix_v);
   return K;
 }
+// Area and volume of a block in shared memory: fixed point, and what was out
+// of its range.
+struct BodySums {
+  long long fix[2];
+  double far[2];
+  // in units of lo; q: size of one
+  __device__ __forceinline__ double units(int i, double q) const {
+    const double n = (double)fix[i];
+    return __double_as_longlong(far[i]) == 0 ? n : n + far[i] / q;
+  }
+};
 __device__ __forceinline__ long long warp_fixed(float v, float s) {
   const int hi = __float2int_rn(v * s);
   const int lo = __float2int_rn(fmaf(v, s, -(float)hi) * 4194304.0f);
   return ((long long)__reduce_add_sync(0xffffffffu, hi) << 22) + __reduce_add_sync(0xffffffffu, lo);
 }
-// Adds the warp's values to sum[0] (area) and sum[1] (volume) in shared memory.
-__device__ __forceinline__ void warp_fixed_sum(float area, float volume, const MembraneScale& K, long long* sum) {
+__device__ __forceinline__ void warp_far_sum(float area, float volume, BodySums* sums) {
+  double a = area, v = volume;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    a += __shfl_xor_sync(0xffffffffu, a, o);
+    v += __shfl_xor_sync(0xffffffffu, v, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&sums->far[0], a);
+    atomicAdd(&sums->far[1], v);
+  }
+}
+// Adds the warp's values to the block's area and volume.
+__device__ __forceinline__ void warp_fixed_sum(float area, float volume, const MembraneScale& K, BodySums* sums) {
+  constexpr float most = 67108864.0f;  // 32 lanes below it add up to less than 2^31
+  if (__any_sync(0xffffffffu, !(fabsf(area * K.sa) < most && fabsf(volume * K.sv) < most))) {
+    warp_far_sum(area, volume, sums);
+    return;
+  }
   const long long a = warp_fixed(area, K.sa), v = warp_fixed(volume, K.sv);
   if ((threadIdx.x & 31) == 0) {
-    atomicAdd(reinterpret_cast<unsigned long long*>(sum), (unsigned long long)a);
-    atomicAdd(reinterpret_cast<unsigned long long*>(sum + 1), (unsigned long long)v);
+    atomicAdd(reinterpret_cast<unsigned long long*>(&sums->fix[0]), (unsigned long long)a);
+    atomicAdd(reinterpret_cast<unsigned long long*>(&sums->fix[1]), (unsigned long long)v);
   }
 }
 
@@ -311,13 +342,13 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
   float* sN = S.sN;
   float* sA = S.sA;
   __shared__ float s_dev[2];
-  __shared__ long long s_fix[2];
+  __shared__ BodySums s_sum;
   __shared__ unsigned s_qmax;
   const MembraneScale K = membrane_scale(mesh);
   for (int i = threadIdx.x; i < 3 * nv; i += blockDim.x) sQ[i] = 0;
   if (threadIdx.x == 0) {
     s_qmax = 0u;
-    s_fix[0] = s_fix[1] = 0;
+    s_sum = BodySums{};
   }
   __syncthreads();  // the sums are cleared before the first warp adds to them
   // x_a - x_b, exact in the integer part, one FP32 rounding in the fraction
@@ -340,11 +371,11 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
     // triangle's first vertex from vertex 0
     v_part += dot(dv(Tr.x, 0), N) * (1.0f / 6.0f);
   }
-  warp_fixed_sum(a_part, v_part, K, s_fix);
+  warp_fixed_sum(a_part, v_part, K, &s_sum);
   __syncthreads();  // normals, areas and sums are visible
   // A - A0 and V - V0 in FP64 (small differences of large sums)
-  if (threadIdx.x == 0) s_dev[0] = (float)((double)s_fix[0] * K.qa - (double)mesh.A0) / mesh.A0;
-  if (threadIdx.x == 32) s_dev[1] = (float)((double)s_fix[1] * K.qv - (double)mesh.V0) / mesh.V0;
+  if (threadIdx.x == 0) s_dev[0] = (float)(s_sum.units(0, K.qa) * K.qa - (double)mesh.A0) / mesh.A0;
+  if (threadIdx.x == 32) s_dev[1] = (float)(s_sum.units(1, K.qv) * K.qv - (double)mesh.V0) / mesh.V0;
   __syncthreads();
   const float cg = k_g * s_dev[0];
   const float cv = k_v * s_dev[1];

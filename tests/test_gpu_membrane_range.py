@@ -42,3 +42,9 @@ def _forces_match(cuda_lib, w):
 @pytest.mark.parametrize('factor', [1e-32, 1e-28, 1e-22])
 def test_tiny_forces(cuda_lib, n, factor):
     _forces_match(cuda_lib, _bodies(n, 1.0, factor))
+
+
+@pytest.mark.parametrize('n', [2, 40])
+@pytest.mark.parametrize('swell', [20.0, 70.0, 300.0])
+def test_swollen_cells(cuda_lib, n, swell):
+    _forces_match(cuda_lib, _bodies(n, swell, 1.0))
