@@ -209,12 +209,18 @@ bool chained(const ibm_lbm_t* h) {
   return !h->timing && h->n_rows > 0 && h->L.N <= CHAINED_CELLS_MAX && (h->n_rigids > 0) != (h->n_membranes > 0);
 }
 
+// Blocks of n clusters on an SM: one while they are all resident so, for
+// larger boxes.
+int per_sm(const ibm_lbm_t* h, int n) { return n <= h->clusters_one ? 1 : CLUSTER_PER_SM; }
+
 void enqueue_cluster(ibm_lbm_t* h, int k, int next, bool interp, bool forces, bool spread) {
   const LatticeDev L = lattice_of(h, CLUSTERED, k), Ln = lattice_of(h, CLUSTERED, next);
   launch_couple_cluster(L, Ln.g, Ln.flags, h->m, h->d_bodies, h->rigid_list, h->n_rigids, false, h->cluster_max,
-                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, interp && chained(h), h->stream);
+                        h->mesh, h->cluster_boxes, per_sm(h, h->n_rigids), interp, forces, spread,
+                        interp && chained(h), h->stream);
   launch_couple_cluster(L, Ln.g, Ln.flags, h->m, h->d_bodies, h->membrane_list, h->n_membranes, true, h->mesh.nv,
-                        h->mesh, h->cluster_boxes, h->n_sm, interp, forces, spread, interp && chained(h), h->stream);
+                        h->mesh, h->cluster_boxes, per_sm(h, h->n_membranes), interp, forces, spread,
+                        interp && chained(h), h->stream);
 }
 
 // Marker forces: each body's own forces (membranes, rigid tethers,
@@ -929,10 +935,9 @@ static int impl_ibm_lbm_create(const ibm_lbm_config* cfg, const ibm_lbm_allocato
     h->n_rows = (int)rows.size();
     if (upload<RowInfo>(h, h->lattice_mem, &h->rows, rows.data(), rows.size())) return bail(IBM_LBM_E_NOMEM);
   }
-  if (cudaDeviceGetAttribute(&h->n_sm, cudaDevAttrMultiProcessorCount, cfg->device) != cudaSuccess)
-    return bail(IBM_LBM_E_CUDA);
   if (transfer_configure() != cudaSuccess || couple_configure() != cudaSuccess ||
-      cluster_configure() != cudaSuccess) {
+      cluster_configure() != cudaSuccess || cluster_capacity(1, &h->clusters_one) != cudaSuccess ||
+      cluster_capacity(CLUSTER_PER_SM, &h->clusters_two) != cudaSuccess) {
     cudaGetLastError();
     return bail(IBM_LBM_E_CUDA);
   }
@@ -1368,11 +1373,11 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
       h->cluster_max = std::max(h->cluster_max, (int)bodies[b].count);
     }
     few = few && (h->n_rigids == 0 ||
-                  cluster_box_cells(cluster_fixed_words(h->cluster_max, 0, 0), h->n_rigids, h->n_sm) > 0);
+                  cluster_box_cells(cluster_fixed_words(h->cluster_max, 0, 0), per_sm(h, h->n_rigids)) > 0);
     few = few && (h->n_membranes == 0 ||
                   (h->mesh.part_tris > 0 &&
-                   cluster_box_cells(cluster_fixed_words(h->mesh.nv, h->mesh.nv, h->mesh.part_tris), h->n_membranes,
-                                     h->n_sm) > 0));
+                   cluster_box_cells(cluster_fixed_words(h->mesh.nv, h->mesh.nv, h->mesh.part_tris),
+                                     per_sm(h, h->n_membranes)) > 0));
     if (few) {
       const size_t bytes = sizeof(int4) * 2 * CLUSTER * (size_t)n_bodies;
       int4* boxes = (int4*)dalloc(h, h->marker_mem, bytes);

@@ -210,23 +210,41 @@ void launch_solid_cluster(const MarkersDev& m, BodyDev* bodies, const int* list,
   k_solid_cluster<<<n * CLUSTER, SOLID_THREADS, 4 * (size_t)solid_words(mesh.nv, mesh.part_tris), st>>>(Q);
 }
 
-// Cells of a block's box: what one resident wave of the launch leaves, at
-// most CLUSTER_BOX_MAX (a block of a larger box adds its markers one by one
-// with global atomics). 0: the fixed part alone does not fit.
-int cluster_box_cells(size_t fixed_words, int n_clusters, int n_sm) {
-  const int per_sm = std::max(1, (n_clusters * CLUSTER + n_sm - 1) / n_sm);
-  const size_t share = std::min<size_t>(CLUSTER_SMEM_MAX, (size_t)(CLUSTER_SMEM_SM / std::min(per_sm, CLUSTER_PER_SM)) - 5 * 1024);
+// Clusters the device holds at once with `per_sm` blocks on an SM. Fewer than
+// its SMs give room for: a cluster's blocks lie in one GPC, and GPCs are not
+// all of a size (152 SMs: 15 clusters of one block an SM, 36 of two, not 19
+// and 38; with one block an SM 16 to 19 bodies took two waves, 72 us a step
+// instead of 45 with two for membranes of 642 vertices at 72^3).
+cudaError_t cluster_capacity(int per_sm, int* out) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CLUSTER);
+  cfg.blockDim = dim3(CLUSTER_THREADS);
+  cfg.dynamicSmemBytes = per_sm == 1 ? (size_t)CLUSTER_SMEM_MAX : (size_t)CLUSTER_SHARE;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = CLUSTER;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaOccupancyMaxActiveClusters(out, k_couple_cluster<GEOM_TUBE, 1>, &cfg);
+}
+
+// Cells of a block's box: what `per_sm` blocks on an SM leave, at most
+// CLUSTER_BOX_MAX (a block of a larger box adds its markers one by one with
+// global atomics). 0: the fixed part alone does not fit.
+int cluster_box_cells(size_t fixed_words, int per_sm) {
+  const size_t share = per_sm == 1 ? (size_t)CLUSTER_SMEM_MAX : (size_t)CLUSTER_SHARE;
   if (4 * fixed_words + 12 * 1024 > share) return 0;
   return (int)std::min<size_t>(CLUSTER_BOX_MAX, (share / 4 - fixed_words) / 3) & ~3;  // (cleared 16 bytes at a time)
 }
 
 void launch_couple_cluster(const LatticeDev& L, float4* g_next, uint8_t* flags_next, const MarkersDev& m,
                            BodyDev* bodies, const int* list, int n, bool membranes, int max_count,
-                           const MeshDev& mesh, int4* boxes, int n_sm, bool interp, bool forces, bool spread,
+                           const MeshDev& mesh, int4* boxes, int per_sm, bool interp, bool forces, bool spread,
                            bool programmatic, cudaStream_t st) {
   if (n == 0) return;
   const size_t fixed = cluster_fixed_words(max_count, membranes ? mesh.nv : 0, membranes ? mesh.part_tris : 0);
-  const int cap = cluster_box_cells(fixed, n, n_sm);
+  const int cap = cluster_box_cells(fixed, per_sm);
   const ClusterLaunch Q{L, g_next, flags_next, m, bodies, list, mesh, boxes, cap, interp, forces, spread};
   const size_t smem = 4 * fixed + 12 * (size_t)cap;
   if (membranes) launch_kind<1>(Q, n, smem, programmatic, st);

@@ -47,10 +47,11 @@ void launch_couple(const LatticeDev& L, float4* g_next, const MarkersDev& m, Bod
 
 // cluster.cu (few bodies: a cluster of thread blocks per body)
 cudaError_t cluster_configure();
-int cluster_box_cells(size_t fixed_words, int n_clusters, int n_sm);
+cudaError_t cluster_capacity(int per_sm, int* out);
+int cluster_box_cells(size_t fixed_words, int per_sm);
 void launch_couple_cluster(const LatticeDev& L, float4* g_next, uint8_t* flags_next, const MarkersDev& m,
                            BodyDev* bodies, const int* list, int n, bool membranes, int max_count,
-                           const MeshDev& mesh, int4* boxes, int n_sm, bool interp, bool forces, bool spread,
+                           const MeshDev& mesh, int4* boxes, int per_sm, bool interp, bool forces, bool spread,
                            bool programmatic, cudaStream_t st);
 // many steps of the solid-only dynamics of few membranes in one launch
 bool solid_cluster_fits(const MeshDev& mesh);

@@ -453,7 +453,7 @@ int admit(ibm_lbm_server_t* s) {
     if (h->cluster_boxes && ensure_second_buffer(h)) {
       const int words = std::max(h->n_rigids ? cluster_fixed_words(h->cluster_max, 0, 0) : 0,
                                  h->n_membranes ? cluster_fixed_words(h->mesh.nv, h->mesh.nv, h->mesh.part_tris) : 0);
-      c->cluster_cap = cluster_box_cells(words, 1 << 20, h->n_sm);
+      c->cluster_cap = cluster_box_cells(words, CLUSTER_PER_SM);
     }
     c->h = h;
     c->held = ibm_lbm_device_bytes(h);

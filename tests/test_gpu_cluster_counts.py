@@ -1,0 +1,67 @@
+"""Couplings by clusters of thread blocks where the count of bodies changes
+how they run (Sec. 2.3): one or two blocks on an SM, and the counts around
+those the device holds at once (15 and 36 clusters on 152 SMs). The same steps
+as the stage interface, which takes the separate kernels; tolerances as in
+test_gpu_cluster.py."""
+import numpy as np
+import pytest
+
+from paper_1704_04551_gb300 import inputs as I
+from tests._cases import rel_l2
+
+pytestmark = pytest.mark.gpu
+
+LAT = dict(nx=50, ny=48, nz=46, tau=0.8, geometry=0, body_force=[2e-6, -1e-6, 5e-7])
+
+
+def _places(n):
+    k = int(np.ceil(n ** (1 / 3)))
+    i = np.arange(n)
+    return (np.stack([i % k, i // k % k, i // (k * k)], 1) + 0.5) * [50 / k, 48 / k, 46 / k]
+
+
+def _rigid(n, freq, direct):
+    rng = np.random.default_rng(2)
+    X, bodies, first = [], [], 0
+    for c in _places(n):
+        x, b = I.rigid_ellipsoid(c, (4.0, 3.5, 3.0), I.random_quaternion(rng), first, freq=freq, kappa=0.01,
+                                 direct=direct)
+        X.append(x)
+        bodies.append(dict(b, vel=(1e-3 * rng.standard_normal(3)).tolist()))
+        first += x.shape[1]
+    return dict(lattice=LAT, mesh=None, bodies=bodies, X=np.concatenate(X, axis=1))
+
+
+def _membranes(n, freq):
+    rest, tris = I.rbc_rest_shape(9.0, freq)
+    V = rest.shape[1]
+    rng = np.random.default_rng(3)
+    X = [rest * np.exp(rng.uniform(-0.05, 0.05, (3, 1))) + c[:, None] for c in _places(n)]
+    bodies = [I._body(I.BODY_MEMBRANE, k * V, V, kBT_p=1e-3, k_b=5e-4, k_l=3e-3, k_g=2e-3, k_v=2e-3) for k in range(n)]
+    return dict(lattice=LAT, mesh=dict(rest_X=rest, tris=tris), bodies=bodies, X=np.concatenate(X, axis=1))
+
+
+def _match_stages(cuda_lib, w):
+    a, b = cuda_lib.Simulation.from_workload(w), cuda_lib.Simulation.from_workload(w)
+    for n in (1, 18):
+        a.step(n)
+        for _ in range(n):
+            for st in (cuda_lib.STAGE_FORCES, cuda_lib.STAGE_SPREAD, cuda_lib.STAGE_COLLIDE, cuda_lib.STAGE_INTERP):
+                b.stage(st)
+    (Xa, _, Fa), (Xb, _, Fb) = a.markers(), b.markers()
+    assert np.abs(Fa).max() > 1e-6
+    assert rel_l2(a.fields()[1], b.fields()[1]) < 1e-6
+    assert np.abs(Xa - Xb).max() < 1e-7
+    assert np.abs(Fa - Fb).max() < 1e-4 * np.abs(Fb).max()
+    assert np.abs(a.force_density()).max() == 0.0
+
+
+@pytest.mark.parametrize('n,freq,direct', [(15, 4, False), (16, 4, False), (36, 4, True), (37, 4, True),
+                                           (37, 6, False), (72, 6, False), (73, 6, False)])
+def test_rigid_counts_match_stages(cuda_lib, n, freq, direct):
+    _match_stages(cuda_lib, _rigid(n, freq, direct))
+
+
+@pytest.mark.parametrize('n,freq', [(1, 4), (15, 6), (16, 6), (16, 8), (36, 8), (37, 8)])
+def test_membrane_counts_match_stages(cuda_lib, n, freq):
+    _match_stages(cuda_lib, _membranes(n, freq))
