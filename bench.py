@@ -407,11 +407,14 @@ def kernels_per_step(w):
 
 def clustered_path(w):
     """Whether ibm_lbm_step couples workload w by clusters of blocks: rigid
-    bodies of any number and membranes up to 38, nothing else."""
+    bodies of any number and membranes up to what the device holds at once (15
+    clusters with one block on an SM, 36 with two), nothing else."""
     kinds = [b['kind'] for b in w['bodies']]
     if not kinds or (w.get('morse') or {}).get('rc', 0) > 0 or any(k == 2 for k in kinds):
         return False
-    return (sum(b['count'] for b in w['bodies']) == w['X'].shape[1] and kinds.count(0) <= 38
+    nv = max([b['count'] for b in w['bodies'] if b['kind'] == 0], default=0)
+    most = 36 if nv >= 512 or kinds.count(0) < len(kinds) else 15 if nv >= 256 else 0
+    return (sum(b['count'] for b in w['bodies']) == w['X'].shape[1] and kinds.count(0) <= most
             and max(b['count'] for b in w['bodies']) <= 4096)
 
 

@@ -176,10 +176,24 @@ int tiles(const LatticeDev& L) { return L.ntx * L.nty * L.ntz; }
 // tile flags) that the next collision reads; the buffers alternate.
 enum Path { SEPARATE, FUSED, CLUSTERED };
 
-// Membranes take clusters up to this many bodies. One block per body
-// (couple.cu) does less work in all, but its latency decides while the
-// bodies do not fill the chip.
-constexpr int CLUSTER_MEMBRANES_MAX = 38;
+// Up to how many membranes of nv vertices clusters pay. One block per body
+// (couple.cu; over ~938 vertices the separate kernels) does less work in all,
+// but its latency decides while the bodies do not fill the chip, the more so
+// the larger the template. us a step in a lattice with n bodies, clusters / one
+// block (152 SMs: 15 clusters at one block an SM, 36 at two):
+//   vertices     n = 1       n = 15      n = 16      n = 36      n = 38
+//     42      30.1/29.0   35.8/32.4   37.0/31.6   43.5/35.3   65.9/35.2
+//    162      33.1/32.2   38.3/35.3   40.2/34.8   46.9/38.4   71.3/38.3
+//    362      34.4/37.5   39.6/40.9   42.3/40.6   48.4/44.4   77.0/44.2
+//    642      36.3/43.8   41.2/47.7   44.8/47.5   51.6/51.8   81.6/51.9
+//   1442      42.0/71.7   47.4/79.5   52.5/79.8   59.6/83.7   94.4/83.7
+//   2562      49.7/91.7   53.8/96.9   82.9/96.9    101/101     126/101
+// Beside rigid bodies, and in a server, there is no kernel of one block per
+// body that couples, only the separate ones: clusters are better in one wave.
+int membrane_clusters_max(const ibm_lbm_t* h, int nv) {
+  if (nv >= 512 || h->n_rigids > 0 || h->served) return h->clusters_two;
+  return nv >= 256 ? h->clusters_one : 0;
+}
 // The solid-only dynamics of a launch, and up to how many membranes it takes
 // clusters.
 constexpr int64_t SOLID_CHUNK = 512;
@@ -1224,7 +1238,7 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.off_vt_start = section(vts.data(), vts.size() * 2);
     D.off_vt = section(vtl.data(), vtl.size() * 2);
     const size_t whole = buf.size();
-    if (!h->lean && h->n_membranes <= std::max(CLUSTER_MEMBRANES_MAX, SOLID_MEMBRANES_MAX)) {
+    if (!h->lean && h->n_membranes <= SOLID_MEMBRANES_MAX) {  // (couplings: fewer)
       // parts of consecutive vertices for the clusters (cluster_body.cuh)
       int table[CLUSTER][8] = {};
       D.part_tris = 0;
@@ -1367,7 +1381,8 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
   }
   // clusters: bodies of a size one cluster takes, nothing else
   if (!h->lean) {
-    bool few = n_bodies > 0 && covered == n_markers && h->n_filaments == 0 && h->n_membranes <= CLUSTER_MEMBRANES_MAX;
+    bool few = n_bodies > 0 && covered == n_markers && h->n_filaments == 0 &&
+               h->n_membranes <= membrane_clusters_max(h, h->mesh.nv);
     for (int b = 0; b < n_bodies && few; ++b) {
       few = bodies[b].count <= CLUSTER_MAX_COUNT;
       h->cluster_max = std::max(h->cluster_max, (int)bodies[b].count);

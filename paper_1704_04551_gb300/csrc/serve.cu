@@ -424,6 +424,7 @@ int admit(ibm_lbm_server_t* s) {
     if (rc == IBM_LBM_OK)
       rc = ibm_lbm_set_lattice(h, c->rho0.empty() ? nullptr : c->rho0.data(), c->u0.empty() ? nullptr : c->u0.data());
     if (rc == IBM_LBM_OK) {
+      h->served = true;
       h->lean = c->lean;
       ibm_lbm_mesh mesh{c->nv, c->nt, c->tris.data(), c->rest.data()};
       const int64_t M = (int64_t)(c->X.size() / 3);
