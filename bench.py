@@ -407,14 +407,19 @@ def kernels_per_step(w):
 
 def clustered_path(w):
     """Whether ibm_lbm_step couples workload w by clusters of blocks: rigid
-    bodies of any number and membranes up to what the device holds at once (15
-    clusters with one block on an SM, 36 with two), nothing else."""
+    bodies and membranes up to what the device holds at once (15 clusters with
+    one block on an SM, 36 with two; tethered bodies of middling size in two
+    waves), nothing else."""
     kinds = [b['kind'] for b in w['bodies']]
     if not kinds or (w.get('morse') or {}).get('rc', 0) > 0 or any(k == 2 for k in kinds):
         return False
     nv = max([b['count'] for b in w['bodies'] if b['kind'] == 0], default=0)
     most = 36 if nv >= 512 or kinds.count(0) < len(kinds) else 15 if nv >= 256 else 0
+    rigid = [b for b in w['bodies'] if b['kind'] != 0]
+    tethers = all(b['kind'] == 1 and 256 <= b['count'] <= 3072 for b in rigid)
+    at_most = 36 if not tethers else 54 if any(b['count'] < 512 for b in rigid) else 72
     return (sum(b['count'] for b in w['bodies']) == w['X'].shape[1] and kinds.count(0) <= most
+            and len(rigid) <= at_most
             and max(b['count'] for b in w['bodies']) <= 4096)
 
 

@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <array>
+#include <climits>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -193,6 +194,27 @@ enum Path { SEPARATE, FUSED, CLUSTERED };
 int membrane_clusters_max(const ibm_lbm_t* h, int nv) {
   if (nv >= 512 || h->n_rigids > 0 || h->served) return h->clusters_two;
   return nv >= 256 ? h->clusters_one : 0;
+}
+// Up to how many rigid bodies of [least, most] markers clusters pay against the
+// separate kernels (a block per body and stage). us a step in a lattice with n
+// tethered bodies, clusters / separate:
+//   markers      n = 1      n = 28      n = 38      n = 57      n = 72      n = 76     n = 1000
+//     92      15.7/34.4  20.3/35.1   34.9/35.1   35.8/35.5   49.9/35.7   51.0/35.9   471/153
+//    362      20.2/47.3  28.3/52.0   47.8/51.9   49.2/52.1   58.6/55.6   71.1/55.8   700/305
+//    812      21.1/63.5  30.3/70.6   53.0/70.6   53.8/71.5   63.1/75.4   78.4/75.4   784/395
+//   2562      36.8/92.0  53.3/101    97.0/101    98.5/122     108/139     137/139
+//   4002      49.4/111   72.3/119     132/120     135/155     147/164     187/164
+// and direct forcing, whose clusters wait for the new pose before they spread:
+//    362      30.3/49.2  39.9/54.6   70.3/54.8   72.9/55.3   81.8/58.8    101/58.6   998/326
+//    812      32.2/70.3  42.8/75.5   76.0/75.6   78.9/76.2   86.6/80.1    109/80.0  1064/422
+// One wave of clusters always wins; two (half a second one from 256 markers)
+// win for tethered bodies of a size that is neither launch-bound nor a large
+// scatter.
+int rigid_clusters_max(const ibm_lbm_t* h, int least, int most, bool direct) {
+  if (h->served) return INT_MAX;
+  const int two = h->clusters_two;
+  if (direct || least < 256 || most > 3072) return two;
+  return least < 512 ? two + two / 2 : 2 * two;
 }
 // The solid-only dynamics of a launch, and up to how many membranes it takes
 // clusters.
@@ -1383,10 +1405,18 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
   if (!h->lean) {
     bool few = n_bodies > 0 && covered == n_markers && h->n_filaments == 0 &&
                h->n_membranes <= membrane_clusters_max(h, h->mesh.nv);
+    int least_rigid = INT_MAX, most_rigid = 0;
+    bool direct = false;
     for (int b = 0; b < n_bodies && few; ++b) {
+      const int count = (int)bodies[b].count;
       few = bodies[b].count <= CLUSTER_MAX_COUNT;
-      h->cluster_max = std::max(h->cluster_max, (int)bodies[b].count);
+      h->cluster_max = std::max(h->cluster_max, count);
+      if (bodies[b].kind == IBM_LBM_BODY_MEMBRANE) continue;
+      least_rigid = std::min(least_rigid, count);
+      most_rigid = std::max(most_rigid, count);
+      direct |= bodies[b].kind == IBM_LBM_BODY_RIGID_DIRECT;
     }
+    few = few && h->n_rigids <= rigid_clusters_max(h, least_rigid, most_rigid, direct);
     few = few && (h->n_rigids == 0 ||
                   cluster_box_cells(cluster_fixed_words(h->cluster_max, 0, 0), per_sm(h, h->n_rigids)) > 0);
     few = few && (h->n_membranes == 0 ||

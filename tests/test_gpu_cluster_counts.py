@@ -57,7 +57,7 @@ def _match_stages(cuda_lib, w):
 
 
 @pytest.mark.parametrize('n,freq,direct', [(15, 4, False), (16, 4, False), (36, 4, True), (37, 4, True),
-                                           (37, 6, False), (72, 6, False), (73, 6, False)])
+                                           (37, 6, False), (54, 6, False), (72, 8, False), (73, 8, False)])
 def test_rigid_counts_match_stages(cuda_lib, n, freq, direct):
     _match_stages(cuda_lib, _rigid(n, freq, direct))
 
@@ -65,3 +65,15 @@ def test_rigid_counts_match_stages(cuda_lib, n, freq, direct):
 @pytest.mark.parametrize('n,freq', [(1, 4), (15, 6), (16, 6), (16, 8), (36, 8), (37, 8)])
 def test_membrane_counts_match_stages(cuda_lib, n, freq):
     _match_stages(cuda_lib, _membranes(n, freq))
+
+
+@pytest.mark.parametrize('n,freq,direct,clusters', [(30, 4, True, True), (200, 4, False, False), (200, 6, False, False),
+                                                    (100, 6, True, False)])
+def test_many_rigid_bodies_take_the_separate_kernels(cuda_lib, n, freq, direct, clusters):
+    """Clusters need a second force density from the second step on; the
+    separate kernels, which many bodies take, need none."""
+    sim = cuda_lib.Simulation.from_workload(_rigid(n, freq, direct))
+    held = sim.device_bytes
+    sim.step(4)
+    assert (sim.device_bytes - held >= 16 * sim.N) == clusters
+    assert clusters or sim.device_bytes == held
