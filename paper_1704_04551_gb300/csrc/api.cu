@@ -240,9 +240,12 @@ LatticeDev lattice_of(const ibm_lbm_t* h, Path p, int k) {
 // lattice with fluid), nothing timed between them, and a small lattice: at 32^3
 // a step goes from 22.5 to 20.5 us, but blocks that wait in residence cost a
 // collision of many waves more than the gap between two kernels (256^3 tube:
-// 187 -> 206 ms per 200 steps).
+// 187 -> 206 ms per 200 steps). Nor where the clusters fill the device: blocks
+// of a collision that waits take the places of some, which then run as a second
+// wave (60^3, 36 tethered bodies of 812 markers: 52 us a step, ordered 33).
 bool chained(const ibm_lbm_t* h) {
-  return !h->timing && h->n_rows > 0 && h->L.N <= CHAINED_CELLS_MAX && (h->n_rigids > 0) != (h->n_membranes > 0);
+  return !h->timing && h->n_rows > 0 && h->L.N <= CHAINED_CELLS_MAX && (h->n_rigids > 0) != (h->n_membranes > 0) &&
+         leaves_room(h->n_rigids + h->n_membranes, h->clusters_two);
 }
 
 // Blocks of n clusters on an SM: one while they are all resident so, for

@@ -17,6 +17,12 @@ constexpr int MAX_MESH_VERTICES = 4096;
 constexpr int CHAINED_CELLS_MAX = 1 << 18;  // collision and coupling start ahead of one another (api.cu, chained)
 constexpr int BODY_GROUP = 1024;   // markers per transfer block within a body
 
+// n clusters of `most` the device holds: few enough to start beside a collision
+// whose blocks are still there (api.cu, chained). 50^3 and 60^3 lattices,
+// n of 36, ahead / in order: 31 bodies 30.3/30.6 and 30.2/32.2 us a step, 32:
+// 33.3/30.7 and 31.5/32.2, 34: 48.0/30.6 and 45.6/32.4.
+inline bool leaves_room(int n, int most) { return 8 * n <= 7 * most; }
+
 struct Alloc {
   void* p;
   size_t bytes;

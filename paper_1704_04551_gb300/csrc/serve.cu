@@ -588,7 +588,8 @@ int rebuild(ibm_lbm_server_t* s) {
   for (int gm = 0; gm < 3; ++gm) geometries += s->geom_first[gm + 1] > s->geom_first[gm];
   size_t cells = 0;
   for (const CaseDev& C : s->h_cases) cells += C.n_cells;
-  const bool chained = !separate && geometries == 1 && cells <= (size_t)CHAINED_CELLS_MAX && (n_cr > 0) != (n_cm > 0);
+  const bool chained = !separate && geometries == 1 && cells <= (size_t)CHAINED_CELLS_MAX && (n_cr > 0) != (n_cm > 0) &&
+                       leaves_room(n_cr + n_cm, s->running[0]->h->clusters_two);
   auto couple = [&](int step) {
     const bool ahead = chained && step >= 0;
     if (n_cr)
