@@ -216,10 +216,19 @@ int rigid_clusters_max(const ibm_lbm_t* h, int least, int most, bool direct) {
   if (direct || least < 256 || most > 3072) return two;
   return least < 512 ? two + two / 2 : 2 * two;
 }
-// The solid-only dynamics of a launch, and up to how many membranes it takes
-// clusters.
+// Steps of the solid-only dynamics in one launch of clusters, and up to how
+// many membranes of nv vertices they take it. A wave holds clusters_one of them
+// (a block on an SM each), and takes 7 us a step (42 vertices) to 14 (2562); the
+// general path (a block per body, three launches) grows slowly with the count.
+// us a step, clusters / general:
+//   vertices    n = 15     n = 30     n = 45     n = 60     n = 75     n = 90     n = 120
+//     42       6.9/15.6  13.7/16.8  20.5/16.7  27.2/16.6  34.0/17.0  40.8/17.4  54.3/16.6
+//    252       7.2/19.7  14.3/20.7  21.2/20.4  28.4/22.8  35.4/22.8  42.3/22.8  56.4/26.9
+//    642       8.4/26.9  16.5/28.9  24.6/33.0  32.8/33.0  40.9/35.1  49.0/39.2  65.2/41.5
+//   1442      11.4/41.0  22.6/47.2  34.0/53.3  45.1/55.6  56.3/61.9  67.7/66.7  89.9/77.3
+//   2562      14.4/60.1  28.6/70.4  42.8/80.3  57.0/85.9  71.2/95.6   85.3/105   113/122
 constexpr int64_t SOLID_CHUNK = 512;
-constexpr int SOLID_MEMBRANES_MAX = 128;
+int solid_clusters_max(const ibm_lbm_t* h, int nv) { return (2 + nv / 400) * h->clusters_one; }
 
 Path path_of(const ibm_lbm_t* h) {
   if (h->m.M == 0 || h->morse_rc > 0.0) return SEPARATE;
@@ -1263,7 +1272,8 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.off_vt_start = section(vts.data(), vts.size() * 2);
     D.off_vt = section(vtl.data(), vtl.size() * 2);
     const size_t whole = buf.size();
-    if (!h->lean && h->n_membranes <= SOLID_MEMBRANES_MAX) {  // (couplings: fewer)
+    if (!h->lean &&
+        h->n_membranes <= std::max(membrane_clusters_max(h, mesh->n_vertices), solid_clusters_max(h, mesh->n_vertices))) {
       // parts of consecutive vertices for the clusters (cluster_body.cuh)
       int table[CLUSTER][8] = {};
       D.part_tris = 0;
@@ -1486,10 +1496,10 @@ static int impl_ibm_lbm_solid_steps(ibm_lbm_t* h, int64_t n_steps, double dt, do
     }
   }
   // Few membranes and nothing else: a cluster per body, SOLID_CHUNK steps a
-  // launch (a few ms). Its work is ~1.5 times that of one block per body and
-  // its latency a tenth: better while the clusters fill the chip a few times.
+  // launch (a few ms).
   const bool clusters = h->n_membranes > 0 && h->n_membranes == h->n_bodies && !h->need_zero_F &&
-                        !(h->morse_rc > 0.0) && h->mesh.part_tris > 0 && solid_cluster_fits(h->mesh);
+                        !(h->morse_rc > 0.0) && h->n_membranes <= solid_clusters_max(h, h->mesh.nv) &&
+                        h->mesh.part_tris > 0 && solid_cluster_fits(h->mesh);
   if (clusters) {
     for (int64_t s = 0; s < n_steps; s += SOLID_CHUNK)
       launch_solid_cluster(h->m, h->d_bodies, h->membrane_list, h->n_membranes, h->mesh, h->solid_v, fe, dt, gamma,

@@ -7,6 +7,7 @@ import numpy as np
 import pytest
 
 from paper_1704_04551_gb300 import inputs as I
+from tests import test_gpu_solid
 from tests._cases import rel_l2
 
 pytestmark = pytest.mark.gpu
@@ -77,3 +78,9 @@ def test_many_rigid_bodies_take_the_separate_kernels(cuda_lib, n, freq, direct, 
     sim.step(4)
     assert (sim.device_bytes - held >= 16 * sim.N) == clusters
     assert clusters or sim.device_bytes == held
+
+
+# clusters in one wave, in two, and the general path
+@pytest.mark.parametrize('freq,bodies', [(2, 15), (2, 30), (2, 31), (6, 45)])
+def test_solid_counts_match_oracle(cuda_lib, freq, bodies):
+    test_gpu_solid.test_solid_steps_of_several_bodies_match_oracle(cuda_lib, freq, bodies, (1, 7))
