@@ -191,8 +191,15 @@ enum Path { SEPARATE, FUSED, CLUSTERED };
 //   2562      49.7/91.7   53.8/96.9   82.9/96.9    101/101     126/101
 // Beside rigid bodies, and in a server, there is no kernel of one block per
 // body that couples, only the separate ones: clusters are better in one wave.
+// A server's wave is that of all its cases. A case's path must not depend on
+// what else is served, so the slots count, not the cases there are. us a step,
+// clusters / separate, cases x membranes of 642 vertices: 8 x 1 55.5/76.8, 8 x 3
+// 62.2/79.7, 32 x 1 153/169, 16 x 3 138/117, 8 x 8 108/86.1, 64 x 1 299/275, 64 x 8
+// 804/393 (a server of 64 slots may hold few: 4 x 1 44.5/62.8).
+constexpr int SERVED_MAX = 64;
 int membrane_clusters_max(const ibm_lbm_t* h, int nv) {
-  if (nv >= 512 || h->n_rigids > 0 || h->served) return h->clusters_two;
+  if (h->served_slots > 0) return (nv >= 512 && h->n_membranes == 1 ? SERVED_MAX : h->clusters_two) / h->served_slots;
+  if (nv >= 512 || h->n_rigids > 0) return h->clusters_two;
   return nv >= 256 ? h->clusters_one : 0;
 }
 // Up to how many rigid bodies of [least, most] markers clusters pay against the
@@ -209,9 +216,13 @@ int membrane_clusters_max(const ibm_lbm_t* h, int nv) {
 //    812      32.2/70.3  42.8/75.5   76.0/75.6   78.9/76.2   86.6/80.1    109/80.0  1064/422
 // One wave of clusters always wins; two (half a second one from 256 markers)
 // win for tethered bodies of a size that is neither launch-bound nor a large
-// scatter.
+// scatter. In a server of shear cells with one body each (24^3 to 64^3), cells of
+// 92 and of 812 markers: 24 118/130 and 121/163, 48 215/207 and 223/241, 64 277/257
+// and 283/292, 80 349/323 and 365/359, 128 538/485 and 557/521, 512 1962/1749 and
+// 2031/1866; eight bodies of 812 markers in 8 cells 78.1/90.3, in 16 161/125: up to
+// 64 bodies over its slots.
 int rigid_clusters_max(const ibm_lbm_t* h, int least, int most, bool direct) {
-  if (h->served) return INT_MAX;
+  if (h->served_slots > 0) return SERVED_MAX / h->served_slots;
   const int two = h->clusters_two;
   if (direct || least < 256 || most > 3072) return two;
   return least < 512 ? two + two / 2 : 2 * two;
@@ -1273,7 +1284,8 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     D.off_vt = section(vtl.data(), vtl.size() * 2);
     const size_t whole = buf.size();
     if (!h->lean &&
-        h->n_membranes <= std::max(membrane_clusters_max(h, mesh->n_vertices), solid_clusters_max(h, mesh->n_vertices))) {
+        h->n_membranes <= std::max(membrane_clusters_max(h, mesh->n_vertices),
+                                   h->served_slots > 0 ? 0 : solid_clusters_max(h, mesh->n_vertices))) {
       // parts of consecutive vertices for the clusters (cluster_body.cuh)
       int table[CLUSTER][8] = {};
       D.part_tris = 0;

@@ -85,7 +85,7 @@ struct ibm_lbm {
   // does the same (cluster_body.cuh); boxes of its blocks [n_bodies][CLUSTER][2].
   int4* cluster_boxes = nullptr;  // set: the path applies to these markers
   int cluster_max = 0;            // largest marker count of a body
-  bool served = false;            // a case of a server, which couples it in batched launches
+  int served_slots = 0;           // > 0: a case of a server with so many, which couples all in batched launches
   bool lean = false;              // markers set without what only clusters need
   uint8_t* fbuf2 = nullptr;       // second tile flags (beside gbuf2)
   bool density_waiting = false;   // a SPREAD stage's force density is in gbuf, for the next step

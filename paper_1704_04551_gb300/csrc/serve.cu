@@ -12,7 +12,8 @@
 // from which a kernel derives whether a case takes part in a step of the chunk
 // and whether it is its last one (dense moments). Cases whose bodies take
 // clusters (cluster_body.cuh) need two launches a step, collision and coupling;
-// the others, with tracers or large suspensions, run the separate stages. A
+// the others, with tracers, large suspensions or in a server of many slots (api.cu,
+// rigid_clusters_max, membrane_clusters_max), run the separate stages. A
 // chunk of steps is captured once per set of admitted cases and replayed as
 // a CUDA graph; a case that reaches its step count mid-chunk is skipped for
 // the rest of it. Between chunks finished cases are retired (results copied
@@ -424,7 +425,7 @@ int admit(ibm_lbm_server_t* s) {
     if (rc == IBM_LBM_OK)
       rc = ibm_lbm_set_lattice(h, c->rho0.empty() ? nullptr : c->rho0.data(), c->u0.empty() ? nullptr : c->u0.data());
     if (rc == IBM_LBM_OK) {
-      h->served = true;
+      h->served_slots = s->cfg.max_active;
       h->lean = c->lean;
       ibm_lbm_mesh mesh{c->nv, c->nt, c->tris.data(), c->rest.data()};
       const int64_t M = (int64_t)(c->X.size() / 3);
