@@ -1136,6 +1136,31 @@ static void clear_markers(ibm_lbm_t* h) {
   h->need_zero_F = false;
 }
 
+// Lattices of more cells mark packed tracers' tiles (see set_markers_into).
+constexpr int PACKED_TRACERS_CELLS = 1 << 23;
+
+// Whether tracers lie in a sixteenth of the tiles or more.
+static bool tracers_scattered(const ibm_lbm_t* h, const std::vector<MarkerGroup>& groups, const double* X, int M) {
+  const LatticeDev& L = h->L;
+  const int n[3] = {L.nx, L.ny, L.nz}, shift[3] = {TILE_X_SHIFT, TILE_Y_SHIFT, TILE_Z_SHIFT};
+  std::vector<char> seen((size_t)tiles(L), 0);
+  int64_t found = 0;
+  for (const MarkerGroup& G : groups)
+    for (int k = G.first; k < G.first + G.count; ++k) {
+      int t[3];
+      for (int a = 0; a < 3; ++a) {
+        const double x = X[a * (size_t)M + k];
+        const int c = (int)(x - n[a] * std::floor(x / n[a]));  // in [0, n]
+        t[a] = std::min(c, n[a] - 1) >> shift[a];
+      }
+      char& s = seen[(size_t)t[0] + (size_t)L.ntx * (t[1] + (size_t)L.nty * t[2])];
+      found += !s;
+      s = 1;
+      if (16 * found >= (int64_t)seen.size()) return true;
+    }
+  return false;
+}
+
 // set_markers after the old markers are gone; on error the caller clears
 // whatever this allocated, so that a failed call leaves no half-built state.
 static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bodies, const ibm_lbm_body* bodies,
@@ -1335,6 +1360,7 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     }
   }
   // transfer groups: bodies in chunks of BODY_GROUP, tracer runs in chunks of TRACER_GROUP
+  std::vector<MarkerGroup> tracer_groups;
   {
     std::vector<MarkerGroup> groups;
     std::vector<std::pair<int64_t, int>> cuts;  // (first marker, body) in marker order
@@ -1395,6 +1421,7 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
         if (!tracers) h->n_body_groups = (int)ordered.size();
       }
       groups.swap(ordered);
+      tracer_groups.assign(groups.begin() + h->n_body_groups, groups.end());
     }
     h->n_groups = (int)groups.size();
     if ((rc = upload<MarkerGroup>(h, h->marker_mem, &h->groups, groups.data(), groups.size()))) return rc;
@@ -1458,9 +1485,15 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
   }
   h->need_zero_F = covered < n_markers;
   // From a tracer per four tiles on the stencils (up to 8 tiles each) reach
-  // most of them: marking costs more than the velocities of the other cells (a
-  // 131x96x110 box with 150,000: 63 us against 16 bytes of 168 per cell).
-  h->tracers_everywhere = 4 * (n_markers - covered) >= (int64_t)tiles(h->L);
+  // most of them where they are scattered: marking costs more than the
+  // velocities of the other cells (a 131x96x110 box with 150,000: 63 us against
+  // 16 bytes of 168 per cell). Packed tracers are marked instead where those
+  // velocities do not stay in L2: us a step, marked / all velocities, tracers
+  // in 0, 7, 22 and 100 % of the tiles: 256^3, 20,000 of them 418/437, 426/440,
+  // 438/443, 469/444; 150,000 439/451, 470/456, 478/463, 536/492; 176^3, 2904
+  // 144/149, -, -, -, 150,000 170/164; 128^3, 20,000 67/66, 71/67, 77/67, 81/69.
+  h->tracers_everywhere = 4 * (n_markers - covered) >= (int64_t)tiles(h->L) &&
+                          (h->L.N <= PACKED_TRACERS_CELLS || tracers_scattered(h, tracer_groups, X, M));
   if (h->morse_rc > 0.0) return prepare_morse(h);
   return IBM_LBM_OK;
 }

@@ -54,3 +54,29 @@ def test_tracers_beside_bodies_match_oracle(cuda_lib, M):
     w = dict(w, lattice=lat, bodies=w['bodies'] + [rigid], X=np.concatenate([w['X'], R, T], axis=1))
     F = _check(cuda_lib.Simulation.from_workload(w), O.Oracle.from_workload(w), lat, 20)
     assert np.abs(F[:, -M:]).max() == 0.0 and np.abs(F[:, :n]).max() > 0.0
+
+
+@pytest.mark.parametrize('packed', [True, False])
+def test_many_tracers_of_a_large_lattice_match_stages(cuda_lib, packed):
+    """Past 2^23 cells packed tracers are marked, scattered ones are not; the
+    stage interface, which computes every velocity, moves them the same way
+    (the same arithmetic; populations FP32 in both)."""
+    lat = dict(nx=256, ny=188, nz=178, tau=0.8, geometry=0, body_force=[2e-6, -1e-6, 5e-7])
+    n = np.array(shape(lat), float)[:, None]
+    M = 4400  # tiles: 16920
+    rng = np.random.default_rng(5)
+    X = (0.5 * n + 6.0 * (2 * rng.random((3, M)) - 1)) if packed else n * rng.random((3, M))
+    X[:, :40] = rng.uniform(-3.0, 3.0, (3, 40))  # a few across the boundaries
+    u = 0.02 * rng.standard_normal((3, 1)) * np.ones((3, int(n.prod())))
+    a, b = cuda_lib.Simulation(lat), cuda_lib.Simulation(lat)
+    for s in (a, b):
+        s.set_lattice(None, u)
+        s.set_markers(None, [], X)
+    a.step(5)
+    for _ in range(5):
+        for st in (cuda_lib.STAGE_FORCES, cuda_lib.STAGE_SPREAD, cuda_lib.STAGE_COLLIDE, cuda_lib.STAGE_INTERP):
+            b.stage(st)
+    (Xa, Ua, _), (Xb, Ub, _) = a.markers(), b.markers()
+    assert np.abs(Xa - X).max() > 1e-3
+    assert np.abs(Xa - Xb).max() < 1e-7 and rel_l2(Ua, Ub) < 1e-6
+    assert rel_l2(a.fields()[1], b.fields()[1]) < 1e-6
