@@ -343,7 +343,9 @@ const char* ibm_lbm_server_last_error(const ibm_lbm_server_t* s);
  * density, N = nx*ny*nz, fully overwritten (cells outside every stencil get
  * 0). geometry / tube_radius as in ibm_lbm_config; stream is a cudaStream_t
  * or NULL. The call only enqueues work on the stream and returns; g is ready
- * when the stream reaches that point.
+ * when the stream reaches that point. The work is one cooperative kernel of up
+ * to four thread blocks of 256 threads on every SM: beside other work on the
+ * GPU it starts when all its blocks fit at once.
  * Every call looks up the array's device address in the current context
  * (so a device reset by the caller is safe); the first call on a device may
  * load the library's device code there, so make it before any stream

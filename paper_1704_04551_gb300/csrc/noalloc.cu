@@ -156,15 +156,17 @@ int spread_noalloc(const double* X, const double* F, int64_t n_markers, int32_t 
   }
   // all blocks resident at once (grid barrier); fewer where there is little to do
   const long long work = std::max((N + 1) / 2, (long long)M * SPREAD_LANES);
-  const unsigned blocks = (unsigned)std::min<long long>((work + SPREAD_THREADS - 1) / SPREAD_THREADS,
-                                                        (long long)sms * SPREAD_BLOCKS_PER_SM);
+  unsigned blocks = (unsigned)std::min<long long>((work + SPREAD_THREADS - 1) / SPREAD_THREADS,
+                                                  (long long)sms * SPREAD_BLOCKS_PER_SM);
   void* args[] = {&G, &X, &F, &M, &acc, &g};
-  if (cudaLaunchCooperativeKernel((const void*)k_spread_noalloc, dim3(blocks), dim3(SPREAD_THREADS), args, 0, st) !=
-      cudaSuccess) {
+  // (a context may have fewer SMs than the device; the kernel's loops cover any grid)
+  for (;; blocks = (blocks + 1) / 2) {
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_spread_noalloc, dim3(blocks),
+                                                      dim3(SPREAD_THREADS), args, 0, st);
+    if (e == cudaSuccess) return IBM_LBM_OK;
     cudaGetLastError();
-    return IBM_LBM_E_CUDA;
+    if (e != cudaErrorCooperativeLaunchTooLarge || blocks == 1) return IBM_LBM_E_CUDA;
   }
-  return IBM_LBM_OK;
 }
 }  // namespace
 
