@@ -100,6 +100,17 @@ bool pages_mapped(const void* p, size_t bytes, size_t page) {
   return true;
 }
 
+// Whether a caller's buffer is ordinary host memory. A copy also takes device,
+// managed and pinned memory, whose pages are not to be touched from here.
+bool pageable(const void* p) {
+  cudaPointerAttributes a{};
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeUnregistered;
+}
+
 // Take the page faults of a host buffer before a copy, which would fault its
 // pages one by one from the device's side: one byte per page is written (an
 // output that is about to be overwritten) or read (an input), by several
@@ -110,7 +121,7 @@ bool pages_mapped(const void* p, size_t bytes, size_t page) {
 // less than the threads below (get_fields of a 77x94x67 lattice into arrays in
 // use before: 0.14 of 1.88 ms of a two-step run).
 void touch_pages(const void* p, size_t bytes, bool write) {
-  if (!p || bytes < ((size_t)64 << 10)) return;
+  if (!p || bytes < ((size_t)64 << 10) || !pageable(p)) return;
   const long pg = sysconf(_SC_PAGESIZE);
   const size_t page = pg > 0 ? (size_t)pg : 4096;
   if (bytes < ((size_t)16 << 20) && pages_mapped(p, bytes, page)) return;
