@@ -218,7 +218,7 @@ __device__ __forceinline__ void couple_membrane(const LatticeDev& L, float4* g_n
   // by residue now, while the membrane part runs
   const long long ex = (long long)s_hi[0] - s_lo[0] + 4, ey = (long long)s_hi[1] - s_lo[1] + 4,
                   ez = (long long)s_hi[2] - s_lo[2] + 4;
-  const int kind = box_kind(ex, ey, ez);
+  const int kind = box_kind(ex, ey, ez, slab_budget_fused(nv));
   const bool fits = kind != 0;
   const int4 dims2 = make_int4(fits ? (int)ex : 0, fits ? (int)ey : 0, fits ? (int)ez : 0, kind);
   int l2[COUPLE_PER_THREAD];

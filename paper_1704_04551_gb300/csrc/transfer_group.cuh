@@ -79,14 +79,43 @@ constexpr int SPREAD_LANES_SMEM = 3 * BOX_CELLS * (int)sizeof(int);
 // one; the scatter's do not, and a marker adds the layers that a slab holds.
 // (A tumbling red cell's box reaches ~6800 cells. Per-marker global atomics and
 // gathers, the path of every larger box, made one such body set the time of
-// the fused kernel: 207 instead of 47 us per 64^3 step.) box_kind: 1 whole,
-// 2 in slabs, 0 neither.
+// the fused kernel: 207 instead of 47 us per 64^3 step.) Slabs cost by the
+// cells, which the gather loads with their overlaps and the scatter clears and
+// flushes, the other way by the markers: a box with more cells in all than
+// `budget`, a line in the group's markers for each family of kernels, takes
+// the latter. box_kind: 1 whole, 2 in slabs, 0 neither.
+//
+// us a step, slabs / marker by marker, spheres of radius R (a box of (2R + 4.5)^3
+// cells; over R = 13.7 the layers leave five in a slab, two of them new):
+//   few groups, four lanes a marker (60 - 80 bodies):
+//     markers    R = 7.3     R = 8.3    R = 9.5     R = 11      R = 14
+//       162    73.1/68.0   87.8/81.9    108/95.0    136/112     261/167
+//       362    82.8/83.9   97.6/97.8    120/112     150/129     256/185
+//       812     103/117     117/134     142/147     173/164     296/221
+//      1442    93.7/113     105/122     128/135     165/150     316/175
+//   many groups, one thread a marker (520 - 540 bodies):
+//     markers    R = 8       R = 10      R = 12     R = 14      R = 16
+//        92                                        1044/984   1834/1275
+//       162     345/488     508/647     755/847    1066/1095   1892/1400
+//       362     380/729     550/925     802/1149   1125/1441   2001/1790
+//       812     447/1102    637/1386    902/1621   1250/1923   2253/2298
+//   the fused kernel (60 bodies):
+//     markers    R = 10      R = 12      R = 13.5   R = 14      R = 16
+//        92                               155/160    205/165
+//       252    94.0/144     136/176       172/198    229/203     389/235
+//       642     113/262     162/311       212/334    281/349     457/388
 constexpr int BOX_SLABBED = 8 * BOX_CELLS;
-__device__ __forceinline__ int box_kind(long long ex, long long ey, long long ez) {
+__device__ __forceinline__ float slab_budget_lanes(int markers) { return (float)(8200 + 30 * markers); }
+__device__ __forceinline__ float slab_budget_threads(int markers) { return (float)(90000 + 250 * markers); }
+__device__ __forceinline__ float slab_budget_fused(int markers) { return (float)(80000 + 110 * markers); }
+__device__ __forceinline__ int box_kind(long long ex, long long ey, long long ez, float budget) {
   if (ex <= 0 || ey <= 0 || ez <= 0 || ex > BOX_SLABBED || ey > BOX_SLABBED || ez > BOX_SLABBED) return 0;
-  const long long layer = ex * ey;
-  if (layer * ez <= BOX_CELLS) return 1;
-  return layer * 4 <= BOX_CELLS && layer * ez <= BOX_SLABBED ? 2 : 0;
+  if (ex * ey * ez <= BOX_CELLS) return 1;
+  if (ex * ey * 4 > BOX_CELLS || ex * ey * ez > BOX_SLABBED) return 0;
+  const float layer = (float)(int)(ex * ey), layers = (float)(int)ez;
+  const float depth = floorf(__fdividef((float)BOX_CELLS, layer));    // about 4 <= depth < layers
+  const float slabs = ceilf(__fdividef(layers - 3.0f, depth - 3.0f));  // of the gather
+  return layer * (layers + slabs * depth) <= budget ? 2 : 0;           // (false for no new layer in a slab)
 }
 // z layers a slab of the box holds (all of them for a box held whole)
 __device__ __forceinline__ int slab_depth(int4 dims) { return min(dims.z, BOX_CELLS / (dims.x * dims.y)); }
@@ -235,7 +264,8 @@ __device__ __forceinline__ void mark_box_tiles(const LatticeDev& L, int4 lo, int
 
 // Bounding box of the group's stencil nodes (unwrapped coordinates) and the
 // group's largest force component.
-__device__ inline void group_box(const MarkersDev& m, const MarkerGroup& G, int4& lo, int4& dims, float& fmax) {
+__device__ inline void group_box(const MarkersDev& m, const MarkerGroup& G, float budget, int4& lo,
+                                 int4& dims, float& fmax) {
   __shared__ int s_lo[3], s_hi[3];
   __shared__ unsigned s_fmax;
   if (threadIdx.x < 3) {
@@ -273,7 +303,7 @@ __device__ inline void group_box(const MarkersDev& m, const MarkerGroup& G, int4
   const long long ex = (long long)s_hi[0] - s_lo[0] + 4, ey = (long long)s_hi[1] - s_lo[1] + 4,
                   ez = (long long)s_hi[2] - s_lo[2] + 4;
   lo = make_int4(s_lo[0] - 1, s_lo[1] - 1, s_lo[2] - 1, 0);
-  const int kind = box_kind(ex, ey, ez);
+  const int kind = box_kind(ex, ey, ez, budget);
   dims = make_int4(kind ? (int)ex : 0, kind ? (int)ey : 0, kind ? (int)ez : 0, kind);
   fmax = __uint_as_float(s_fmax);
 }
@@ -543,7 +573,7 @@ __device__ __forceinline__ void spread_group(const LatticeDev& L, const MarkersD
                                              int4* box_out, unsigned char* smem) {
   int4 lo, dims;
   float fmax;
-  group_box(m, G, lo, dims, fmax);  // synchronises
+  group_box(m, G, slab_budget_threads(G.count), lo, dims, fmax);  // synchronises
   if (threadIdx.x == 0) {
     box_out[0] = lo;
     box_out[1] = dims;
@@ -746,7 +776,7 @@ __device__ __forceinline__ void spread_group_lanes(const LatticeDev& L, const Ma
                                                    int4* box_out, int* ibox) {
   int4 lo, dims;
   float fmax;
-  group_box(m, G, lo, dims, fmax);  // synchronises
+  group_box(m, G, slab_budget_lanes(G.count), lo, dims, fmax);  // synchronises
   if (threadIdx.x == 0) {
     box_out[0] = lo;
     box_out[1] = dims;

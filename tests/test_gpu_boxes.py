@@ -76,3 +76,37 @@ def test_transfer_in_slabs(cuda_lib, geom, n_clusters):
     Xo, Uo, _ = ora.markers()
     assert np.abs(Ug - Uo).max() < 2e-5 * np.abs(Uo).max()
     assert np.abs(Xg - Xo).max() < 1e-6
+
+
+# spheres around the size from which boxes are no longer worth slabs: with four
+# lanes a marker by their markers (362 and 812), with one block a membrane far
+# beyond (whose layers also leave the fewest new layers in a slab)
+@pytest.mark.parametrize('kind,n,freq,R', [('rigid', 75, 6, 7.3), ('rigid', 75, 6, 8.6), ('rigid', 75, 9, 9.5),
+                                           ('rigid', 75, 9, 10.6), ('membrane', 40, 3, 13.4), ('membrane', 40, 3, 14.2)])
+def test_spheres_around_the_slab_limit(cuda_lib, kind, n, freq, R):
+    S, tris = I.geodesic_sphere(freq)
+    V = S.shape[0]
+    rest = (R * S).T.copy()
+    lat = dict(nx=96, ny=90, nz=94, tau=1.0, geometry=0, body_force=[2e-6, 0, 0])
+    rng = np.random.default_rng(8)
+    C = rng.random((n, 3)) * [96, 90, 94]
+    if kind == 'membrane':
+        X = [rest * np.exp(rng.uniform(-0.02, 0.02, (3, 1))) + c[:, None] for c in C]
+        bodies = [I._body(I.BODY_MEMBRANE, k * V, V, kBT_p=1e-4, k_b=5e-5, k_l=3e-3, k_g=2e-3, k_v=2e-3)
+                  for k in range(n)]
+        mesh = dict(rest_X=rest, tris=tris)
+    else:
+        X, bodies, mesh = [], [], None
+        for k, c in enumerate(C):
+            x, b = I.rigid_ellipsoid(c, (R, R, R), I.random_quaternion(rng), k * V, freq=freq, kappa=0.02)
+            X.append(x)
+            bodies.append(dict(b, vel=(1e-3 * rng.standard_normal(3)).tolist()))
+    w = dict(lattice=lat, mesh=mesh, bodies=bodies, X=np.concatenate(X, axis=1))
+    sim, ora = cuda_lib.Simulation.from_workload(w), O.Oracle.from_workload(w)
+    sim.step(5)
+    ora.step(5)
+    (Xg, _, Fg), (Xo, _, Fo) = sim.markers(), ora.markers()
+    assert rel_l2(sim.fields()[1], ora.fields()[1]) < 1e-5
+    assert np.abs(Xg - Xo).max() < 1e-5
+    assert np.abs(Fg - Fo).max() < 1e-3 * np.abs(Fo).max()
+    assert np.abs(sim.force_density()).max() == 0.0
