@@ -1147,6 +1147,23 @@ static void clear_markers(ibm_lbm_t* h) {
   h->need_zero_F = false;
 }
 
+// Mean cells of the box of a body's stencils, over at most 64 of the bodies.
+static double mean_box(const ibm_lbm_body* bodies, int n, const double* X, int M) {
+  const int taken = std::min(n, 64);
+  double sum = 0.0;
+  for (int i = 0; i < taken; ++i) {
+    const ibm_lbm_body& B = bodies[(int64_t)i * n / taken];
+    double cells = 1.0;
+    for (int a = 0; a < 3; ++a) {
+      const double* x = X + a * (size_t)M + B.first;
+      const auto ends = std::minmax_element(x, x + B.count);
+      cells *= std::floor(*ends.second) - std::floor(*ends.first) + 4.0;
+    }
+    sum += cells;
+  }
+  return sum / taken;
+}
+
 // Lattices of more cells mark packed tracers' tiles (see set_markers_into).
 constexpr int PACKED_TRACERS_CELLS = 1 << 23;
 
@@ -1440,6 +1457,15 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
     // fused kernel, one transfer group per body
     bool fused = n_bodies > 0 && covered == n_markers && any_membrane && couple_fits(h->mesh);
     for (int b = 0; b < n_bodies && fused; ++b) fused = bodies[b].kind == IBM_LBM_BODY_MEMBRANE;
+    // While the separate kernels have four lanes a marker (few groups), they are
+    // the faster ones for large cells, whose slabs or markers one block works off
+    // alone. us a step, fused / separate, 60 spheres of radius 6, 8, 10, 14 (boxes
+    // of 4.5, 8.6, 14.7, 34 thousand cells): 92 vertices 33.5/34.5, 52.8/38.7,
+    // 83.5/58.1, 164/94; 252 39/42, 60/52, 94/70, 201/105; 642 50/60, 75/75, 114/102,
+    // 282/140; 812 54/68, 80/84, 122/121, 305/155; 250 of them with 642 116/138,
+    // 181/200, 271/271, 676/479; 520 (one thread a marker) 222/233, -, 544/545, 1253/1215.
+    if (fused && n_bodies < LANE_MAX_GROUPS)
+      fused = mean_box(bodies, n_bodies, X, M) <= BOX_CELLS + 8.0 * h->mesh.nv;
     if (fused) {
       std::unordered_map<int, int> body_of_first;
       for (int b = 0; b < n_bodies; ++b) body_of_first[(int)bodies[b].first] = b;
@@ -1480,6 +1506,10 @@ static int set_markers_into(ibm_lbm_t* h, const ibm_lbm_mesh* mesh, int32_t n_bo
       direct |= bodies[b].kind == IBM_LBM_BODY_RIGID_DIRECT;
     }
     few = few && h->n_rigids <= rigid_clusters_max(h, least_rigid, most_rigid, direct);
+    // a second wave of bodies whose boxes do not fit one block's shared memory
+    // loses to the separate kernels (60 of 36 x 24 x 24: 262 us a step, 254)
+    if (few && h->served_slots == 0 && h->n_rigids > h->clusters_two)
+      few = mean_box(bodies, n_bodies, X, M) <= BOX_CELLS;
     few = few && (h->n_rigids == 0 ||
                   cluster_box_cells(cluster_fixed_words(h->cluster_max, 0, 0), per_sm(h, h->n_rigids)) > 0);
     few = few && (h->n_membranes == 0 ||
