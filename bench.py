@@ -416,7 +416,7 @@ def clustered_path(w):
     nv = max([b['count'] for b in w['bodies'] if b['kind'] == 0], default=0)
     most = 36 if nv >= 512 or kinds.count(0) < len(kinds) else 15 if nv >= 256 else 0
     rigid = [b for b in w['bodies'] if b['kind'] != 0]
-    tethers = all(b['kind'] == 1 and 256 <= b['count'] <= 3072 for b in rigid)
+    tethers = len(rigid) == len(kinds) and all(b['kind'] == 1 and 256 <= b['count'] <= 3072 for b in rigid)
     at_most = 36 if not tethers else 54 if any(b['count'] < 512 for b in rigid) else 72
     return (sum(b['count'] for b in w['bodies']) == w['X'].shape[1] and kinds.count(0) <= most
             and len(rigid) <= at_most

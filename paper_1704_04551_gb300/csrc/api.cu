@@ -227,7 +227,9 @@ int membrane_clusters_max(const ibm_lbm_t* h, int nv) {
 //    812      32.2/70.3  42.8/75.5   76.0/75.6   78.9/76.2   86.6/80.1    109/80.0  1064/422
 // One wave of clusters always wins; two (half a second one from 256 markers)
 // win for tethered bodies of a size that is neither launch-bound nor a large
-// scatter. In a server of shear cells with one body each (24^3 to 64^3), cells of
+// scatter, but not beside membranes, whose clusters run after them while the
+// separate kernels take both at once (5 membranes of 642 vertices and 20 bodies
+// of 812: 77.9/91.6 us a step, and 40: 99.1/91.5). In a server of shear cells with one body each (24^3 to 64^3), cells of
 // 92 and of 812 markers: 24 118/130 and 121/163, 48 215/207 and 223/241, 64 277/257
 // and 283/292, 80 349/323 and 365/359, 128 538/485 and 557/521, 512 1962/1749 and
 // 2031/1866; eight bodies of 812 markers in 8 cells 78.1/90.3, in 16 161/125: up to
@@ -235,7 +237,7 @@ int membrane_clusters_max(const ibm_lbm_t* h, int nv) {
 int rigid_clusters_max(const ibm_lbm_t* h, int least, int most, bool direct) {
   if (h->served_slots > 0) return SERVED_MAX / h->served_slots;
   const int two = h->clusters_two;
-  if (direct || least < 256 || most > 3072) return two;
+  if (direct || least < 256 || most > 3072 || h->n_membranes > 0) return two;
   return least < 512 ? two + two / 2 : 2 * two;
 }
 // Steps of the solid-only dynamics in one launch of clusters, and up to how

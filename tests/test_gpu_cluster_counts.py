@@ -84,3 +84,16 @@ def test_many_rigid_bodies_take_the_separate_kernels(cuda_lib, n, freq, direct, 
 @pytest.mark.parametrize('freq,bodies', [(2, 15), (2, 30), (2, 31), (6, 45)])
 def test_solid_counts_match_oracle(cuda_lib, freq, bodies):
     test_gpu_solid.test_solid_steps_of_several_bodies_match_oracle(cuda_lib, freq, bodies, (1, 7))
+
+
+@pytest.mark.parametrize('rigids,clusters', [(20, True), (40, False)])
+def test_rigid_bodies_beside_membranes(cuda_lib, rigids, clusters):
+    r, m = _rigid(rigids, 6, False), _membranes(5, 4)
+    n = r['X'].shape[1]
+    X = np.concatenate([r['X'], m['X'] + 2.0], axis=1)
+    w = dict(m, bodies=r['bodies'] + [dict(b, first=b['first'] + n) for b in m['bodies']], X=X)
+    sim = cuda_lib.Simulation.from_workload(w)
+    held = sim.device_bytes
+    sim.step(4)
+    assert (sim.device_bytes - held >= 16 * sim.N) == clusters
+    _match_stages(cuda_lib, w)
