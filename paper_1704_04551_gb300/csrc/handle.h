@@ -66,10 +66,11 @@ struct ibm_lbm {
   ibm::MorseDev morse{};
   bool morse_ready = false;       // cell-list buffers match the markers
   std::vector<Alloc> morse_mem;
+  int n_sm = 0;
   int clusters_one = 0, clusters_two = 0;  // clusters the device holds at once, by blocks on an SM
   MarkerGroup* groups = nullptr;  // transfer blocks
   int n_groups = 0;
-  int n_body_groups = 0;          // groups [n_body_groups, n_groups) are runs of tracers
+  int n_body_groups = 0;          // groups [n_body_groups, n_groups): tracers, in kernels of their own
   bool tracers_everywhere = false;  // they reach most tiles: the collision writes every velocity instead
   int4* boxes = nullptr;          // per group: stencil box origin and size
   // Fused coupling (suspensions of membranes only): one block per body

@@ -108,3 +108,24 @@ BODIES = dict(rigid=_tethered, cluster_membranes=lambda: _membranes(3), fused_me
 def test_spread_then_step_with_bodies(cuda_lib, kind, before, after):
     """Both parities: a coupled step's buffer goes with the parity, the stage's does not."""
     _run(cuda_lib, BODIES[kind](), before, after)
+
+
+@pytest.mark.parametrize('M', [7, 45000])
+def test_spread_then_step_with_tracers_beside_a_body(cuda_lib, M):
+    """Tracers in the bodies' kernels (few) and in kernels of their own (more
+    blocks than the device's SMs take beside the body's)."""
+    w = _tethered()
+    T = markers_inside(w['lattice'], M, 3)
+    w = dict(w, X=np.concatenate([w['X'], T], axis=1))
+    # (the same force on a cell for any number of tracers)
+    F = 2e-3 / max(1.0, M / 1000.0) * np.random.default_rng(4).standard_normal(w['X'].shape)
+    sim, ora = cuda_lib.Simulation.from_workload(w), O.Oracle.from_workload(w)
+    for before, n in ((1, 3), (2, 18)):
+        sim.step(before)
+        ora.step(before)
+        sim.set_marker_forces(F)
+        sim.stage(cuda_lib.STAGE_SPREAD)
+        sim.step(n)
+        _oracle_step(ora, F)
+        ora.step(n - 1)
+        _check(sim, ora, w['lattice'])
