@@ -1,6 +1,7 @@
 // Coupling of few bodies in one lattice: one cluster of thread blocks per
 // body (cluster_body.cuh).
 #include <algorithm>
+#include <atomic>
 
 #include "cluster_body.cuh"
 #include "common.cuh"
@@ -215,7 +216,15 @@ void launch_solid_cluster(const MarkersDev& m, BodyDev* bodies, const int* list,
 // all of a size (152 SMs: 15 clusters of one block an SM, 36 of two, not 19
 // and 38; with one block an SM 16 to 19 bodies took two waves, 72 us a step
 // instead of 45 with two for membranes of 642 vertices at 72^3).
+// (Asked once per device: ~8 us, and every handle needs both.)
 cudaError_t cluster_capacity(int per_sm, int* out) {
+  constexpr int DEVICES = 64;
+  static std::atomic<int> known[2][DEVICES];  // 0: not asked yet
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::atomic<int>* slot = dev < DEVICES ? &known[per_sm == 1 ? 0 : 1][dev] : nullptr;
+  if (slot && (*out = slot->load()) > 0) return cudaSuccess;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(CLUSTER);
   cfg.blockDim = dim3(CLUSTER_THREADS);
@@ -226,7 +235,9 @@ cudaError_t cluster_capacity(int per_sm, int* out) {
   attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(out, k_couple_cluster<GEOM_TUBE, 1>, &cfg);
+  e = cudaOccupancyMaxActiveClusters(out, k_couple_cluster<GEOM_TUBE, 1>, &cfg);
+  if (e == cudaSuccess && slot) slot->store(*out);
+  return e;
 }
 
 // Cells of a block's box: what `per_sm` blocks on an SM leave, at most
