@@ -146,6 +146,11 @@ int spread_noalloc(const double* X, const double* F, int64_t n_markers, int32_t 
     return IBM_LBM_E_CUDA;
   }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
+  if (n_markers == 0) {  // (100^3: 16.5 us with the accumulator cleared and read)
+    if (cudaMemsetAsync(g, 0, 3 * sizeof(double) * (size_t)N, st) == cudaSuccess) return IBM_LBM_OK;
+    cudaGetLastError();
+    return IBM_LBM_E_CUDA;
+  }
   Grid G{nx, ny, nz, (int)N, geometry, 0.5f * (float)(ny - 1), 0.5f * (float)(nz - 1),
          (float)(tube_radius * tube_radius)};
   int M = (int)n_markers, dev = 0, sms = 0;

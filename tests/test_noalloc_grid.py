@@ -27,6 +27,7 @@ int __cudaPopCallConfiguration(void) { return 1; }
 int cudaGetDevice(int* d) { *d = 0; return 0; }
 int cudaDeviceGetAttribute(int* v, int attr, int dev) { (void)attr; (void)dev; *v = 152; return 0; }
 int cudaGetSymbolAddress(void** p, const void* s) { (void)s; *p = scratch; return 0; }
+int cudaMemsetAsync(void* p, int v, size_t n, void* st) { (void)p; (void)v; (void)n; (void)st; return 0; }
 int cudaGetLastError(void) { int e = last_error; last_error = 0; return e; }
 int cudaLaunchCooperativeKernel(const void* f, dim3_t grid, dim3_t block, void** args, size_t smem, void* st) {
   (void)f; (void)block; (void)args; (void)smem; (void)st;

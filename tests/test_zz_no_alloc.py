@@ -121,3 +121,17 @@ def test_spread_noalloc_rejects_oversized_lattice(cuda_lib):
     assert rc == binding.E_ARG
     rc = binding.ibm_lbm_spread_noalloc(X.data_ptr(), X.data_ptr(), 1, 2, 8, 8, 0, 0.0, g.data_ptr())
     assert rc == binding.E_ARG
+
+
+def test_spread_noalloc_without_markers(cuda_lib):
+    """No markers: the whole density is written, as zeros."""
+    import torch
+    dev = torch.device('cuda', 0)
+    for n in (4, 33, 100):
+        g = torch.full((3, n ** 3 + 1), float('nan'), dtype=torch.float64, device=dev)
+        out = g.view(-1)[:3 * n ** 3]
+        rc = cuda_lib.ibm_lbm_spread_noalloc(0, 0, 0, n, n, n, 0, 0.0, out.data_ptr(),
+                                             torch.cuda.current_stream(dev).cuda_stream)
+        torch.cuda.synchronize(dev)
+        assert rc == cuda_lib.OK
+        assert (out == 0).all() and torch.isnan(g.view(-1)[3 * n ** 3:]).all()
