@@ -2,7 +2,7 @@
 // the interpolation and advection of step n, the body's forces, and the
 // spreading of step n+1 (Secs. 2.2 and 2.3 of arXiv:1704.04551), for rigid
 // bodies (penalty tether or direct forcing) and membranes. Shared by the
-// single-lattice kernels (couple.cu) and the batched serving kernels
+// single-lattice kernels (cluster.cu) and the batched serving kernels
 // (serve.cu).
 //
 // A case with few bodies is bound by the latency of one body's chain of
@@ -301,7 +301,7 @@ __device__ __forceinline__ float cluster_membrane(ClusterShare& S, const Membran
   __syncthreads();
   if (tid < 2 * CLUSTER) {
     const int r = tid >> 1, q = tid & 1;
-    cl.map_shared_rank(&S.sum[0][0], r)[6 * rank + q] = S.part_sum.units(q, q == 0 ? K.qa : K.qv);
+    cl.map_shared_rank(&S.sum[0][0], r)[6 * rank + q] = S.part_sum.units(q, q == 0 ? K.sa : K.sv);
   }
   // the area and volume terms need the other blocks' sums; the edges do not
   cl.barrier_arrive();

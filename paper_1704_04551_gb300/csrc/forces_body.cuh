@@ -102,10 +102,11 @@ __device__ __forceinline__ MembraneScale membrane_scale(const MeshDev& mesh) {
 struct BodySums {
   long long fix[2];
   double far[2];
-  // in units of lo; q: size of one
-  __device__ __forceinline__ double units(int i, double q) const {
-    const double n = (double)fix[i];
-    return __double_as_longlong(far[i]) == 0 ? n : n + far[i] / q;
+  // in units of lo; s: units of hi per area or volume (a power of two)
+  __device__ __forceinline__ double units(int i, float s) const {
+    double n = (double)fix[i];
+    if (__double_as_longlong(far[i]) != 0) n += far[i] * (double)s * 4194304.0;
+    return n;
   }
 };
 __device__ __forceinline__ long long warp_fixed(float v, float s) {
@@ -128,7 +129,7 @@ __device__ __forceinline__ void warp_far_sum(float area, float volume, BodySums*
 // Adds the warp's values to the block's area and volume.
 __device__ __forceinline__ void warp_fixed_sum(float area, float volume, const MembraneScale& K, BodySums* sums) {
   constexpr float most = 67108864.0f;  // 32 lanes below it add up to less than 2^31
-  if (__any_sync(0xffffffffu, !(fabsf(area * K.sa) < most && fabsf(volume * K.sv) < most))) {
+  if (__any_sync(0xffffffffu, !(fabsf(area * K.sa) + fabsf(volume * K.sv) < most))) {
     warp_far_sum(area, volume, sums);
     return;
   }
@@ -253,9 +254,9 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
 
 // The scatter of a block's force contributions where the last step's largest
 // one gives no scale (none yet, or contributions above its headroom): their
-// maximum is taken first, then they are added in fixed point with the scale it allows, qcap. The sums depend on no
-// order, unlike float atomics, which reruns of a body's first step differed
-// by. Contributions that are not finite are added as floats, to reach the
+// maximum is taken first, then they are added in fixed point with the scale
+// that maximum allows. The sums depend on no order, unlike those of float
+// atomics, by which reruns of a body's first step differed. Contributions that are not finite are added as floats, to reach the
 // forces, and so are those of a body whose largest one is below REDO_TINY: the
 // scale qcap / q and its inverse stay normal numbers down to there (qcap < 2^31).
 // pass(add) hands out the contributions; vertices [v0, v0 + n) are
@@ -374,8 +375,8 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
   warp_fixed_sum(a_part, v_part, K, &s_sum);
   __syncthreads();  // normals, areas and sums are visible
   // A - A0 and V - V0 in FP64 (small differences of large sums)
-  if (threadIdx.x == 0) s_dev[0] = (float)(s_sum.units(0, K.qa) * K.qa - (double)mesh.A0) / mesh.A0;
-  if (threadIdx.x == 32) s_dev[1] = (float)(s_sum.units(1, K.qv) * K.qv - (double)mesh.V0) / mesh.V0;
+  if (threadIdx.x == 0) s_dev[0] = (float)(s_sum.units(0, K.sa) * K.qa - (double)mesh.A0) / mesh.A0;
+  if (threadIdx.x == 32) s_dev[1] = (float)(s_sum.units(1, K.sv) * K.qv - (double)mesh.V0) / mesh.V0;
   __syncthreads();
   const float cg = k_g * s_dev[0];
   const float cv = k_v * s_dev[1];
