@@ -97,3 +97,32 @@ def test_rigid_bodies_beside_membranes(cuda_lib, rigids, clusters):
     sim.step(4)
     assert (sim.device_bytes - held >= 16 * sim.N) == clusters
     _match_stages(cuda_lib, w)
+
+
+@pytest.mark.parametrize('kind', ['rigid', 'cluster_membranes', 'fused_membranes'])
+def test_no_memory_for_the_second_density(cuda_lib, kind):
+    """An allocator that has nothing left when the first coupled step asks for
+    the second force density: the same steps, one at a time."""
+    import torch
+
+    class Full(cuda_lib.TorchMemory):
+        full = False
+
+        def _on_alloc(self, nbytes, ctx):
+            return None if self.full else super()._on_alloc(nbytes, ctx)
+
+    w = _rigid(3, 4, False) if kind == 'rigid' else _membranes(3 if kind == 'cluster_membranes' else 40, 8)
+    mem = Full(torch.device('cuda', 0))
+    a, b = cuda_lib.Simulation.from_workload(w, memory=mem), cuda_lib.Simulation.from_workload(w)
+    held = a.device_bytes
+    mem.full = True
+    for n in (2, 19):
+        a.step(n)
+        b.step(n)
+    assert a.device_bytes == held
+    mem.full = False
+    (Xa, _, Fa), (Xb, _, Fb) = a.markers(), b.markers()
+    assert np.abs(Xa - Xb).max() < 1e-7
+    assert np.abs(Fa - Fb).max() < 1e-4 * np.abs(Fb).max()
+    assert rel_l2(a.fields()[1], b.fields()[1]) < 1e-6
+    assert np.abs(a.force_density()).max() == 0.0
