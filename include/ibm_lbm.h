@@ -37,7 +37,11 @@
  *     a time.
  *   - Device memory is owned by the handle and allocated at create /
  *     set_markers time through the caller's allocator (or cudaMalloc when
- *     none is given). Stepping allocates nothing.
+ *     none is given). Stepping allocates nothing but one array: a handle of
+ *     membranes alone (but for few large ones), or of few rigid bodies with
+ *     or without membranes, takes a second force density, 16 bytes a cell, in
+ *     its first ibm_lbm_step of two steps or more; without memory for it it
+ *     steps by kernels that need none.
  */
 #ifndef IBM_LBM_H
 #define IBM_LBM_H
@@ -248,7 +252,7 @@ int ibm_lbm_get_force_density(ibm_lbm_t* h, double* g);
 int ibm_lbm_set_timing(ibm_lbm_t* h, int64_t max_steps);
 int ibm_lbm_get_timing(ibm_lbm_t* h, double out[6]);
 /* Timing of the production path of suspensions. With on != 0 and timing on,
- * a handle that takes a fused coupling (membranes, or rigid bodies, and no
+ * a handle that takes a fused coupling (membranes or few rigid bodies, and no
  * other markers) runs its timed steps on that path, with direct launches:
  * each step that launches the coupling is timed, out[2] receiving its
  * collision and out[3] the coupling (interpolation and advection of the
@@ -270,8 +274,9 @@ int ibm_lbm_set_timing_fused(ibm_lbm_t* h, int on);
  * together (batched launches, a chunk replayed as a CUDA graph), retires
  * the cases that reached their step count (their results are copied to host
  * memory and their device memory is released) and admits waiting ones. A
- * case's result is the same as running it alone with ibm_lbm_step. Cases use
- * FP32 storage.
+ * case's result is the same as running it alone with ibm_lbm_step (to rounding;
+ * how its bodies are coupled depends on the case and on max_active, never on
+ * what else is served). Cases use FP32 storage.
  * --------------------------------------------------------------------------- */
 typedef struct ibm_lbm_server ibm_lbm_server_t;
 

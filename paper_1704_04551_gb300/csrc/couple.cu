@@ -22,7 +22,7 @@
 // and forces, which part 3 still reads. Part 3 also stores its vertex
 // order in global memory beside the box, for part 1 of the next step,
 // which gathers at the same positions. A box that does not fit whole is
-// taken in slabs of z layers by parts 1 and 3 (no order is stored then).
+// taken in slabs of z layers by parts 1 and 3, in the same order.
 #include <type_traits>
 
 #include "common.cuh"

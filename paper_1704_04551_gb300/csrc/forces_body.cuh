@@ -256,12 +256,12 @@ __device__ __forceinline__ ForceSums membrane_core(BodyDev* Bp, const MeshDev& m
 // one gives no scale (none yet, or contributions above its headroom): their
 // maximum is taken first, then they are added in fixed point with the scale
 // that maximum allows. The sums depend on no order, unlike those of float
-// atomics, by which reruns of a body's first step differed. Contributions that are not finite are added as floats, to reach the
-// forces, and so are those of a body whose largest one is below REDO_TINY: the
-// scale qcap / q and its inverse stay normal numbers down to there (qcap < 2^31).
-// pass(add) hands out the contributions; vertices [v0, v0 + n) are
-// summed in sQ [3][stride] (zero entries [n, stride) included in the clear).
-// Returns the unit of the sums.
+// atomics, by which reruns of a body's first step differed. Contributions that
+// are not finite are added as floats, to reach the forces, and so are those of
+// a body whose largest one is below REDO_TINY: the scale qcap / q and its
+// inverse stay normal numbers down to there (qcap < 2^31). pass(add) hands out
+// the contributions; vertices [v0, v0 + n) are summed in sQ [3][stride] (zero
+// entries [n, stride) included in the clear). Returns the unit of the sums.
 constexpr float REDO_TINY = 1e-25f;
 template <class Pass>
 __device__ __forceinline__ float redo_scatter(Pass&& pass, int* sQ, int stride, int n, int v0, int n_clear, float qcap,

@@ -75,7 +75,10 @@ __global__ void __launch_bounds__(COLLIDE_THREADS, (collide_min_blocks<S, ODD>()
 // 256^3 tube, FP16: even step 186 -> 158 us, odd 208 -> 187 us; 7 resident
 // blocks (72 registers) measured best (even: 6: 166, 8: 160 us). From
 // PAIR_CELLS_MIN fluid cells on: below, the single-cell kernel is one wave, and
-// half the threads only wait longer (60x47x33, odd: 9.0 against 10.6 us).
+// half the threads only wait longer (60x47x33, odd: 9.0 against 10.6 us). Mean
+// of both steps, pairs / single, cubes of 32, 48, 60, 64, 80, 96, 128: periodic
+// 6.3/6.3, 6.9/7.2, 8.3/8.5, 8.3/9.3, 11.4/13.4, 15.5/18.6, 30.0/38.0; y walls
+// 7.3/6.3, 7.7/7.5, 9.4/9.4, 8.8/10.0, 12.5/13.9, 16.7/19.6, 30.6/39.1 us.
 constexpr unsigned PAIR_CELLS_MIN = 1u << 18;
 constexpr int PAIR_MIN_BLOCKS = 7;
 template <int S, int ODD, int GEOM, bool DENSE, bool IDX32>
